@@ -17,6 +17,7 @@ struct pv_scene {
   uint32_t n_tris = 0, n_objects = 0, n_static = 0, n_dyn_tris = 0, n_dyn = 0;
   uint32_t B = 0;
   float diag = 0.f, tmin = 0.f, close_tol = 0.f;
+  float box_lo[3] = {0.f, 0.f, 0.f}, box_hi[3] = {0.f, 0.f, 0.f};   // box of the triangles as given (sizes the splat's grid)
   uint32_t flags = 0;
 
   // shared BVH arrays: triangles [static references | dynamic]; binary nodes

@@ -187,6 +187,7 @@ extern "C" int pv_build_scene(const pv_scene_desc* d, void* stream, pv_scene** o
   std::vector<uint32_t> static_prims;
   std::vector<uint8_t> pslot(d->n_tris, 255);
   std::vector<float4> palb(d->n_tris), pnrm(d->n_tris);
+  float lo[3] = {d->verts[0], d->verts[1], d->verts[2]}, hi[3] = {d->verts[0], d->verts[1], d->verts[2]};
   for (uint32_t t = 0; t < d->n_tris; ++t) {
     const uint32_t o = d->tri_object[t];
     const float* a = d->object_albedo + 3 * (size_t)o;
@@ -194,6 +195,10 @@ extern "C" int pv_build_scene(const pv_scene_desc* d, void* stream, pv_scene** o
     const float* v = d->verts + 9 * (size_t)t;
     const double e1[3] = {(double)v[3] - v[0], (double)v[4] - v[1], (double)v[5] - v[2]};
     const double e2[3] = {(double)v[6] - v[0], (double)v[7] - v[1], (double)v[8] - v[2]};
+    for (int k = 0; k < 9; ++k) {
+      lo[k % 3] = std::fmin(lo[k % 3], v[k]);
+      hi[k % 3] = std::fmax(hi[k % 3], v[k]);
+    }
     pnrm[t] = make_float4((float)(e1[1] * e2[2] - e1[2] * e2[1]), (float)(e1[2] * e2[0] - e1[0] * e2[2]),
                           (float)(e1[0] * e2[1] - e1[1] * e2[0]), 0.f);
     if (slot_of[o] >= 0) {
@@ -204,6 +209,8 @@ extern "C" int pv_build_scene(const pv_scene_desc* d, void* stream, pv_scene** o
       static_prims.push_back(t);
     }
   }
+  std::memcpy(s->box_lo, lo, sizeof lo);
+  std::memcpy(s->box_hi, hi, sizeof hi);
   for (uint32_t sl = 0; sl < s->n_dyn; ++sl) s->h_objs[sl].user_object = s->dyn_object[sl];
   // initial poses
   s->h_xf_new.assign(12 * (size_t)s->n_dyn, 0.f);

@@ -2,10 +2,10 @@
 // The paper only cites its splatting method, so this is a plain radius
 // kernel, evaluated as a gather.  k_gbuffer casts one primary ray per pixel
 // through the scene's BVH (visible point, normal facing the camera,
-// primitive).  k_grid_fill hashes every stored photon into a grid of cells
-// of edge r (count, scan of the buckets, place), skipping photons whose
+// primitive).  Photons and visible points are both sorted by the cells of a
+// grid over space (count with ranks, scan, place), skipping photons whose
 // kernel cube reaches the near plane.  k_gather then gives each pixel the
-// photons of the 27 cells around its visible point p: every photon x with
+// photons of the cells around its visible point p: every photon x with
 // energy E arriving on the visible side and s = |p - x| / r < 1 adds
 // rho/pi E 2 (1 - s^2) / (pi r^2).  Each pixel is written once, without
 // atomics, and the work per pixel is bounded by the photons near it, not by
@@ -31,10 +31,53 @@ struct GPixel {              // 32 bytes per pixel
   float4 n;                  // normal facing the camera
 };
 
-__global__ void __launch_bounds__(256) k_gbuffer(SceneView sv, Cam c, GPixel* g) {
-  const uint32_t px = blockIdx.x * blockDim.x + threadIdx.x;
-  if (px >= c.W * c.H) return;
-  const uint32_t i = px % c.W, j = px / c.W;
+// Grid over space for photons and visible points: cells of edge ``edge`` =
+// radius / kCellsPerRadius, wrapped around after nx, ny, nz cells per axis and
+// numbered with x fastest.  A photon within ``radius`` of a point lies at most
+// kReach cells from the point's cell along every axis; each axis has at least
+// 2 kReach + 2 cells, so the cells around a point are distinct and hold every
+// photon once.  Wrapping lets points far apart share a cell: such photons fail
+// the distance test.  Cells next to each other in x are next to each other in
+// the sorted photons, so the cells around points in a box are a few ranges.
+constexpr int kCellsPerRadius = 1;
+constexpr int kReach = kCellsPerRadius;
+
+struct Grid {
+  float inv_edge;
+  int nx, ny, nz;
+  uint32_t cells;              // nx ny nz
+};
+
+__device__ __forceinline__ int3 grid_cell(const Grid& g, float3 x) {
+  const float lim = 1.0e9f;
+  return make_int3((int)fminf(fmaxf(floorf(x.x * g.inv_edge), -lim), lim),
+                   (int)fminf(fmaxf(floorf(x.y * g.inv_edge), -lim), lim),
+                   (int)fminf(fmaxf(floorf(x.z * g.inv_edge), -lim), lim));
+}
+
+__device__ __forceinline__ int wrap(int c, int n) {
+  const int m = c % n;
+  return m < 0 ? m + n : m;
+}
+
+__device__ __forceinline__ uint32_t grid_row(const Grid& g, int cy, int cz) {
+  return ((uint32_t)wrap(cz, g.nz) * g.ny + (uint32_t)wrap(cy, g.ny)) * g.nx;
+}
+
+__device__ __forceinline__ uint32_t grid_index(const Grid& g, int3 c) {
+  return grid_row(g, c.y, c.z) + (uint32_t)wrap(c.x, g.nx);
+}
+
+// One primary ray per pixel, a warp per 8 x 4 pixels (its rays then visit much
+// the same nodes: city at 1920 x 1080 0.277 ms in rows of 32 pixels, 0.232 ms in
+// tiles, 0.222 ms with five blocks per SM asked of the register allocator; six
+// take 0.237 ms).
+__global__ void __launch_bounds__(256, 5) k_gbuffer(SceneView sv, Cam c, GPixel* g) {
+  const uint32_t tiles_x = (c.W + 15u) / 16u;
+  const uint32_t w = threadIdx.x >> 5, l = threadIdx.x & 31u;
+  const uint32_t i = (blockIdx.x % tiles_x) * 16u + (w & 1u) * 8u + (l & 7u);
+  const uint32_t j = (blockIdx.x / tiles_x) * 16u + (w >> 1) * 4u + (l >> 3);
+  if (i >= c.W || j >= c.H) return;
   const float x = (2.0f * ((float)i + 0.5f) / (float)c.W - 1.0f) * c.tx;
   const float y = (1.0f - 2.0f * ((float)j + 0.5f) / (float)c.H) * c.ty;
   const float3 d = normalize(c.f + x * c.r + y * c.u);
@@ -53,7 +96,7 @@ __global__ void __launch_bounds__(256) k_gbuffer(SceneView sv, Cam c, GPixel* g)
     o.p = make_float4(p.x, p.y, p.z, T.v0.w);
     o.n = make_float4(nn.x, nn.y, nn.z, 0.f);
   }
-  g[px] = o;
+  g[(size_t)j * c.W + i] = o;
 }
 
 // A photon takes part when every corner of its kernel cube lies beyond the
@@ -68,51 +111,79 @@ __device__ __forceinline__ bool in_front(const Cam& c, float3 x, float radius) {
   return true;
 }
 
-// Photon grid: cells of edge ``radius``, hashed into a power-of-two number of
-// buckets; a photon within ``radius`` of a point lies in one of the 27 cells
-// around the point's cell.
-struct Grid {
-  float inv_r;                 // 1 / radius
-  uint32_t mask;               // buckets - 1
+// The photons that take part, sorted by cell: position, the segment they
+// arrive along (position minus the path's previous vertex) and energy.
+struct Photons {
+  float4* xd;                  // pairs: position, w = energy.x; arriving segment, w = energy.y
+  float* e;                    // energy.z
 };
 
-__device__ __forceinline__ int3 grid_cell(const Grid& g, float3 x) {
-  const float lim = 1.0e9f;
-  return make_int3((int)fminf(fmaxf(floorf(x.x * g.inv_r), -lim), lim), (int)fminf(fmaxf(floorf(x.y * g.inv_r), -lim), lim),
-                   (int)fminf(fmaxf(floorf(x.z * g.inv_r), -lim), lim));
+constexpr uint32_t kSkipped = 0xFFFFFFFFu;
+
+// Count the photons per cell; rank[k n + p] = the photon's rank within its
+// cell, so that placing needs no second round of atomics.  A thread per path,
+// which has the loads (and then the atomics) of kRowsAtOnce rows in flight.
+// (Measured on the city, 2.0M photons: count 54 us and place 73 us at 2 rows, 57 and 85 us at 4, 49 and 110 us
+// one at a time; a thread per photon, exiting where a path is shorter, 57 and 107 us.)
+constexpr uint32_t kRowsAtOnce = 2;
+
+__global__ void __launch_bounds__(256) k_photon_count(Cam c, Grid g, float radius, uint32_t n, uint32_t B,
+                                                      const uint32_t* info, const float4* pa, uint32_t* counts,
+                                                      uint32_t* rank) {
+  const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= n) return;
+  const uint32_t L = min(info_nseg(info[p]), B);
+  for (uint32_t k0 = 0; k0 < L; k0 += kRowsAtOnce) {
+    float4 x[kRowsAtOnce];
+    uint32_t r[kRowsAtOnce];
+#pragma unroll
+    for (uint32_t q = 0; q < kRowsAtOnce; ++q)
+      if (k0 + q < L) x[q] = pa[(size_t)(k0 + q) * n + p];
+#pragma unroll
+    for (uint32_t q = 0; q < kRowsAtOnce; ++q) {
+      r[q] = kSkipped;
+      if (k0 + q < L && in_front(c, f3(x[q]), radius)) r[q] = atomicAdd(counts + grid_index(g, grid_cell(g, f3(x[q]))), 1u);
+    }
+#pragma unroll
+    for (uint32_t q = 0; q < kRowsAtOnce; ++q)
+      if (k0 + q < L) rank[(size_t)(k0 + q) * n + p] = r[q];
+  }
 }
 
-__device__ __forceinline__ uint32_t grid_bucket(const Grid& g, int3 c) {
-  return (((uint32_t)c.x * 73856093u) ^ ((uint32_t)c.y * 19349663u) ^ ((uint32_t)c.z * 83492791u)) & g.mask;
-}
-
-struct PhotonRec {           // 32 bytes
-  float4 x;                  // position, w = path index * 16 + row (int bits)
-  float4 e;                  // incident energy
-};
-
-// pass 0: count the photons per bucket; pass 1: place them (heads: exclusive
-// prefix of the counts on entry, each bucket's end on exit).
-template <int kPass>
-__global__ void __launch_bounds__(256) k_grid_fill(Cam c, Grid g, float radius, uint32_t n, uint32_t B,
-                                                   const uint32_t* info, const float4* pa, const float4* pb,
-                                                   uint32_t* heads, PhotonRec* rec) {
-  for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
-    const uint32_t L = min(info_nseg(info[p]), B);
-    for (uint32_t k = 0; k < L; ++k) {
-      const float4 xv = pa[(size_t)k * n + p];
-      const float3 x = f3(xv);
-      if (!in_front(c, x, radius)) continue;
-      const uint32_t b = grid_bucket(g, grid_cell(g, x));
-      if (kPass == 0) {
-        atomicAdd(heads + b, 1u);
-      } else {
-        const uint32_t slot = atomicAdd(heads + b, 1u);
-        PhotonRec r;
-        r.x = make_float4(x.x, x.y, x.z, __int_as_float((int)(p * 16u + k)));
-        r.e = pb[(size_t)k * n + p];
-        rec[slot] = r;
+// Place the photons (starts: exclusive prefix of the counts).
+__global__ void __launch_bounds__(256) k_photon_place(Grid g, uint32_t n, uint32_t B, const uint32_t* info,
+                                                      const float* origin, const float4* pa, const float4* pb,
+                                                      const uint32_t* starts, const uint32_t* rank, Photons out) {
+  const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= n) return;
+  const uint32_t L = min(info_nseg(info[p]), B);
+  if (L == 0) return;
+  float3 prev = make_float3(origin[p], origin[n + p], origin[2 * (size_t)n + p]);
+  for (uint32_t k0 = 0; k0 < L; k0 += kRowsAtOnce) {
+    float4 x[kRowsAtOnce], e[kRowsAtOnce];
+    uint32_t r[kRowsAtOnce];
+#pragma unroll
+    for (uint32_t q = 0; q < kRowsAtOnce; ++q) {
+      r[q] = kSkipped;
+      if (k0 + q < L) {
+        x[q] = pa[(size_t)(k0 + q) * n + p];
+        e[q] = pb[(size_t)(k0 + q) * n + p];
+        r[q] = rank[(size_t)(k0 + q) * n + p];
       }
+    }
+#pragma unroll
+    for (uint32_t q = 0; q < kRowsAtOnce; ++q)
+      if (r[q] != kSkipped) r[q] += starts[grid_index(g, grid_cell(g, f3(x[q])))];
+#pragma unroll
+    for (uint32_t q = 0; q < kRowsAtOnce; ++q) {
+      if (k0 + q >= L) break;
+      if (r[q] != kSkipped) {
+        const float3 d = f3(x[q]) - prev;
+        out.xd[2 * (size_t)r[q]] = make_float4(x[q].x, x[q].y, x[q].z, e[q].x);
+        out.xd[2 * (size_t)r[q] + 1] = make_float4(d.x, d.y, d.z, e[q].y);
+        out.e[r[q]] = e[q].z;
+      }
+      prev = f3(x[q]);
     }
   }
 }
@@ -159,53 +230,175 @@ __global__ void __launch_bounds__(1024) k_tile_scan(uint32_t* v, const uint32_t*
   *p = make_uint4(base, base + x.x, base + x.x + x.y, base + x.x + x.y + x.z);
 }
 
-// One pixel per thread: the photons of the 27 cells around its visible point.
-__global__ void __launch_bounds__(256) k_gather(SceneView sv, Cam c, Grid g, float radius, uint32_t n,
-                                                const float* origin, const float4* pa, const GPixel* gb,
-                                                const uint32_t* heads, const PhotonRec* rec, float* image) {
-  const uint32_t px = blockIdx.x * blockDim.x + threadIdx.x;
-  if (px >= c.W * c.H) return;
-  const GPixel gp = gb[px];
-  const int prim = __float_as_int(gp.p.w);
-  float3 acc = make_float3(0.f, 0.f, 0.f);
-  if (prim >= 0) {
-    const float3 P = f3(gp.p), nrm = f3(gp.n);
-    const float r2 = radius * radius;
-    const int3 cp = grid_cell(g, P);
-    for (int dz = -1; dz <= 1; ++dz)
-      for (int dy = -1; dy <= 1; ++dy)
-        for (int dx = -1; dx <= 1; ++dx) {
-          const int3 cc = make_int3(cp.x + dx, cp.y + dy, cp.z + dz);
-          const uint32_t b = grid_bucket(g, cc);
-          const uint32_t beg = b ? heads[b - 1] : 0u, end = heads[b];
-          for (uint32_t i = beg; i < end; ++i) {
-            const float4 xv = __ldg(&rec[i].x);
-            const float3 x = f3(xv);
-            const float3 d = P - x;
-            const float s2 = dot(d, d) / r2;
-            if (!(s2 < 1.0f)) continue;
-            const int3 xc = grid_cell(g, x);         // each photon once: only from its own cell
-            if (xc.x != cc.x || xc.y != cc.y || xc.z != cc.z) continue;
-            const uint32_t id = (uint32_t)__float_as_int(xv.w), p = id >> 4, k = id & 15u;
-            const float3 prev = k == 0 ? make_float3(origin[p], origin[n + p], origin[2 * (size_t)n + p])
-                                       : f3(__ldg(pa + (size_t)(k - 1) * n + p));
-            if (!(dot(nrm, x - prev) < 0.0f)) continue;   // arrives on the visible side
-            const float4 e = __ldg(&rec[i].e);
-            const float w = 1.0f - s2;
-            acc = make_float3(fmaf(e.x, w, acc.x), fmaf(e.y, w, acc.y), fmaf(e.z, w, acc.z));
-          }
+// Order-preserving map of floats to integers, for warp-wide minima and maxima.
+__device__ __forceinline__ int ordered(float f) {
+  const int i = __float_as_int(f);
+  return i >= 0 ? i : i ^ 0x7FFFFFFF;
+}
+__device__ __forceinline__ float unordered(int i) { return __int_as_float(i >= 0 ? i : i ^ 0x7FFFFFFF); }
+__device__ __forceinline__ float warp_min(float f) { return unordered(__reduce_min_sync(0xffffffffu, ordered(f))); }
+__device__ __forceinline__ float warp_max(float f) { return unordered(__reduce_max_sync(0xffffffffu, ordered(f))); }
+
+// Every visible pixel gathers the photons around its visible point.  A block
+// takes 8 x 4 pixels, one per lane of each of its four warps, which mostly see
+// points close to each other.  A warp looks up the rows of cells around the box
+// of these points (a lane per row), deals their photons out to its lanes 32 at
+// a time (coalesced loads), keeps those within the radius of the box in shared
+// memory, and walks the kept ones with all lanes together: every photon is a
+// broadcast read and a test against each lane's pixel.  Where the points spread
+// over more than kSpread cells beyond the first one (an edge in depth), the
+// warp takes them group by group.  Each warp takes every fourth 32 photons.
+//
+// Bound by issue: on the 1M-path city at 1920 x 1080 and r = 0.3 m (2.0M
+// photons, up to a few thousand in the cells around a point) 3.9e8 warp
+// instructions at 26 of 32 lanes, 67 % of the issue slots.  There it takes
+// 0.47 ms, where a thread per pixel walking 27 hashed cells, which read each
+// photon's previous vertex from the path buffers, took 3.57 ms (1.14 ms with
+// cells sorted by row and the segment in the record: long waits on loads
+// at 12 of 32 lanes).  One warp for 8 x 4 pixels takes 0.99 ms and two 0.62:
+// neighbouring tiles in one block thrash L1 and the densest tiles finish late;
+// two pixels per lane take 0.58 ms and cells of half the radius 0.63 ms.
+constexpr int kParts = 4;          // warps of a block
+constexpr int kSpread = 2;         // measured on the city: 1 0.51 ms, 2 0.47, 3 0.51, 4 0.60
+
+__global__ void __launch_bounds__(32 * kParts) k_gather(SceneView sv, Cam c, Grid g, float radius, const GPixel* gb,
+                                                        const uint32_t* starts, Photons ph, float* image) {
+  constexpr int kBuf = 64;         // photons kept before they are tested: fewer than 32 left over plus 32 new
+  __shared__ float4 s_x[kParts][kBuf], s_d[kParts][kBuf];
+  __shared__ float s_e[kParts][kBuf];
+  __shared__ float s_acc[kParts][3][32];
+  const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
+  const uint32_t tiles_x = (c.W + 7u) / 8u;
+  const uint32_t pi = (blockIdx.x % tiles_x) * 8u + (lane & 7), pj = (blockIdx.x / tiles_x) * 4u + (lane >> 3);
+  const bool inside = pi < c.W && pj < c.H;
+  const float inv_r2 = 1.0f / (radius * radius);
+  const float away = 3.0e18f;      // beyond every photon's radius
+  float3 P = make_float3(0.f, 0.f, 0.f), nrm = P, acc = P, Q = P, N = P;   // Q, N: P and nrm within the group
+  int prim = -1;
+  if (inside) {
+    const GPixel* q = gb + ((size_t)pj * c.W + pi);
+    const float4 p = q->p;
+    prim = __float_as_int(p.w);
+    if (prim >= 0) {
+      P = f3(p);
+      nrm = f3(q->n);
+    }
+  }
+  const int3 cell = grid_cell(g, P);
+  bool todo = prim >= 0;
+  uint32_t kept = 0;               // photons in the buffer
+  auto test_kept = [&]() {
+    const uint32_t n4 = (kept + 3u) & ~3u;
+    if (kept + lane < n4) {        // filled up with photons that light no side
+      s_x[part][kept + lane] = make_float4(-away, -away, -away, 0.f);
+      s_d[part][kept + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __syncwarp();
+    for (uint32_t i = 0; i < n4; i += 4) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float4 x = s_x[part][i + u];
+        const float ax = Q.x - x.x, ay = Q.y - x.y, az = Q.z - x.z;
+        const float w = fmaf(-inv_r2, fmaf(az, az, fmaf(ay, ay, ax * ax)), 1.0f);
+        if (!(w > 0.0f)) continue;
+        const float4 d = s_d[part][i + u];
+        if (!(N.x * d.x + N.y * d.y + N.z * d.z < 0.0f)) continue;       // arrives on the visible side
+        acc.x = fmaf(x.w, w, acc.x);
+        acc.y = fmaf(d.w, w, acc.y);
+        acc.z = fmaf(s_e[part][i + u], w, acc.z);
+      }
+    }
+    __syncwarp();
+    kept = 0;
+  };
+  for (;;) {
+    // the group: the first pixel left and those within kSpread cells of it
+    const unsigned left = __ballot_sync(0xffffffffu, todo);
+    if (!left) break;
+    const int src = __ffs(left) - 1;
+    const int3 c0 = make_int3(__shfl_sync(0xffffffffu, cell.x, src), __shfl_sync(0xffffffffu, cell.y, src),
+                              __shfl_sync(0xffffffffu, cell.z, src));
+    const bool in = todo && abs(cell.x - c0.x) <= kSpread && abs(cell.y - c0.y) <= kSpread &&
+                    abs(cell.z - c0.z) <= kSpread;
+    todo = todo && !in;
+    Q = in ? P : make_float3(away, away, away);
+    N = in ? nrm : make_float3(0.f, 0.f, 0.f);
+    const int3 lo = make_int3(__reduce_min_sync(0xffffffffu, in ? cell.x : c0.x),
+                              __reduce_min_sync(0xffffffffu, in ? cell.y : c0.y),
+                              __reduce_min_sync(0xffffffffu, in ? cell.z : c0.z));
+    const int3 hi = make_int3(__reduce_max_sync(0xffffffffu, in ? cell.x : c0.x),
+                              __reduce_max_sync(0xffffffffu, in ? cell.y : c0.y),
+                              __reduce_max_sync(0xffffffffu, in ? cell.z : c0.z));
+    float3 bl = make_float3(warp_min(in ? P.x : away), warp_min(in ? P.y : away), warp_min(in ? P.z : away));
+    float3 bh = make_float3(warp_max(in ? P.x : -away), warp_max(in ? P.y : -away), warp_max(in ? P.z : -away));
+    // the box grown by the radius, and by what rounding may take off its corners and the distances
+    const float mag = fmaxf(fmax3(fabsf(bl.x), fabsf(bl.y), fabsf(bl.z)), fmax3(fabsf(bh.x), fabsf(bh.y), fabsf(bh.z)));
+    const float grow = radius * 1.00001f + mag * 4.0e-7f;
+    bl = make_float3(bl.x - grow, bl.y - grow, bl.z - grow);
+    bh = make_float3(bh.x + grow, bh.y + grow, bh.z + grow);
+    // rows of cells around the group (each axis at most once around the grid); a row is two ranges where it wraps
+    const int ny = min(hi.y - lo.y + 1 + 2 * kReach, g.ny), nz = min(hi.z - lo.z + 1 + 2 * kReach, g.nz);
+    const int len = min(hi.x - lo.x + 1 + 2 * kReach, g.nx);
+    const int x0 = wrap(lo.x - kReach, g.nx), over = x0 + len - g.nx;
+    const int rows = ny * nz, ranges = over > 0 ? 2 * rows : rows;
+    for (int r0 = 0; r0 < ranges; r0 += 32) {
+      uint32_t beg = 0, cnt = 0;
+      if (r0 + lane < ranges) {
+        const bool second = r0 + lane >= rows;
+        const int r = second ? r0 + lane - rows : r0 + lane;
+        const uint32_t row = grid_row(g, lo.y - kReach + r % ny, lo.z - kReach + r / ny);
+        beg = starts[row + (second ? 0 : x0)];
+        cnt = starts[row + (second ? over : min(x0 + len, g.nx))] - beg;
+      }
+      uint32_t incl = cnt;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+      const uint32_t shift = beg - (incl - cnt);             // the photon of rank t, if in this lane's range: shift + t
+      for (uint32_t t0 = 32u * part; t0 < total; t0 += 32u * kParts) {
+        const uint32_t t = t0 + lane;
+        int row = 0;                                         // the range that holds rank t: the first with incl > t
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+          if (__shfl_sync(0xffffffffu, incl, row + o - 1) <= t) row += o;
+        const uint32_t i = __shfl_sync(0xffffffffu, shift, row) + t;
+        bool keep = false;
+        float4 x;
+        if (t < total) {
+          x = __ldg(ph.xd + 2 * (size_t)i);
+          keep = x.x >= bl.x && x.x <= bh.x && x.y >= bl.y && x.y <= bh.y && x.z >= bl.z && x.z <= bh.z;
         }
+        const unsigned m = __ballot_sync(0xffffffffu, keep);
+        if (keep) {
+          const uint32_t at = kept + __popc(m & ((1u << lane) - 1u));
+          s_x[part][at] = x;
+          s_d[part][at] = __ldg(ph.xd + 2 * (size_t)i + 1);
+          s_e[part][at] = __ldg(ph.e + i);
+        }
+        kept += __popc(m);
+        if (kept > 32u) test_kept();
+      }
+    }
+    if (kept) test_kept();
   }
+  // the parts of a pixel's sum meet in shared memory
+  s_acc[part][0][lane] = acc.x;
+  s_acc[part][1][lane] = acc.y;
+  s_acc[part][2][lane] = acc.z;
+  __syncthreads();
+  if (part > 0 || !inside) return;
+#pragma unroll
+  for (int q = 1; q < kParts; ++q)
+    acc = acc + make_float3(s_acc[q][0][lane], s_acc[q][1][lane], s_acc[q][2][lane]);
   const float norm = 2.0f / (3.14159265f * radius * radius) / 3.14159265f;   // kernel normalisation and 1/pi
-  float* o = image + 3 * (size_t)px;
-  if (prim >= 0) {
-    const float4 alb = __ldg(sv.prim_alb + prim);
-    o[0] = alb.x * acc.x * norm;
-    o[1] = alb.y * acc.y * norm;
-    o[2] = alb.z * acc.z * norm;
-  } else {
-    o[0] = o[1] = o[2] = 0.0f;
-  }
+  const float4 alb = prim >= 0 ? __ldg(sv.prim_alb + prim) : make_float4(0.f, 0.f, 0.f, 0.f);
+  float* o = image + 3 * ((size_t)pj * c.W + pi);
+  o[0] = alb.x * acc.x * norm;
+  o[1] = alb.y * acc.y * norm;
+  o[2] = alb.z * acc.z * norm;
 }
 
 Cam make_cam(const pv_scene* s, const pv_camera* cam) {
@@ -252,26 +445,49 @@ bool camera_ok(const pv_camera* c) {
   return f[0] * f[0] + f[1] * f[1] + f[2] * f[2] > 0.0 && cr[0] * cr[0] + cr[1] * cr[1] + cr[2] * cr[2] > 0.0;
 }
 
-}  // namespace
-
-namespace {
-
-// Workspace layout: G-buffer, bucket heads, tile sums, photon records.
+// Workspace layout: G-buffer, photons per cell (padded to whole scan
+// tiles), tile sums, photon ranks, sorted photons.
 struct SplatLayout {
-  size_t gbuf, heads, sums, rec, bytes;
-  uint32_t buckets, tiles;
+  size_t gbuf, counts, sums, rank, xd, e, bytes;
+  uint32_t cells;                                   // most cells a grid may have
   SplatLayout(uint64_t photons, uint32_t width, uint32_t height) {
-    buckets = 4096;                                 // a power of two >= the photons, at least one scan tile
-    while (buckets < photons && buckets < (1u << 30)) buckets <<= 1;
-    tiles = buckets / 4096;
+    cells = 4096;                                   // a power of two >= the photons, at least one scan tile
+    while (cells < photons && cells < (1u << 30)) cells <<= 1;
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const size_t npx = (size_t)width * height;
     gbuf = 0;
-    heads = up(gbuf + (size_t)width * height * sizeof(GPixel));
-    sums = up(heads + (size_t)buckets * sizeof(uint32_t));
-    rec = up(sums + (size_t)(tiles + 1) * sizeof(uint32_t));
-    bytes = up(rec + (size_t)photons * sizeof(PhotonRec));
+    counts = up(gbuf + npx * sizeof(GPixel));
+    sums = up(counts + (size_t)tiles(cells) * 4096 * sizeof(uint32_t));
+    rank = up(sums + (size_t)(tiles(cells) + 1) * sizeof(uint32_t));
+    xd = up(rank + (size_t)photons * sizeof(uint32_t));
+    e = up(xd + 2 * (size_t)photons * sizeof(float4));
+    bytes = up(e + (size_t)photons * sizeof(float));
   }
+  // scan tiles over the counters of a grid of c cells and the total behind them
+  static uint32_t tiles(uint32_t c) { return (uint32_t)(((uint64_t)c + 1 + 4095) / 4096); }
 };
+
+// Cells of edge radius / kCellsPerRadius over the scene's extent, each axis
+// with at least 2 kReach + 2 cells; where that is more than ``most`` cells, the
+// longest axes wrap around earlier.
+Grid make_grid(const pv_scene* s, float radius, uint32_t most) {
+  Grid g;
+  g.inv_edge = (float)kCellsPerRadius / radius;
+  int n[3];
+  for (int k = 0; k < 3; ++k) {
+    const double c = ((double)s->box_hi[k] - s->box_lo[k]) * g.inv_edge + 2.0;
+    n[k] = c < 1048576.0 ? std::max((int)c, 2 * kReach + 2) : 1048576;      // NaN: the most
+  }
+  while ((uint64_t)n[0] * n[1] * n[2] > most) {
+    int* longest = std::max_element(n, n + 3);
+    *longest = std::max((*longest + 1) / 2, 2 * kReach + 2);
+  }
+  g.nx = n[0];
+  g.ny = n[1];
+  g.nz = n[2];
+  g.cells = (uint32_t)n[0] * n[1] * n[2];
+  return g;
+}
 
 }  // namespace
 
@@ -285,36 +501,31 @@ extern "C" int pv_splat(pv_scene* s, const pv_paths* paths, const pv_camera* cam
   const int rc = pvh::check_paths(s, paths);
   if (rc != PV_OK) return rc;
   if (!camera_ok(cam) || !d_image || !d_work || !(radius > 0.0f)) return PV_ERR_ARG;
-  if (paths->n > (1u << 27)) return PV_ERR_LIMIT;            // a photon is named by path * 16 + row
+  if (paths->n > (1u << 27)) return PV_ERR_LIMIT;            // photon ranks are 32-bit
   const SplatLayout lay((uint64_t)paths->n * paths->max_bounces, cam->width, cam->height);
   if (work_bytes < lay.bytes || (reinterpret_cast<uintptr_t>(d_work) & 255u)) return PV_ERR_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   s->last_stream = st;
   const Cam c = make_cam(s, cam);
-  const size_t npx = (size_t)cam->width * cam->height;
+  const Grid g = make_grid(s, radius, lay.cells);
   char* w = static_cast<char*>(d_work);
   GPixel* gbuf = reinterpret_cast<GPixel*>(w + lay.gbuf);
-  uint32_t* heads = reinterpret_cast<uint32_t*>(w + lay.heads);
+  uint32_t* counts = reinterpret_cast<uint32_t*>(w + lay.counts);
   uint32_t* sums = reinterpret_cast<uint32_t*>(w + lay.sums);
-  PhotonRec* rec = reinterpret_cast<PhotonRec*>(w + lay.rec);
+  uint32_t* rank = reinterpret_cast<uint32_t*>(w + lay.rank);
+  const Photons ph = {reinterpret_cast<float4*>(w + lay.xd), reinterpret_cast<float*>(w + lay.e)};
   const pvk::SceneView sv = pvh::view(s);
-  k_gbuffer<<<(unsigned)((npx + 255) / 256), 256, 0, st>>>(sv, c, gbuf);
-  Grid g;
-  g.inv_r = 1.0f / radius;
-  g.mask = lay.buckets - 1;
-  PV_CHECK(cudaMemsetAsync(heads, 0, (size_t)lay.buckets * sizeof(uint32_t), st));
+  const uint32_t tiles = SplatLayout::tiles(g.cells);
+  PV_CHECK(cudaMemsetAsync(counts, 0, (size_t)tiles * 4096 * sizeof(uint32_t), st));
+  k_gbuffer<<<((c.W + 15) / 16) * ((c.H + 15) / 16), 256, 0, st>>>(sv, c, gbuf);
   const uint32_t n = paths->n;
   const float4* pa = reinterpret_cast<const float4*>(paths->pa);
   const float4* pb = reinterpret_cast<const float4*>(paths->pb);
-  if (n) {
-    const uint32_t blocks = std::min<uint32_t>((n + 255) / 256, 16u * (uint32_t)s->num_sms);
-    k_grid_fill<0><<<blocks, 256, 0, st>>>(c, g, radius, n, s->B, paths->info, pa, pb, heads, rec);
-    k_tile_sums<<<lay.tiles, 1024, 0, st>>>(heads, sums);
-    pvh::exclusive_scan(sums, lay.tiles, st);
-    k_tile_scan<<<lay.tiles, 1024, 0, st>>>(heads, sums);
-    k_grid_fill<1><<<blocks, 256, 0, st>>>(c, g, radius, n, s->B, paths->info, pa, pb, heads, rec);
-  }
-  k_gather<<<(unsigned)((npx + 255) / 256), 256, 0, st>>>(sv, c, g, radius, n, paths->origin, pa, gbuf, heads, rec,
-                                                          d_image);
+  if (n) k_photon_count<<<(n + 255) / 256, 256, 0, st>>>(c, g, radius, n, s->B, paths->info, pa, counts, rank);
+  k_tile_sums<<<tiles, 1024, 0, st>>>(counts, sums);
+  pvh::exclusive_scan(sums, tiles, st);
+  k_tile_scan<<<tiles, 1024, 0, st>>>(counts, sums);
+  if (n) k_photon_place<<<(n + 255) / 256, 256, 0, st>>>(g, n, s->B, paths->info, paths->origin, pa, pb, counts, rank, ph);
+  k_gather<<<((c.W + 7) / 8) * ((c.H + 3) / 4), 32 * kParts, 0, st>>>(sv, c, g, radius, gbuf, counts, ph, d_image);
   return pvh::cuda_status(cudaGetLastError());
 }
