@@ -159,21 +159,27 @@ __global__ void __launch_bounds__(256) k_b_dm_prune(const BScene* S, const BFram
   block_add_n<1>(ctr, val, s_red);
 }
 
-// Pass 2 (dm_commit_path): flag[p] becomes the free-path flag for the compaction.
+// Pass 2 (dm_commit_block): flag[p] becomes the free-path flag for the compaction.
 __global__ void __launch_bounds__(256) k_b_dm_commit(const BScene* S, const BFrame* F, uint32_t sc, uint32_t* flag,
                                                      uint32_t* free_count) {
+  __shared__ uint32_t s_free[PV_MAX_LIGHTS];
   const BScene& B = S[sc];
-  const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= B.V.n) return;
-  flag[p] = dm_commit_path(F[sc].L, p, B.V.info, flag[p], free_count);
+  dm_commit_block(F[sc].L, blockIdx.x * blockDim.x + threadIdx.x, B.V.n, B.V.info, flag, free_count, s_free);
 }
 
-__global__ void k_b_dm_deficit(const BFrame* F, uint32_t sc, uint32_t l, uint32_t* def) {
+// The deficits' prefix of light l (dm_deficit_tile, then dm_prefix_tile).
+__global__ void __launch_bounds__(kDmThreads) k_b_dm_deficit(const BFrame* F, uint32_t sc, uint32_t l, uint32_t* def,
+                                                             uint32_t* sums) {
+  __shared__ uint32_t sh[kDmThreads / 32];
   const FrameLights& L = F[sc].L;
-  if (!dm_moved(L, l)) return;
-  const DmLight& D = L.dm[l];
-  for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c <= D.cells; c += gridDim.x * blockDim.x)
-    def[c] = dm_deficit(D, c);
+  if (dm_moved(L, l)) dm_deficit_tile(L.dm[l], blockIdx.x, def, sums, sh);
+}
+
+__global__ void __launch_bounds__(kDmThreads) k_b_dm_prefix(const BFrame* F, uint32_t sc, uint32_t l, uint32_t* def,
+                                                            const uint32_t* sums) {
+  __shared__ uint32_t sh[64];
+  const FrameLights& L = F[sc].L;
+  if (dm_moved(L, l)) dm_prefix_tile(L.dm[l].cells, blockIdx.x, def, sums, sh);
 }
 
 // Fill (dm_fill_path) for the free paths of light l, listed after those of the lights before it.
@@ -823,8 +829,9 @@ int enqueue_frame(pv_batch* b, cudaStream_t st, bool vis, const pv_batch_config&
     const FrameLights L = pvh::frame_lights(s);
     for (uint32_t l = 0; l < L.n; ++l) {
       if (!L.dm[l].dims) continue;
-      k_b_dm_deficit<<<(L.dm[l].cells + 256) / 256, 256, 0, st>>>(b->d_frames, i, l, s->dm_scan);
-      pvh::exclusive_scan(s->dm_scan, L.dm[l].cells + 1, st);
+      const uint32_t tiles = dm_tiles(L.dm[l].cells);
+      k_b_dm_deficit<<<tiles, kDmThreads, 0, st>>>(b->d_frames, i, l, s->dm_scan, s->dm_sums);
+      k_b_dm_prefix<<<tiles, kDmThreads, 0, st>>>(b->d_frames, i, l, s->dm_scan, s->dm_sums);
       const uint32_t fb = std::min<uint32_t>((s->lights_new[l].n_paths + 255) / 256, 8u * (uint32_t)s->num_sms);
       k_b_dm_fill<<<std::max<uint32_t>(fb, 1u), 256, 0, st>>>(b->d_scenes, b->d_frames, i, l, s->dm_free, s->dm_ctr,
                                                              s->dm_scan);

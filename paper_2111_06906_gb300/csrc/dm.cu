@@ -4,7 +4,7 @@
 //     counts as computed; k_dm_commit edits the counts and flags the free
 //     paths (pruned, or no longer from the light);
 //   the free paths are compacted into an ascending list;
-//   fill DM_C: k_dm_deficit + an exclusive scan give each cell's range of
+//   fill DM_C: k_dm_deficit and k_dm_prefix give each cell's range of
 //     deficit slots; k_dm_fill gives the j-th free path of a light the cell
 //     whose range holds j (any further ones spread evenly) and counts it.
 // Every decision is an integer one (counts, the 24-bit draw), so the result
@@ -36,19 +36,23 @@ __global__ void __launch_bounds__(256) k_dm_prune(FrameLights L, uint32_t n, uin
   block_add_n<1>(ctr, val, s_red);
 }
 
-// Pass 2 (dm_commit_path): the pruned paths leave their cells; every fresh
+// Pass 2 (dm_commit_block): the pruned paths leave their cells; every fresh
 // emission of a light with a moved map is flagged free (bit 30, for the
 // compaction) and counted.
 __global__ void __launch_bounds__(256) k_dm_commit(FrameLights L, uint32_t n, const uint32_t* info, uint32_t* flag,
                                                    uint32_t* free_count) {
-  const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
-  flag[p] = dm_commit_path(L, p, info, flag[p], free_count);
+  __shared__ uint32_t s_free[PV_MAX_LIGHTS];
+  dm_commit_block(L, blockIdx.x * blockDim.x + threadIdx.x, n, info, flag, free_count, s_free);
 }
 
-__global__ void k_dm_deficit(DmLight D, uint32_t* def) {
-  for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c <= D.cells; c += gridDim.x * blockDim.x)
-    def[c] = dm_deficit(D, c);
+__global__ void __launch_bounds__(kDmThreads) k_dm_deficit(DmLight D, uint32_t* def, uint32_t* sums) {
+  __shared__ uint32_t sh[kDmThreads / 32];
+  dm_deficit_tile(D, blockIdx.x, def, sums, sh);
+}
+
+__global__ void __launch_bounds__(kDmThreads) k_dm_prefix(uint32_t cells, uint32_t* def, const uint32_t* sums) {
+  __shared__ uint32_t sh[64];
+  dm_prefix_tile(cells, blockIdx.x, def, sums, sh);
 }
 
 // Fill (dm_fill_path) for the free paths of light l, listed after those of
@@ -95,8 +99,8 @@ int dm_frame(pv_scene* s, const pv_paths* p, const FrameLights& L, const pv_veri
   for (uint32_t l = 0; l < s->n_lights; ++l) {
     if (!((moved >> l) & 1u)) continue;
     const DmLight& D = L.dm[l];
-    k_dm_deficit<<<(D.cells + 256) / 256, 256, 0, st>>>(D, s->dm_scan);
-    exclusive_scan(s->dm_scan, D.cells + 1, st);
+    k_dm_deficit<<<dm_tiles(D.cells), kDmThreads, 0, st>>>(D, s->dm_scan, s->dm_sums);
+    k_dm_prefix<<<dm_tiles(D.cells), kDmThreads, 0, st>>>(D.cells, s->dm_scan, s->dm_sums);
     const uint32_t fb = std::min<uint32_t>((s->lights_new[l].n_paths + 255) / 256, 8u * (uint32_t)s->num_sms);
     k_dm_fill<<<std::max<uint32_t>(fb, 1u), 256, 0, st>>>(L, l, s->dm_free, s->dm_ctr, s->dm_scan, p->info, stats);
   }

@@ -101,6 +101,7 @@ struct pv_scene {
   uint32_t* dm_flag = nullptr;                // [n_paths] pruned mark, then free-path flags
   uint32_t* dm_free = nullptr;                // [n_paths] free paths, ascending
   uint32_t* dm_scan = nullptr;                // [max cells + 1] deficits, then their exclusive prefix
+  uint32_t* dm_sums = nullptr;                // [tiles of the largest map] sums of its tiles (behind dm_scan)
   uint32_t* dm_ctr = nullptr;                 // [8] free paths per light, free-list length
   bool has_dm = false;
   uint64_t* b_keys[2] = {nullptr, nullptr};   // [n_paths] budget ranking sort keys (ping-pong)

@@ -5,6 +5,7 @@
 #include <utility>
 #include <vector>
 
+#include "dm_core.cuh"
 #include "pv_scene.h"
 
 using namespace pvk;
@@ -248,7 +249,8 @@ extern "C" int pv_build_scene(const pv_scene_desc* d, void* stream, pv_scene** o
   if (s->has_dm) {
     fail(cudaMalloc(&s->dm_flag, (size_t)s->n_paths_total * sizeof(uint32_t)));
     fail(cudaMalloc(&s->dm_free, (size_t)s->n_paths_total * sizeof(uint32_t)));
-    fail(cudaMalloc(&s->dm_scan, ((size_t)dm_max + 1) * sizeof(uint32_t)));
+    fail(cudaMalloc(&s->dm_scan, ((size_t)dm_max + 1 + dm_tiles(dm_max)) * sizeof(uint32_t)));
+    s->dm_sums = s->dm_scan + dm_max + 1;
     fail(cudaMalloc(&s->dm_ctr, 8 * sizeof(uint32_t)));
   }
   for (int b = 0; b < 2; ++b) {
