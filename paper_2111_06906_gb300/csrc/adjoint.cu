@@ -19,6 +19,7 @@
 // stored photons.  The adjoint runs the chain backwards per path:
 //   dx_k/dx_{k-1} = I - d nu^T/(nu.d),  dx_k/dq_k = d nu^T/(nu.d),
 //   dx_1/do = I - d0 nu^T/(nu.d0),      dx_1/dd0 = tau_1 (I - d0 nu^T/(nu.d0)).
+#include <algorithm>
 #include <cstring>
 
 #include "pv_scene.h"
@@ -350,30 +351,168 @@ __global__ void __launch_bounds__(128) k_adjoint(SceneView sv, FrameLights L, Mo
     if (s_acc[j] != 0.f) atomicAdd(dtheta + j, s_acc[j]);
 }
 
-// Sort keys of the listed paths: high word = complemented score bits (score
-// descending); unlisted slots (and ids out of range) sort last.  The radix sort over the high word is
-// stable, and the list is ascending, so equal scores keep ascending ids.
-__global__ void k_budget_keys(const uint32_t* list, const uint32_t* count, const float* score, uint32_t n,
-                              uint64_t* keys, uint32_t* vals) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const uint32_t id = i < min(*count, n) ? list[i] : 0xffffffffu;
-  if (id < n) {
-    const float s = score[id];
-    const uint32_t bits = s > 0.f ? __float_as_uint(s) : 0u;     // NaN, zero and negatives rank last
-    keys[i] = ((uint64_t)(~bits) << 32) | id;
-    vals[i] = id;
-  } else {
-    keys[i] = ~0ull;
-    vals[i] = 0xffffffffu;
+// ---- ray budget: the ``budget`` listed paths of largest score by radix select
+// A listed path's key is its score's bits if the score is positive, else 0 (NaN,
+// zero and negatives rank last); equal keys rank by their place in the list.  Three
+// histograms of 11, 11 and 9 key bits, each over the keys that share the bits
+// picked so far, give the key T of the last path kept and how many paths of key
+// T are kept; then the paths above T, and the first of those at T, are marked.
+// Sorting all n slots on 32 bits instead took 12 launches, four of them a scan by
+// one block: 151 us for 400k paths, where these five take 22 us.
+constexpr uint32_t kBudgetThreads = 256, kBudgetBins = 2048, kBudgetItems = 8;
+constexpr uint32_t kBudgetStep = kBudgetThreads * kBudgetItems;
+constexpr uint32_t kNoKey = 0xFFFFFFFFu;     // an id out of range
+
+// What a level has picked: the key bits so far and how many paths of those bits are still to be kept.
+struct BudgetState {
+  uint32_t prefix, want;
+};
+
+// Workspace (32-bit words): three histograms, three states, ties per tile.
+struct BudgetWork {
+  uint32_t hist[3][kBudgetBins];
+  BudgetState state[3];
+  uint32_t ties[pvh::kBudgetTiles];
+};
+static_assert(sizeof(BudgetWork) <= pvh::kBudgetWords * sizeof(uint32_t), "workspace of the ray budget");
+
+// The highest bin b whose count, with the counts of all bins above it, reaches
+// ``want`` (> 0, at most the total); want becomes what bin b has to give.  All
+// threads of the block call; ``sh``: 10 words.
+__device__ __forceinline__ uint32_t budget_pick(const uint32_t* hist, uint32_t& want, uint32_t* sh) {
+  constexpr uint32_t kPer = kBudgetBins / kBudgetThreads;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  const uint32_t top = kBudgetBins - 1u - kPer * threadIdx.x;
+  uint32_t v[kPer], own = 0;
+#pragma unroll
+  for (uint32_t k = 0; k < kPer; ++k) own += v[k] = hist[top - k];
+  uint32_t incl = own;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+    if ((int)lane >= o) incl += y;
+  }
+  if (lane == 31u) sh[warp] = incl;
+  __syncthreads();
+  uint32_t above = incl - own;
+  for (uint32_t w = 0; w < warp; ++w) above += sh[w];
+#pragma unroll
+  for (uint32_t k = 0; k < kPer; ++k) {
+    if (above < want && want <= above + v[k]) {
+      sh[8] = top - k;
+      sh[9] = want - above;
+    }
+    above += v[k];
+  }
+  __syncthreads();
+  const uint32_t bin = sh[8];
+  want = sh[9];
+  return bin;
+}
+
+// Level kLevel (0, 1, 2): pick the bin of the level before and count this
+// level's bins over the keys that match.  Level 0 also makes the keys and
+// clears the marks.
+template <int kLevel>
+__global__ void __launch_bounds__(kBudgetThreads) k_budget_hist(const uint32_t* list, const uint32_t* count,
+                                                                const float* score, uint32_t n, uint32_t budget,
+                                                                uint32_t* keys, uint32_t* marks, BudgetWork* W) {
+  __shared__ uint32_t s_hist[kBudgetBins];
+  __shared__ uint32_t sh[10];
+  constexpr uint32_t kShift = kLevel == 0 ? 20u : kLevel == 1 ? 9u : 0u;      // lowest bit of this level
+  constexpr uint32_t kMask = kLevel == 2 ? 511u : 2047u;
+  constexpr uint32_t kAbove = kLevel == 1 ? 20u : 9u;                         // lowest bit of the levels before
+  for (uint32_t i = threadIdx.x; i < kBudgetBins; i += kBudgetThreads) s_hist[i] = 0u;
+  BudgetState st = {0u, 0u};
+  if (kLevel > 0) {
+    if (kLevel == 1) {
+      uint32_t total = 0;                      // paths in range
+      for (uint32_t i = threadIdx.x & 31u; i < kBudgetBins; i += 32u) total += W->hist[0][i];
+      st.want = min(budget, __reduce_add_sync(0xffffffffu, total));
+    } else {
+      st = W->state[kLevel - 2];
+    }
+    if (st.want) st.prefix = st.prefix * kBudgetBins + budget_pick(W->hist[kLevel - 1], st.want, sh);
+    if (blockIdx.x == 0 && threadIdx.x == 0) W->state[kLevel - 1] = st;
+    if (!st.want) return;
+  }
+  __syncthreads();
+  const uint32_t m = min(*count, n);
+  const uint32_t end = kLevel == 0 ? n : m;
+  for (uint32_t i = blockIdx.x * kBudgetThreads + threadIdx.x; i < end; i += gridDim.x * kBudgetThreads) {
+    uint32_t key = kNoKey;
+    if (kLevel == 0) {
+      marks[i] = 0u;
+      if (i >= m) continue;
+      const uint32_t id = list[i];
+      if (id < n) {
+        const float s = score[id];
+        key = s > 0.f ? __float_as_uint(s) : 0u;
+      }
+      keys[i] = key;
+      if (key != kNoKey) atomicAdd(s_hist + (key >> kShift), 1u);
+    } else {
+      key = keys[i];
+      if (key != kNoKey && key >> kAbove == st.prefix) atomicAdd(s_hist + ((key >> kShift) & kMask), 1u);
+    }
+  }
+  __syncthreads();
+  for (uint32_t i = threadIdx.x; i < kBudgetBins; i += kBudgetThreads)
+    if (s_hist[i]) atomicAdd(&W->hist[kLevel][i], s_hist[i]);
+}
+
+// The last key T, and the paths of key T in every tile of the list (a block per tile).
+__global__ void __launch_bounds__(kBudgetThreads) k_budget_ties(const uint32_t* count, uint32_t n, uint32_t tile,
+                                                                const uint32_t* keys, BudgetWork* W) {
+  __shared__ uint32_t sh[10];
+  BudgetState st = W->state[1];
+  if (st.want) st.prefix = st.prefix * 512u + budget_pick(W->hist[2], st.want, sh);
+  if (blockIdx.x == 0 && threadIdx.x == 0) W->state[2] = st;
+  if (!st.want) return;
+  const uint64_t b = (uint64_t)blockIdx.x * tile;
+  const uint32_t m = min(*count, n), e = (uint32_t)min(b + tile, (uint64_t)m);
+  uint32_t ties = 0;
+  for (uint64_t i = b + threadIdx.x; i < e; i += kBudgetThreads) ties += keys[i] == st.prefix ? 1u : 0u;
+  ties = __reduce_add_sync(0xffffffffu, ties);
+  __syncthreads();
+  if ((threadIdx.x & 31u) == 0u) sh[threadIdx.x >> 5] = ties;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint32_t t = 0;
+    for (uint32_t w = 0; w < kBudgetThreads / 32u; ++w) t += sh[w];
+    W->ties[blockIdx.x] = t;
   }
 }
 
-// Mark the first min(budget, count) sorted paths (bit 30, as in the info word).
-__global__ void k_budget_mark(const uint32_t* vals, const uint32_t* count, uint32_t budget, uint32_t n,
-                              uint32_t* flags) {
-  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < budget && i < min(*count, n) && vals[i] < n) flags[vals[i]] = PV_INFO_REPLACE;
+// Mark (bit 30, as in the info word) the paths above T and the first state.want of those at T.
+__global__ void __launch_bounds__(kBudgetThreads) k_budget_mark(const uint32_t* list, const uint32_t* count, uint32_t n,
+                                                                uint32_t tile, const uint32_t* keys,
+                                                                const BudgetWork* W, uint32_t* marks) {
+  __shared__ uint32_t sh[kBudgetThreads / 32u + 1u];
+  const BudgetState st = W->state[2];
+  if (!st.want) return;
+  const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+  uint32_t before = 0;                         // ties in the tiles before this one
+  for (uint32_t t = lane; t < blockIdx.x; t += 32u) before += W->ties[t];
+  before = __reduce_add_sync(0xffffffffu, before);
+  const uint64_t b = (uint64_t)blockIdx.x * tile;
+  const uint32_t m = min(*count, n), e = (uint32_t)min(b + tile, (uint64_t)m);
+  for (uint64_t i0 = b; i0 < e; i0 += kBudgetThreads) {
+    const uint64_t i = i0 + threadIdx.x;
+    const uint32_t key = i < e ? keys[i] : kNoKey;
+    const bool tie = key == st.prefix;
+    const unsigned tm = __ballot_sync(0xffffffffu, tie);
+    if (lane == 0) sh[warp] = __popc(tm);
+    __syncthreads();
+    uint32_t rank = before + __popc(tm & ((1u << lane) - 1u)), all = 0;
+    for (uint32_t w = 0; w < kBudgetThreads / 32u; ++w) {
+      if (w < warp) rank += sh[w];
+      all += sh[w];
+    }
+    before += all;
+    if (key != kNoKey && (key > st.prefix || (tie && rank < st.want))) marks[list[i]] = PV_INFO_REPLACE;
+    __syncthreads();
+  }
 }
 
 int model_args(const pv_scene* s, const pv_paths* p, const float* theta, uint32_t width, uint32_t height,
@@ -458,13 +597,18 @@ extern "C" int pv_budget_list(pv_scene* s, const uint32_t* d_list, const uint32_
   s->last_stream = st;
   const uint32_t n = s->n_paths_total;
   if (n == 0) return pvh::cuda_status(cudaMemsetAsync(d_out_count, 0, sizeof(uint32_t), st));
-  uint64_t *k0 = s->b_keys[0], *k1 = s->b_keys[1];
-  uint32_t *v0 = s->b_vals[0], *v1 = s->b_vals[1];
-  k_budget_keys<<<(n + 255) / 256, 256, 0, st>>>(d_list, d_count, d_score, n, k0, v0);
-  pvh::radix_sort(k0, v0, k1, v1, n, s->b_hist, 32, 64, st);
-  PV_CHECK(cudaMemsetAsync(s->ws_mask, 0, (size_t)n * sizeof(uint32_t), st));
-  const uint32_t m = budget < n ? budget : n;
-  if (m) k_budget_mark<<<(m + 255) / 256, 256, 0, st>>>(v0, d_count, m, n, s->ws_mask);
+  BudgetWork* W = reinterpret_cast<BudgetWork*>(s->b_work);
+  uint32_t* const keys = s->b_keys;
+  PV_CHECK(cudaMemsetAsync(W, 0, sizeof W->hist, st));
+  const uint32_t blocks = std::min((n + kBudgetStep - 1) / kBudgetStep, 4u * (uint32_t)s->num_sms);
+  k_budget_hist<0><<<blocks, kBudgetThreads, 0, st>>>(d_list, d_count, d_score, n, budget, keys, s->ws_mask, W);
+  k_budget_hist<1><<<blocks, kBudgetThreads, 0, st>>>(d_list, d_count, d_score, n, budget, keys, s->ws_mask, W);
+  k_budget_hist<2><<<blocks, kBudgetThreads, 0, st>>>(d_list, d_count, d_score, n, budget, keys, s->ws_mask, W);
+  // tiles of whole steps, at most kBudgetTiles of them
+  const uint32_t tile = std::max<uint32_t>((n / pvh::kBudgetTiles / kBudgetStep + 1u) * kBudgetStep, kBudgetStep);
+  const uint32_t tiles = (n + tile - 1) / tile;
+  k_budget_ties<<<tiles, kBudgetThreads, 0, st>>>(d_count, n, tile, keys, W);
+  k_budget_mark<<<tiles, kBudgetThreads, 0, st>>>(d_list, d_count, n, tile, keys, W, s->ws_mask);
   pvh::launch_compact(s, s->ws_mask, n, d_out, d_out_count, nullptr, st);
   return pvh::cuda_status(cudaGetLastError());
 }

@@ -104,9 +104,8 @@ struct pv_scene {
   uint32_t* dm_sums = nullptr;                // [tiles of the largest map] sums of its tiles (behind dm_scan)
   uint32_t* dm_ctr = nullptr;                 // [8] free paths per light, free-list length
   bool has_dm = false;
-  uint64_t* b_keys[2] = {nullptr, nullptr};   // [n_paths] budget ranking sort keys (ping-pong)
-  uint32_t* b_vals[2] = {nullptr, nullptr};
-  uint32_t* b_hist = nullptr;                 // [256][radix tiles of n_paths]
+  uint32_t* b_keys = nullptr;                 // [n_paths] keys of the ray budget's ranking
+  uint32_t* b_work = nullptr;                 // [kBudgetWords] its histograms and counts
   int* status = nullptr;             // sticky device status
   cudaStream_t last_stream = nullptr;
 
@@ -125,6 +124,8 @@ struct ContArgs;                     // verify_core.cuh
 
 namespace pvh {
 
+constexpr uint32_t kBudgetTiles = 1024;       // list tiles of the ray budget's tie counts, at most
+constexpr uint32_t kBudgetWords = 3 * 2048 + 6 + kBudgetTiles;
 constexpr int kStageEvents = 5;      // events per timed pv_verify_retrace call
 constexpr int kTraceThreads = 128;
 constexpr int kVerifyThreads = 256;

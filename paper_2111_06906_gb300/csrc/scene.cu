@@ -53,8 +53,8 @@ void free_scene(pv_scene* s) {
   void* ptrs[] = {s->nodes, s->wnodes, s->wsrc, s->wcount, s->cq, s->tris, s->root, s->d_local, s->d_tri_prim, s->d_leaf_parent, s->d_node_parent,
                   s->d_fit_flags, s->w_link, s->w_nch, s->w_arrive, s->t_link, s->pair_link, s->pair_tri, s->pair_warps, s->pair_acc, s->pair_count, s->obox, s->d_tri_slot, s->objs, s->groups, s->r_keys[0], s->r_keys[1], s->r_vals[0], s->r_vals[1],
                   s->r_hist, s->r_tris, s->r_local, s->r_prim, s->prim_slot, s->prim_dyn, s->prim_alb, s->prim_nrm,
-                  s->xf_old, s->xf_new, s->ws_mask, s->ws_cont, s->ws_list, s->ws_touched, s->ws_tiles, s->ws_ctr, s->status, s->b_keys[0], s->b_keys[1],
-                  s->b_vals[0], s->b_vals[1], s->b_hist, s->dm_c[0], s->dm_c[1], s->dm_c[2], s->dm_c[3],
+                  s->xf_old, s->xf_new, s->ws_mask, s->ws_cont, s->ws_list, s->ws_touched, s->ws_tiles, s->ws_ctr, s->status, s->b_keys, s->b_work,
+                  s->dm_c[0], s->dm_c[1], s->dm_c[2], s->dm_c[3],
                   s->dm_flag, s->dm_free, s->dm_scan, s->dm_ctr};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -253,11 +253,8 @@ extern "C" int pv_build_scene(const pv_scene_desc* d, void* stream, pv_scene** o
     s->dm_sums = s->dm_scan + dm_max + 1;
     fail(cudaMalloc(&s->dm_ctr, 8 * sizeof(uint32_t)));
   }
-  for (int b = 0; b < 2; ++b) {
-    fail(cudaMalloc(&s->b_keys[b], (size_t)s->n_paths_total * sizeof(uint64_t)));
-    fail(cudaMalloc(&s->b_vals[b], (size_t)s->n_paths_total * sizeof(uint32_t)));
-  }
-  fail(cudaMalloc(&s->b_hist, 256 * (size_t)pvh::radix_tiles(s->n_paths_total) * sizeof(uint32_t)));
+  fail(cudaMalloc(&s->b_keys, (size_t)s->n_paths_total * sizeof(uint32_t)));
+  fail(cudaMalloc(&s->b_work, pvh::kBudgetWords * sizeof(uint32_t)));
   if (rc != PV_OK) {
     free_scene(s);
     return rc;
