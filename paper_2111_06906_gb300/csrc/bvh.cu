@@ -421,7 +421,7 @@ __global__ void k_wide_links(const WNode* wdyn, const uint32_t* n_wide, int w_of
                              uint8_t* w_nch, uint32_t* t_link) {
   const uint32_t w = blockIdx.x * blockDim.x + threadIdx.x;
   if (w >= *n_wide) return;
-  const int4 ch = wdyn[w].child;
+  const int4 ch = *reinterpret_cast<const int4*>(wnode_chunk(wdyn + w, kChild));
   const int c4[4] = {ch.x, ch.y, ch.z, ch.w};
   uint32_t m = 0;
   for (int c = 0; c < 4; ++c) {

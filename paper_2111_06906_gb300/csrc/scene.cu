@@ -86,7 +86,6 @@ SceneView view(const pv_scene* s) {
   v.moved = s->moved;
   v.max_visits = s->visit_limit ? s->visit_limit : 2u * (s->n_static_refs + s->n_dyn_tris) + 256u;
   v.status = s->status;
-  v.n_static_wide = s->w_dyn_off;
   return v;
 }
 
@@ -325,10 +324,13 @@ int stack_need(pv_scene* s, uint32_t* out) {
     if (cudaStreamSynchronize(s->last_stream) != cudaSuccess) return PV_ERR_CUDA;
     int root = INT32_MIN;
     if (cudaMemcpy(&root, s->root, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return PV_ERR_CUDA;
-    std::vector<int4> ch(s->n_wide);
-    if (s->n_wide && cudaMemcpy2D(ch.data(), sizeof(int4), &s->wnodes[0].child, sizeof(WNode), sizeof(int4), s->n_wide,
-                                  cudaMemcpyDeviceToHost) != cudaSuccess)
+    std::vector<float4> places(8 * (size_t)s->n_wide);
+    if (s->n_wide && cudaMemcpy(places.data(), s->wnodes, (size_t)s->n_wide * sizeof(WNode), cudaMemcpyDeviceToHost) !=
+                         cudaSuccess)
       return PV_ERR_CUDA;
+    std::vector<int4> ch(s->n_wide);
+    for (uint32_t i = 0; i < s->n_wide; ++i)   // the place of a chunk follows from the node's device address
+      std::memcpy(&ch[i], &places[8 * (size_t)i + (wnode_chunk(s->wnodes + i, kChild) - s->wnodes[i].place)], sizeof(int4));
     // deepest root-to-leaf path, counted in wide nodes (iterative, bounded)
     uint32_t height = 0;
     std::vector<std::pair<int, uint32_t>> todo;

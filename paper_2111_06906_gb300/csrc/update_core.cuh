@@ -187,12 +187,12 @@ __device__ __forceinline__ void refit_leaf(const float* xf_slot, bool moved_lane
   if (link == 0xFFFFFFFFu) return;             // a one-triangle object: the triangle is the root
   WNode* nd = R.wdyn + (link >> 2);
   const uint32_t c = link & 3u;
-  (&nd->lox.x)[c] = blo.x;
-  (&nd->hix.x)[c] = bhi.x;
-  (&nd->loy.x)[c] = blo.y;
-  (&nd->hiy.x)[c] = bhi.y;
-  (&nd->loz.x)[c] = blo.z;
-  (&nd->hiz.x)[c] = bhi.z;
+  *wnode_float(nd, kLoX, c) = blo.x;
+  *wnode_float(nd, kHiX, c) = bhi.x;
+  *wnode_float(nd, kLoY, c) = blo.y;
+  *wnode_float(nd, kHiY, c) = bhi.y;
+  *wnode_float(nd, kLoZ, c) = blo.z;
+  *wnode_float(nd, kHiZ, c) = bhi.z;
 }
 
 // The refit by climbing: after refit_leaf, the last child to arrive at a wide
@@ -213,23 +213,23 @@ __device__ __forceinline__ void refit_tri(const float* xf_slot, bool moved_lane,
     bhi = make_float3(-3.0e38f, -3.0e38f, -3.0e38f);
     WNode* nd = R.wdyn + w;
     for (uint32_t q = 0; q < m; ++q) {
-      blo.x = fminf(blo.x, __ldcg(&nd->lox.x + q));
-      blo.y = fminf(blo.y, __ldcg(&nd->loy.x + q));
-      blo.z = fminf(blo.z, __ldcg(&nd->loz.x + q));
-      bhi.x = fmaxf(bhi.x, __ldcg(&nd->hix.x + q));
-      bhi.y = fmaxf(bhi.y, __ldcg(&nd->hiy.x + q));
-      bhi.z = fmaxf(bhi.z, __ldcg(&nd->hiz.x + q));
+      blo.x = fminf(blo.x, __ldcg(wnode_float(nd, kLoX, q)));
+      blo.y = fminf(blo.y, __ldcg(wnode_float(nd, kLoY, q)));
+      blo.z = fminf(blo.z, __ldcg(wnode_float(nd, kLoZ, q)));
+      bhi.x = fmaxf(bhi.x, __ldcg(wnode_float(nd, kHiX, q)));
+      bhi.y = fmaxf(bhi.y, __ldcg(wnode_float(nd, kHiY, q)));
+      bhi.z = fmaxf(bhi.z, __ldcg(wnode_float(nd, kHiZ, q)));
     }
     link = R.w_link[w];
     if (link == 0xFFFFFFFFu) return;
     WNode* up = R.wdyn + (link >> 2);
     const uint32_t c = link & 3u;
-    (&up->lox.x)[c] = blo.x;
-    (&up->hix.x)[c] = bhi.x;
-    (&up->loy.x)[c] = blo.y;
-    (&up->hiy.x)[c] = bhi.y;
-    (&up->loz.x)[c] = blo.z;
-    (&up->hiz.x)[c] = bhi.z;
+    *wnode_float(up, kLoX, c) = blo.x;
+    *wnode_float(up, kHiX, c) = bhi.x;
+    *wnode_float(up, kLoY, c) = blo.y;
+    *wnode_float(up, kHiY, c) = bhi.y;
+    *wnode_float(up, kLoZ, c) = blo.z;
+    *wnode_float(up, kHiZ, c) = bhi.z;
   }
 }
 
@@ -261,12 +261,12 @@ struct PairArgs {
 __device__ __forceinline__ void write_slot(const RefitArgs& R, uint32_t link, const int (&r)[6]) {
   WNode* nd = R.wdyn + (link >> 2);
   const uint32_t c = link & 3u;
-  (&nd->lox.x)[c] = of_ord(r[0]);
-  (&nd->loy.x)[c] = of_ord(r[1]);
-  (&nd->loz.x)[c] = of_ord(r[2]);
-  (&nd->hix.x)[c] = of_ord(r[3]);
-  (&nd->hiy.x)[c] = of_ord(r[4]);
-  (&nd->hiz.x)[c] = of_ord(r[5]);
+  *wnode_float(nd, kLoX, c) = of_ord(r[0]);
+  *wnode_float(nd, kLoY, c) = of_ord(r[1]);
+  *wnode_float(nd, kLoZ, c) = of_ord(r[2]);
+  *wnode_float(nd, kHiX, c) = of_ord(r[3]);
+  *wnode_float(nd, kHiY, c) = of_ord(r[4]);
+  *wnode_float(nd, kHiZ, c) = of_ord(r[5]);
 }
 
 // Pair q (every lane of the warp calls it).
@@ -398,20 +398,20 @@ __device__ __forceinline__ void write_wide(WNode* w, const float (*box)[6], cons
     }
     c[i] = i < m ? ref[i] : INT32_MIN;
   }
-  w->lox = make_float4(b[0][0], b[1][0], b[2][0], b[3][0]);
-  w->hix = make_float4(b[0][3], b[1][3], b[2][3], b[3][3]);
-  w->loy = make_float4(b[0][1], b[1][1], b[2][1], b[3][1]);
-  w->hiy = make_float4(b[0][4], b[1][4], b[2][4], b[3][4]);
-  w->loz = make_float4(b[0][2], b[1][2], b[2][2], b[3][2]);
-  w->hiz = make_float4(b[0][5], b[1][5], b[2][5], b[3][5]);
-  w->child = make_int4(c[0], c[1], c[2], c[3]);
-  w->pad = make_int4(0, 0, 0, 0);
+  *wnode_chunk(w, kLoX) = make_float4(b[0][0], b[1][0], b[2][0], b[3][0]);
+  *wnode_chunk(w, kHiX) = make_float4(b[0][3], b[1][3], b[2][3], b[3][3]);
+  *wnode_chunk(w, kLoY) = make_float4(b[0][1], b[1][1], b[2][1], b[3][1]);
+  *wnode_chunk(w, kHiY) = make_float4(b[0][4], b[1][4], b[2][4], b[3][4]);
+  *wnode_chunk(w, kLoZ) = make_float4(b[0][2], b[1][2], b[2][2], b[3][2]);
+  *wnode_chunk(w, kHiZ) = make_float4(b[0][5], b[1][5], b[2][5], b[3][5]);
+  *reinterpret_cast<int4*>(wnode_chunk(w, kChild)) = make_int4(c[0], c[1], c[2], c[3]);
+  *wnode_chunk(w, 7) = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 // Refresh the boxes of wide node w from the binary slots it was collapsed from.
 __device__ __forceinline__ void wide_refit_node(const Node* bnodes, const int* wsrc, WNode* wnodes, uint32_t w) {
-  float* lo[3] = {&wnodes[w].lox.x, &wnodes[w].loy.x, &wnodes[w].loz.x};
-  float* hi[3] = {&wnodes[w].hix.x, &wnodes[w].hiy.x, &wnodes[w].hiz.x};
+  float* lo[3] = {wnode_float(wnodes + w, kLoX, 0), wnode_float(wnodes + w, kLoY, 0), wnode_float(wnodes + w, kLoZ, 0)};
+  float* hi[3] = {wnode_float(wnodes + w, kHiX, 0), wnode_float(wnodes + w, kHiY, 0), wnode_float(wnodes + w, kHiZ, 0)};
   for (int i = 0; i < 4; ++i) {
     const int src = wsrc[4 * w + i];
     if (src < 0) continue;
@@ -431,10 +431,12 @@ __device__ __forceinline__ void ref_box(const WNode* wnodes, const Tri* tris, in
     b[3 + k] = -3.0e38f;
   }
   if (r >= 0) {
-    const WNode& n = wnodes[r];
-    const float lx[4] = {n.lox.x, n.lox.y, n.lox.z, n.lox.w}, hx[4] = {n.hix.x, n.hix.y, n.hix.z, n.hix.w};
-    const float ly[4] = {n.loy.x, n.loy.y, n.loy.z, n.loy.w}, hy[4] = {n.hiy.x, n.hiy.y, n.hiy.z, n.hiy.w};
-    const float lz[4] = {n.loz.x, n.loz.y, n.loz.z, n.loz.w}, hz[4] = {n.hiz.x, n.hiz.y, n.hiz.z, n.hiz.w};
+    const float4 X0 = *wnode_chunk(wnodes + r, kLoX), X1 = *wnode_chunk(wnodes + r, kHiX);
+    const float4 Y0 = *wnode_chunk(wnodes + r, kLoY), Y1 = *wnode_chunk(wnodes + r, kHiY);
+    const float4 Z0 = *wnode_chunk(wnodes + r, kLoZ), Z1 = *wnode_chunk(wnodes + r, kHiZ);
+    const float lx[4] = {X0.x, X0.y, X0.z, X0.w}, hx[4] = {X1.x, X1.y, X1.z, X1.w};
+    const float ly[4] = {Y0.x, Y0.y, Y0.z, Y0.w}, hy[4] = {Y1.x, Y1.y, Y1.z, Y1.w};
+    const float lz[4] = {Z0.x, Z0.y, Z0.z, Z0.w}, hz[4] = {Z1.x, Z1.y, Z1.z, Z1.w};
     for (int c = 0; c < 4; ++c) {
       b[0] = fminf(b[0], lx[c]); b[1] = fminf(b[1], ly[c]); b[2] = fminf(b[2], lz[c]);
       b[3] = fmaxf(b[3], hx[c]); b[4] = fmaxf(b[4], hy[c]); b[5] = fmaxf(b[5], hz[c]);
