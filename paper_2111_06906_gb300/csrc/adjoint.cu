@@ -131,219 +131,347 @@ __device__ __forceinline__ Spline spline(const ModelArgs& A, float x, float z) {
   return b;
 }
 
-// Add 12 consecutive floats (one row of four RGB taps) with the widest
-// aligned vector atomics (sm_90+ global float2/float4 atomicAdd).  O = floats
-// by which p lies past a 16-byte boundary; every index is a constant so v
-// stays in registers.
-template <int O>
-__device__ __forceinline__ void add_row12_at(float* p, const float* v) {
-  int i = 0;
-  if (O == 1) {
-    atomicAdd(p, v[0]);
-    atomicAdd(reinterpret_cast<float2*>(p + 1), make_float2(v[1], v[2]));
-    i = 3;
-  } else if (O == 2) {
-    atomicAdd(reinterpret_cast<float2*>(p), make_float2(v[0], v[1]));
-    i = 2;
-  } else if (O == 3) {
-    atomicAdd(p, v[0]);
-    i = 1;
-  }
-#pragma unroll
-  for (int q = 0; q < 3; ++q)
-    if (i + 4 <= 12) {
-      atomicAdd(reinterpret_cast<float4*>(p + i), make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]));
-      i += 4;
-    }
-  if (i + 2 <= 12) {
-    atomicAdd(reinterpret_cast<float2*>(p + i), make_float2(v[i], v[i + 1]));
-    i += 2;
-  }
-  if (i < 12) atomicAdd(p + i, v[i]);
-}
-
-// p must be 4-byte aligned inside a 16-byte aligned array.
-__device__ __forceinline__ void add_row12(float* p, const float* v) {
-  switch ((reinterpret_cast<uintptr_t>(p) >> 2) & 3u) {
-    case 0: add_row12_at<0>(p, v); break;
-    case 1: add_row12_at<1>(p, v); break;
-    case 2: add_row12_at<2>(p, v); break;
-    default: add_row12_at<3>(p, v); break;
-  }
+// Four floats added at p (16-byte aligned), nothing returned.
+__device__ __forceinline__ void add4(float4* p, const float (&v)[4]) {
+  asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+               "f"(v[3])
+               : "memory");
 }
 
 __device__ __forceinline__ void stage_theta(const ModelArgs& A, float* s_th) {
   for (uint32_t j = threadIdx.x; j < A.n_theta; j += blockDim.x) s_th[j] = A.theta[j];
 }
 
-__global__ void __launch_bounds__(256) k_model_deposit(SceneView sv, FrameLights L, ModelArgs A, float* atlas) {
-  __shared__ float s_th[kMaxTheta];
-  const bool vec_ok = (reinterpret_cast<uintptr_t>(atlas) & 15u) == 0;
-  stage_theta(A, s_th);
-  __syncthreads();
-  const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= A.n) return;
-  const uint32_t w = A.info[p];
-  const uint32_t nseg = min(info_nseg(w), sv.B), l = info_light(w);
-  if (nseg == 0) return;
-  float4 v = A.pa[p];
-  const Emission e = model_emission(L.cur[l], s_th + 7 * l, A, p, f3(v));
-  const float sc = s_th[7 * l + 6];
-  float3 prev = e.o, dir = e.d0;
-  for (uint32_t k = 1; k <= nseg; ++k) {
-    int slot;
-    const float3 nu = photon_normal(sv, v, slot);
-    const float3 q = photon_point(A, s_th, v, slot);
-    const float3 x = prev + (dot(nu, q - prev) / dot(nu, dir)) * dir;
-    const float3 E = sc * f3(A.pb[(size_t)(k - 1) * A.n + p]);
-    const Spline b = spline(A, x.x, x.z);
-    const bool row_inside = b.i0 >= 0 && b.i0 + 3 < (int)A.W;
+// Shared memory of one warp of 32 consecutive paths: per photon (row k, lane of
+// its path, arrays [B][32]) two or three words, and the list of the warp's photons.
+//
+// The chain of a path is serial, but what costs is the 4 x 4 texels of each of
+// its photons.  With a thread per path the rounds over photons run until the
+// warp's longest path ends (two of up to seven photons on average), 8 to 11 of
+// 32 lanes active.  So each lane first walks its path's chain and leaves its
+// photons' x and z here, and then the warp's photons are dealt out to the lanes
+// through the list.  (Dealing out their normals as well took 14-24 % longer: six
+// more words a photon leave room for fewer warps.)
+struct PhotonSmem {
+  float* a;                    // x, then the adjoint's dL/dx
+  float* b;                    // z, then the adjoint's dL/dz
+  float* c;                    // the adjoint's dL/d(intensity)
+  uint16_t* list;              // [32 B] lane | row << 5
+};
+
+// A row of four RGB taps is 12 consecutive floats at any multiple of 4 bytes.  It
+// is read and added through the 16-byte chunks that hold it: four of them from
+// the last 16-byte boundary at or before the row, which starts o = 0..3 floats
+// behind (the fourth holds none of it when o = 0); widths chosen by alignment
+// made the lanes take turns.  k_model_deposit gives the chunks to four lanes next
+// to each other, so that a row is one request to L2; a lane per photon made four.
+// Each lane leaves its photon's taps here, then each four lanes take a photon's rows.
+struct TapSmem {
+  float p[32][19];             // energy x wx of the 12 floats from [3] on, zeros around them (odd stride: no conflicts)
+  float wz[32][5];
+  size_t first[32];            // float index of row 0 (wraps below zero for a row outside)
+  uint32_t rows[32];           // bit r: row r goes by chunks
+};
+static_assert(sizeof(TapSmem) % 8 == 0 && 4 * (sizeof(TapSmem) + 32 * PV_MAX_BOUNCES * 10) <= 46 * 1024, "shared memory of a block");
+
+// Bytes a warp needs: ``taps`` of them for its taps, then kWords words a photon and the list.
+template <uint32_t kWords>
+__host__ __device__ __forceinline__ uint32_t warp_smem_bytes(uint32_t B, uint32_t taps) {
+  return taps + ((32u * B * (4u * kWords + 2u) + 7u) & ~7u);
+}
+
+template <uint32_t kWords>
+__device__ __forceinline__ PhotonSmem photon_smem(unsigned char* warp, uint32_t B) {
+  float* f = reinterpret_cast<float*>(warp);
+  return {f, f + 32 * B, f + 64 * B, reinterpret_cast<uint16_t*>(f + 32 * B * kWords)};
+}
+
+// What a path's chain leaves with its lane.
+struct Chain {
+  uint32_t nseg, light;
+  float sc, tau1;
+  Emission e;
+};
+
+// Walk the chain of path p (>= A.n: no path): photon k's model position into
+// row k of the warp's shared memory, and the warp's photons into its list;
+// returns their number.  All lanes call.
+__device__ __forceinline__ uint32_t walk_chain(const SceneView& sv, const FrameLights& L, const ModelArgs& A,
+                                               const float* s_th, uint32_t p, const PhotonSmem& S, Chain& c) {
+  const int lane = threadIdx.x & 31;
+  c.nseg = 0;
+  c.light = 0;
+  c.sc = c.tau1 = 0.f;
+  if (p < A.n) {
+    const uint32_t w = A.info[p];
+    c.nseg = min(info_nseg(w), sv.B);
+    c.light = info_light(w);
+  }
+  uint32_t at = c.nseg;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, at, o);
+    if (lane >= o) at += y;
+  }
+  const uint32_t total = __shfl_sync(0xffffffffu, at, 31);
+  at -= c.nseg;
+  if (c.nseg > 0) {
+    float4 v = A.pa[p];
+    c.e = model_emission(L.cur[c.light], s_th + 7 * c.light, A, p, f3(v));
+    c.sc = s_th[7 * c.light + 6];
+    float3 prev = c.e.o, dir = c.e.d0;
+    for (uint32_t k = 0; k < c.nseg; ++k) {
+      const float4 vn = k + 1 < c.nseg ? A.pa[(size_t)(k + 1) * A.n + p] : v;
+      int slot;
+      const float3 nu = photon_normal(sv, v, slot);
+      const float3 q = photon_point(A, s_th, v, slot);
+      const float tau = dot(nu, q - prev) / dot(nu, dir);
+      if (k == 0) c.tau1 = tau;
+      const float3 x = prev + tau * dir;
+      S.a[32 * k + lane] = x.x;
+      S.b[32 * k + lane] = x.z;
+      S.list[at + k] = (uint16_t)(lane | (k << 5));
+      dir = f3(vn) - f3(v);                       // stored direction of the next segment
+      v = vn;
+      prev = x;
+    }
+  }
+  __syncwarp();
+  return total;
+}
+
+// This lane's photon into the warp's taps; returns the rows that go by chunks
+// (inside the atlas in x, their 16 floats inside the array, which is 16-byte
+// aligned if ``vec_ok``).
+__device__ __forceinline__ uint32_t tap_store(TapSmem& T, int lane, const ModelArgs& A, const Spline& b, float3 E,
+                                              bool vec_ok) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    T.p[lane][3 + 3 * q] = E.x * b.wx[q];
+    T.p[lane][4 + 3 * q] = E.y * b.wx[q];
+    T.p[lane][5 + 3 * q] = E.z * b.wx[q];
+    T.wz[lane][q] = b.wz[q];
+  }
+  const size_t floats = 3 * (size_t)A.W * A.H;
+  const size_t first = 3 * ((size_t)(int64_t)b.j0 * A.W + (size_t)(int64_t)b.i0);
+  T.first[lane] = first;
+  uint32_t rows = 0;
+  if (vec_ok && b.i0 >= 0 && b.i0 + 3 < (int)A.W)
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
       const int tj = b.j0 + r;
-      if (tj < 0 || tj >= (int)A.H) continue;
-      if (row_inside && vec_ok) {
-        float rv[12];
+      if (tj >= 0 && tj < (int)A.H && first + 3 * (size_t)A.W * r + 16 <= floats) rows |= 1u << r;
+    }
+  return T.rows[lane] = rows;
+}
+
+// Forward splat.  Bound by the atomics' requests in L2.  City, 2.0M photons into
+// 1024 x 1024 texels: 249 us with a thread per path and access widths by
+// alignment, 217 us with the photons dealt out a lane each, 141 us with four lanes
+// a photon (16 lanes: 142 us, a quarter more instructions).
+__global__ void __launch_bounds__(128) k_model_deposit(SceneView sv, FrameLights L, ModelArgs A, float* atlas) {
+  __shared__ float s_th[kMaxTheta];
+  extern __shared__ __align__(16) unsigned char s_photons[];
+  stage_theta(A, s_th);
+  __syncthreads();
+  const bool vec_ok = (reinterpret_cast<uintptr_t>(atlas) & 15u) == 0;
+  unsigned char* const mine = s_photons + (threadIdx.x >> 5) * warp_smem_bytes<2>(sv.B, sizeof(TapSmem));
+  TapSmem& T = *reinterpret_cast<TapSmem*>(mine);
+  const PhotonSmem S = photon_smem<2>(mine + sizeof(TapSmem), sv.B);
+  const int lane = threadIdx.x & 31;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const float wc = b.wx[c] * b.wz[r];
-          rv[3 * c] = E.x * wc;
-          rv[3 * c + 1] = E.y * wc;
-          rv[3 * c + 2] = E.z * wc;
+  for (int i = 0; i < 19; ++i)
+    if (i < 3 || i > 14) T.p[lane][i] = 0.f;
+  const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x, p0 = p - lane;
+  Chain c;
+  const uint32_t total = walk_chain(sv, L, A, s_th, p, S, c);
+  const size_t stride = 3 * (size_t)A.W;
+  for (uint32_t t0 = 0; t0 < total; t0 += 32) {
+    const bool has = t0 + lane < total;
+    const uint32_t id = S.list[has ? t0 + lane : t0], own = id & 31u, k = id >> 5;
+    const float sc = __shfl_sync(0xffffffffu, c.sc, own);
+    if (has) {
+      const float3 E = sc * f3(A.pb[(size_t)k * A.n + p0 + own]);
+      const Spline b = spline(A, S.a[32 * k + own], S.b[32 * k + own]);
+      const uint32_t rows = tap_store(T, lane, A, b, E, vec_ok);
+      if (rows != 15u)                            // at the atlas' edges, or an unaligned atlas: texel by texel
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const int tj = b.j0 + r;
+          if (((rows >> r) & 1u) || tj < 0 || tj >= (int)A.H) continue;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int ti = b.i0 + q;
+            if (ti < 0 || ti >= (int)A.W) continue;
+            float* t = atlas + 3 * ((size_t)tj * A.W + ti);
+            const float wc = b.wx[q] * b.wz[r];
+            atomicAdd(t + 0, E.x * wc);
+            atomicAdd(t + 1, E.y * wc);
+            atomicAdd(t + 2, E.z * wc);
+          }
         }
-        add_row12(atlas + 3 * ((size_t)tj * A.W + b.i0), rv);
-        continue;
-      }
+    }
+    __syncwarp();
+    const uint32_t n = min(32u, total - t0);
+    const int q = lane & 3;
+    for (uint32_t j = lane >> 2; j < n; j += 8) {
+      const uint32_t rows = T.rows[j];
+      size_t first = T.first[j];
+      uint32_t o = (uint32_t)first & 3u;
+      const float* w = &T.p[j][3 + 4 * q - (int)o];
+      float v[4] = {w[0], w[1], w[2], w[3]};
 #pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int ti = b.i0 + c;
-        if (ti < 0 || ti >= (int)A.W) continue;
-        float* t = atlas + 3 * ((size_t)tj * A.W + ti);
-        const float wc = b.wx[c] * b.wz[r];
-        atomicAdd(t + 0, E.x * wc);
-        atomicAdd(t + 1, E.y * wc);
-        atomicAdd(t + 2, E.z * wc);
+      for (int r = 0; r < 4; ++r, first += stride) {
+        if (r > 0 && (A.W & 3u)) {                // rows of another alignment
+          o = (uint32_t)first & 3u;
+          w = &T.p[j][3 + 4 * q - (int)o];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) v[i] = w[i];
+        }
+        if (!((rows >> r) & 1u) || (q == 3 && o == 0u)) continue;
+        const float wz = T.wz[j][r];
+        const float u[4] = {v[0] * wz, v[1] * wz, v[2] * wz, v[3] * wz};
+        add4(reinterpret_cast<float4*>(atlas + (first - o)) + q, u);
       }
     }
-    if (k < nseg) {
-      const float4 vn = A.pa[(size_t)k * A.n + p];
-      dir = f3(vn) - f3(v);                     // stored direction of the next segment
-      v = vn;
-    }
-    prev = x;
+    __syncwarp();
   }
 }
 
-// Reverse mode, one path per thread: the forward pass keeps the splat
-// gradient of each photon position (only x and z are nonzero); the backward
-// pass reloads the planes and directions.  dtheta is reduced per block in
-// shared memory, then added to the global vector.
+// w[o .. o + 11] into v, o = 0..3.
+__device__ __forceinline__ void shift_down(const float (&w)[16], uint32_t o, float (&v)[12]) {
+  const bool s1 = o & 1u, s2 = o & 2u;
+  float t[13];
+#pragma unroll
+  for (int i = 0; i < 13; ++i) t[i] = s2 ? w[i + 2] : w[i];
+#pragma unroll
+  for (int i = 0; i < 12; ++i) v[i] = s1 ? t[i + 1] : t[i];
+}
+
+// Reverse mode: the chain forward, the splat gradient of every photon (only x
+// and z are nonzero) and its share of the intensity's, dealt out over the warp,
+// then the chain backward, which reloads the planes and directions.  dtheta is
+// reduced per block in shared memory, then added to the global vector.
+// Bound by L1's wavefronts (65 %) and the chains' loads.  City, 2.0M photons:
+// 258 us with a thread per path and 48 scalar reads of the gradient a photon,
+// 172 us with the photons dealt out a lane each and four wide reads a row.  (Four
+// lanes a photon, one request a row, 228 us and 16 lanes 316 us: what they save in
+// L1 they spend on summing up and on shared memory.)
 __global__ void __launch_bounds__(128) k_adjoint(SceneView sv, FrameLights L, ModelArgs A, const float* G,
                                                  float* dtheta, float* score) {
   __shared__ float s_th[kMaxTheta];
   __shared__ float s_acc[kMaxTheta];
+  extern __shared__ __align__(16) unsigned char s_photons[];
   stage_theta(A, s_th);
   for (uint32_t j = threadIdx.x; j < A.n_theta; j += blockDim.x) s_acc[j] = 0.f;
   __syncthreads();
-  const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
-  float lc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};   // this path's light gradient
-  int my_l = -1;
-  if (p < A.n) {
-    const uint32_t w = A.info[p];
-    const uint32_t nseg = min(info_nseg(w), sv.B), l = info_light(w);
-    float sgE = 0.f;
-    if (nseg > 0) {
-      my_l = (int)l;
-      float2 gpos[PV_MAX_BOUNCES + 1];
-      const float4 v1 = A.pa[p];
-      const Emission e = model_emission(L.cur[l], s_th + 7 * l, A, p, f3(v1));
-      const float sc = s_th[7 * l + 6];
-      float3 prev = e.o, dir = e.d0;
-      float4 v = v1;
-      float gscale = 0.f, tau1 = 0.f;
-      for (uint32_t k = 1; k <= nseg; ++k) {
-        int slot;
-        const float3 nu = photon_normal(sv, v, slot);
-        const float3 q = photon_point(A, s_th, v, slot);
-        const float tau = dot(nu, q - prev) / dot(nu, dir);
-        if (k == 1) tau1 = tau;
-        const float3 x = prev + tau * dir;
-        const float3 E0 = f3(A.pb[(size_t)(k - 1) * A.n + p]);
-        const Spline b = spline(A, x.x, x.z);
-        float2 g = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const int tj = b.j0 + r;
-          if (tj < 0 || tj >= (int)A.H) continue;
-          float gr = 0.f, gdx = 0.f, gdz = 0.f;       // row sums of ge weighted by wx, dx
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const int ti = b.i0 + c;
-            if (ti < 0 || ti >= (int)A.W) continue;
-            const float* gg = G + 3 * ((size_t)tj * A.W + ti);
-            const float ge = __ldg(gg) * E0.x + __ldg(gg + 1) * E0.y + __ldg(gg + 2) * E0.z;
-            gr = fmaf(ge, b.wx[c], gr);
-            gdx = fmaf(ge, b.dx[c], gdx);
-          }
-          gdz = gr * b.dz[r];
-          g.x = fmaf(gdx, b.wz[r], g.x);
-          g.y += gdz;
-          gscale = fmaf(gr, b.wz[r], gscale);
-        }
-        g.x *= sc * b.sx;
-        g.y *= sc * b.sz;
-        gpos[k] = g;
-        if (k < nseg) {
-          const float4 vn = A.pa[(size_t)k * A.n + p];
-          dir = f3(vn) - f3(v);
-          v = vn;
-        }
-        prev = x;
-      }
-      sgE = sc * gscale;
-      lc[6] = gscale;
-      float3 g = make_float3(0.f, 0.f, 0.f);
-      for (uint32_t k = nseg; k >= 1; --k) {
-        g.x += gpos[k].x;
-        g.z += gpos[k].y;
-        const float4 vk = A.pa[(size_t)(k - 1) * A.n + p];
-        int slot;
-        const float3 nu = photon_normal(sv, vk, slot);
-        const float3 d = k == 1 ? e.d0 : f3(vk) - f3(A.pa[(size_t)(k - 2) * A.n + p]);
-        const float r = dot(d, g) / dot(nu, d);
-        if (slot >= 0) {
-          float* a = s_acc + 7 * A.n_lights + 3 * slot;
-          atomicAdd(a + 0, nu.x * r);
-          atomicAdd(a + 1, nu.y * r);
-          atomicAdd(a + 2, nu.z * r);
-        }
-        g = g - r * nu;
-      }
-      // light: g is now the gradient with respect to o; d0 receives tau_1 g
-      lc[0] = g.x;
-      lc[1] = g.y;
-      lc[2] = g.z;
-      if (e.rect) {
-        const float3 gd = tau1 * g;
-        const float3 gn = e.beta * cross(e.t, g) + e.ell.y * cross(e.t, gd) + e.ell.z * gd;
-        lc[3] = gn.x;
-        lc[4] = gn.y;
-        lc[5] = gn.z;
-      }
-    }
-    if (score) score[p] = fabsf(sgE);
-  }
-  // light entries: summed over the warp per light, one shared atomic per entry
+  const bool vec_ok = (reinterpret_cast<uintptr_t>(G) & 15u) == 0;
+  const size_t floats = 3 * (size_t)A.W * A.H;
+  const PhotonSmem S = photon_smem<3>(s_photons + (threadIdx.x >> 5) * warp_smem_bytes<3>(sv.B, 0), sv.B);
   const int lane = threadIdx.x & 31;
+  const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x, p0 = p - lane;
+  float lc[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};   // this path's light gradient
+  Chain c;
+  const uint32_t total = walk_chain(sv, L, A, s_th, p, S, c);
+  for (uint32_t t0 = 0; t0 < total; t0 += 32) {
+    const bool has = t0 + lane < total;
+    const uint32_t id = S.list[has ? t0 + lane : t0], own = id & 31u, k = id >> 5;
+    const float sc = __shfl_sync(0xffffffffu, c.sc, own);
+    if (!has) continue;
+    const float3 E0 = f3(A.pb[(size_t)k * A.n + p0 + own]);
+    const Spline b = spline(A, S.a[32 * k + own], S.b[32 * k + own]);
+    const bool inside = vec_ok && b.i0 >= 0 && b.i0 + 3 < (int)A.W;
+    float2 g = make_float2(0.f, 0.f);
+    float gscale = 0.f;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int tj = b.j0 + r;
+      if (tj < 0 || tj >= (int)A.H) continue;
+      float v[12];
+      const size_t first = 3 * ((size_t)tj * A.W + (size_t)(int64_t)b.i0);
+      if (inside && first + 16 <= floats) {
+        const uint32_t o = (uint32_t)first & 3u;
+        const float4* at = reinterpret_cast<const float4*>(G + (first - o));
+        float w[16];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float4 x = q < 3 || o ? __ldg(at + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+          w[4 * q] = x.x;
+          w[4 * q + 1] = x.y;
+          w[4 * q + 2] = x.z;
+          w[4 * q + 3] = x.w;
+        }
+        shift_down(w, o, v);
+      } else {
+#pragma unroll
+        for (int q = 0; q < 12; ++q) {
+          const int ti = b.i0 + q / 3;
+          v[q] = ti >= 0 && ti < (int)A.W ? __ldg(G + 3 * ((size_t)tj * A.W + ti) + q % 3) : 0.f;
+        }
+      }
+      float gr = 0.f, gdx = 0.f;                  // row sums of ge weighted by wx, dx
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float ge = v[3 * q] * E0.x + v[3 * q + 1] * E0.y + v[3 * q + 2] * E0.z;
+        gr = fmaf(ge, b.wx[q], gr);
+        gdx = fmaf(ge, b.dx[q], gdx);
+      }
+      g.x = fmaf(gdx, b.wz[r], g.x);
+      g.y += gr * b.dz[r];
+      gscale = fmaf(gr, b.wz[r], gscale);
+    }
+    S.a[32 * k + own] = g.x * (sc * b.sx);
+    S.b[32 * k + own] = g.y * (sc * b.sz);
+    S.c[32 * k + own] = gscale;
+  }
+  __syncwarp();
+  if (c.nseg > 0) {
+    const Emission& e = c.e;
+    float gscale = 0.f;
+    float3 g = make_float3(0.f, 0.f, 0.f);
+    float4 vk = A.pa[(size_t)(c.nseg - 1) * A.n + p];
+    for (uint32_t k = c.nseg; k >= 1; --k) {
+      g.x += S.a[32 * (k - 1) + lane];
+      g.z += S.b[32 * (k - 1) + lane];
+      gscale += S.c[32 * (k - 1) + lane];
+      const float4 vp = k == 1 ? vk : A.pa[(size_t)(k - 2) * A.n + p];
+      int slot;
+      const float3 nu = photon_normal(sv, vk, slot);
+      const float3 d = k == 1 ? e.d0 : f3(vk) - f3(vp);
+      const float r = dot(d, g) / dot(nu, d);
+      if (slot >= 0) {
+        float* a = s_acc + 7 * A.n_lights + 3 * slot;
+        atomicAdd(a + 0, nu.x * r);
+        atomicAdd(a + 1, nu.y * r);
+        atomicAdd(a + 2, nu.z * r);
+      }
+      g = g - r * nu;
+      vk = vp;
+    }
+    // light: g is now the gradient with respect to o; d0 receives tau_1 g
+    lc[0] = g.x;
+    lc[1] = g.y;
+    lc[2] = g.z;
+    lc[6] = gscale;
+    if (e.rect) {
+      const float3 gd = c.tau1 * g;
+      const float3 gn = e.beta * cross(e.t, g) + e.ell.y * cross(e.t, gd) + e.ell.z * gd;
+      lc[3] = gn.x;
+      lc[4] = gn.y;
+      lc[5] = gn.z;
+    }
+  }
+  if (score && p < A.n) score[p] = fabsf(c.sc * lc[6]);
+  // light entries: summed over the warp per light, one shared atomic per entry
   for (uint32_t ll = 0; ll < A.n_lights; ++ll) {
-    const bool mine = my_l == (int)ll;
+    const bool mine = c.nseg > 0 && c.light == ll;
     if (!__any_sync(0xffffffffu, mine)) continue;
 #pragma unroll
-    for (int c = 0; c < 7; ++c) {
-      float v = mine ? lc[c] : 0.f;
+    for (int q = 0; q < 7; ++q) {
+      float v = mine ? lc[q] : 0.f;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0 && v != 0.f) atomicAdd(&s_acc[7 * ll + c], v);
+      if (lane == 0 && v != 0.f) atomicAdd(&s_acc[7 * ll + q], v);
     }
   }
   __syncthreads();
@@ -569,8 +697,12 @@ extern "C" int pv_model_deposit(pv_scene* s, const pv_paths* paths, const float*
   if ((rc = model_args(s, paths, d_theta, width, height, rect, A)) != PV_OK) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   s->last_stream = st;
+  // 128 threads a block at most 40 KB of shared memory (15 photons a path)
+  constexpr uint32_t kThreads = 128;
   if (paths->n)
-    k_model_deposit<<<(paths->n + 255) / 256, 256, 0, st>>>(pvh::view(s), pvh::frame_lights(s), A, d_atlas);
+    k_model_deposit<<<(paths->n + kThreads - 1) / kThreads, kThreads,
+                      kThreads / 32 * warp_smem_bytes<2>(s->B, sizeof(TapSmem)), st>>>(pvh::view(s), pvh::frame_lights(s), A,
+                                                                                     d_atlas);
   return pvh::cuda_status(cudaGetLastError());
 }
 
@@ -584,9 +716,10 @@ extern "C" int pv_adjoint_deposit(pv_scene* s, const pv_paths* paths, const floa
   if ((rc = model_args(s, paths, d_theta, width, height, rect, A)) != PV_OK) return rc;
   cudaStream_t st = (cudaStream_t)stream;
   s->last_stream = st;
+  constexpr uint32_t kThreads = 128;
   if (paths->n)
-    k_adjoint<<<(paths->n + 127) / 128, 128, 0, st>>>(pvh::view(s), pvh::frame_lights(s), A, d_grad_atlas, d_dtheta,
-                                                      d_score);
+    k_adjoint<<<(paths->n + kThreads - 1) / kThreads, kThreads, kThreads / 32 * warp_smem_bytes<3>(s->B, 0), st>>>(
+        pvh::view(s), pvh::frame_lights(s), A, d_grad_atlas, d_dtheta, d_score);
   return pvh::cuda_status(cudaGetLastError());
 }
 
