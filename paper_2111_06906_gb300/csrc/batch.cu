@@ -341,13 +341,14 @@ __global__ void __launch_bounds__(128) k_b_continue(const BScene* B, const BFram
   __syncthreads();
   const uint32_t total = s_pre[n_scenes];
   const int lane = threadIdx.x & 31;
+  const uint32_t lanes = lanes_at_work(total, gridDim.x * (blockDim.x / 32u));
   for (uint32_t guard = 0; guard < kGuard; ++guard) {
     uint32_t base = 0;
-    if (lane == 0) base = atomicAdd(&bc->cont, 32u);
+    if (lane == 0) base = atomicAdd(&bc->cont, lanes);
     base = __shfl_sync(0xffffffffu, base, 0);
     if (base >= total) break;
     const uint32_t i = base + lane;
-    if (i < total) {
+    if (i < total && (uint32_t)lane < lanes) {
       const uint32_t sc = scene_of(s_pre, n_scenes, i);
       const ContArgs& A = s_C[sc];
       ContCounters cc;
@@ -428,7 +429,8 @@ __global__ void __launch_bounds__(pvh::kTraceThreads, PV_BATCH_TRACE_MIN_BLOCKS)
   Trav t;
   TStack<S> stk;
   uint32_t sc = 0, c_rays = 0, c_photons = 0;
-  bool has_ray = false, exhausted = false;
+  bool has_ray = false;
+  bool exhausted = (uint32_t)lane >= lanes_at_work(total, gridDim.x * (pvh::kTraceThreads / 32));
   auto flush = [&]() {                         // the finished path's counters to its scene
     if (c_rays) atomicAdd(s_cnt + 4 * sc + 0, c_rays);
     if (c_photons) atomicAdd(s_cnt + 4 * sc + 1, c_photons);
@@ -445,6 +447,7 @@ __global__ void __launch_bounds__(pvh::kTraceThreads, PV_BATCH_TRACE_MIN_BLOCKS)
       uint32_t base = 0;
       if (lane == leader) base = atomicAdd(&bc->trace, (uint32_t)__popc(nm));
       base = __shfl_sync(0xffffffffu, base, leader);
+      if (base >= total) exhausted = true;       // nothing left for any lane
       if (need) {
         const uint32_t idx = base + __popc(nm & lt);
         if (idx < total) {
@@ -558,7 +561,8 @@ __global__ void __launch_bounds__(pvh::kTraceThreads, PV_BATCH_CT_MIN_BLOCKS) k_
   Trav t;
   TStack<S> stk;
   uint32_t sc = 0, c_rays = 0, c_photons = 0, cmask = 0, cmeta = 0;
-  bool has_ray = false, exhausted = false, cont = false;
+  bool has_ray = false, cont = false;
+  bool exhausted = (uint32_t)lane >= lanes_at_work(total, gridDim.x * (pvh::kTraceThreads / 32));
   auto flush = [&]() {                         // the finished path's counters to its scene
     uint32_t* c = s_cnt + 6 * sc;
     if (c_rays) atomicAdd(c + 0, c_rays);
@@ -583,6 +587,7 @@ __global__ void __launch_bounds__(pvh::kTraceThreads, PV_BATCH_CT_MIN_BLOCKS) k_
       uint32_t base = 0;
       if (lane == leader) base = atomicAdd(&bc->trace, (uint32_t)__popc(nm));
       base = __shfl_sync(0xffffffffu, base, leader);
+      if (base >= total) exhausted = true;       // nothing left for any lane
       if (need) {
         const uint32_t idx = base + __popc(nm & lt);
         if (idx < n_cont) {

@@ -9,6 +9,7 @@
 // many steps.  Rays are generated where the paper generates them (Sec. 4):
 // from the light (start 0), or by Russian roulette and a cosine-weighted
 // bounce at the first photon to re-trace.
+#include <algorithm>
 #include <cstdlib>
 #include <cstring>
 
@@ -112,7 +113,8 @@ __global__ void __launch_bounds__(pvh::kTraceThreads, kDep ? PV_TRACE_DEP_MIN_BL
   __shared__ int s_stk[kStackSharedWords];
   TraceStack stk;
   stk.sh = s_stk + threadIdx.x;
-  bool has_ray = false, exhausted = false;
+  bool has_ray = false;
+  bool exhausted = (uint32_t)lane >= lanes_at_work(total, gridDim.x * (pvh::kTraceThreads / 32));
   uint32_t c_rays = 0, c_photons = 0;
   for (uint32_t guard = 0; guard < (1u << 30); ++guard) {
     const bool need = !has_ray && !exhausted;
@@ -122,6 +124,7 @@ __global__ void __launch_bounds__(pvh::kTraceThreads, kDep ? PV_TRACE_DEP_MIN_BL
       uint32_t base = 0;
       if (lane == leader) base = atomicAdd(A.ticket, (uint32_t)__popc(nm));
       base = __shfl_sync(0xffffffffu, base, leader);
+      if (base >= total) exhausted = true;       // nothing left for any lane
       if (need) {
         const uint32_t idx = base + __popc(nm & lt);
         if (idx < total) {
@@ -219,6 +222,8 @@ __global__ void __launch_bounds__(pvh::kTraceThreads, PV_CONT_TRACE_MIN_BLOCKS)
   stk.sh = s_stk + threadIdx.x;
   uint32_t cmask = 0, cmeta = 0;             // Alg. 1 state beyond s.k (segment), s.E (a_orig), s.excl (a_prim)
   bool has_ray = false, exhausted = false, cont = false;
+  // while there are rays to trace, a short list is spread over the warps; the deposits left over go to every lane
+  bool waits = (uint32_t)lane >= lanes_at_work(n_trace, gridDim.x * (pvh::kTraceThreads / 32));
   uint32_t c_rays = 0, c_photons = 0;
   for (uint32_t guard = 0; guard < (1u << 30); ++guard) {
     if (PV_DEP_WARP && kDeposit && __any_sync(0xffffffffu, dep != 0xFFFFFFFFu)) {
@@ -229,13 +234,15 @@ __global__ void __launch_bounds__(pvh::kTraceThreads, PV_CONT_TRACE_MIN_BLOCKS)
       deposit_path(atlas_map(D.at), A.n, sv.B, A.info, A.pa, A.pb, dep);   // scales per path: no registers held
       dep = 0xFFFFFFFFu;
     }
-    const bool need = !has_ray && !exhausted;
+    const bool need = !has_ray && !exhausted && !waits;
     const unsigned nm = __ballot_sync(0xffffffffu, need);
     if (nm) {
       const int leader = __ffs(nm) - 1;
       uint32_t base = 0;
       if (lane == leader) base = atomicAdd(A.ticket, (uint32_t)__popc(nm));
       base = __shfl_sync(0xffffffffu, base, leader);
+      if (base >= n_trace) waits = false;
+      if (base >= total) exhausted = true;       // nothing left for any lane
       if (need) {
         const uint32_t idx = base + __popc(nm & lt);
         if (idx < n_cont) {
@@ -265,7 +272,7 @@ __global__ void __launch_bounds__(pvh::kTraceThreads, PV_CONT_TRACE_MIN_BLOCKS)
         }
       }
     }
-    if (__all_sync(0xffffffffu, exhausted && !has_ray && dep == 0xFFFFFFFFu)) break;
+    if (__all_sync(0xffffffffu, (exhausted || waits) && !has_ray && dep == 0xFFFFFFFFu)) break;
     if (kDoneLanes > 32 && !has_ray) continue;
     const bool done = step_rays(sv, r, t, stk, s.excl, wk, !has_ray);
     if (!has_ray || !done) continue;
@@ -330,6 +337,11 @@ int persistent_blocks(const pv_scene* s, K kernel) {
   return (per > 0 ? per : 1) * s->num_sms;
 }
 
+// Blocks for n paths: the resident ones, or enough for 32 paths each.  Every warp
+// takes tickets from one counter: with 1064 blocks for the 10 000 paths of a room
+// that cost a quarter of the kernel (37 -> 27 us, with the lanes spread as well).
+int blocks_for(int resident, uint32_t n) { return (int)std::min<uint32_t>((uint32_t)resident, (n + 31u) / 32u); }
+
 TraceArgs trace_args(pv_scene* s, const pv_paths* p, const uint32_t* list, const uint32_t* count, uint64_t seed,
                      uint32_t frame, pv_frame_stats* stats) {
   TraceArgs A;
@@ -362,10 +374,10 @@ void launch_trace(pv_scene* s, const pv_paths* p, const uint32_t* list, const ui
     am.sx = (float)atlas->width / (atlas->x1 - atlas->x0);
     am.sz = (float)atlas->height / (atlas->z1 - atlas->z0);
     if (!s->trace_dep_blocks) s->trace_dep_blocks = persistent_blocks(s, k_trace<true>);
-    k_trace<true><<<s->trace_dep_blocks, kTraceThreads, 0, st>>>(view(s), frame_lights(s), A, am);
+    k_trace<true><<<blocks_for(s->trace_dep_blocks, p->n), kTraceThreads, 0, st>>>(view(s), frame_lights(s), A, am);
   } else {
     if (!s->trace_blocks) s->trace_blocks = persistent_blocks(s, k_trace<false>);
-    k_trace<false><<<s->trace_blocks, kTraceThreads, 0, st>>>(view(s), frame_lights(s), A, am);
+    k_trace<false><<<blocks_for(s->trace_blocks, p->n), kTraceThreads, 0, st>>>(view(s), frame_lights(s), A, am);
   }
 }
 
@@ -407,14 +419,14 @@ void launch_cont_trace(pv_scene* s, const pv_paths* p, const ContArgs& C, const 
     D.touched = touched;
     if (delta) {
       if (!s->cont_trace_delta_blocks) s->cont_trace_delta_blocks = persistent_blocks(s, k_cont_trace<2>);
-      launch_cont_trace_pdl<2>(s->cont_trace_delta_blocks, view(s), frame_lights(s), A, C, D, st);
+      launch_cont_trace_pdl<2>(blocks_for(s->cont_trace_delta_blocks, p->n), view(s), frame_lights(s), A, C, D, st);
     } else {
       if (!s->cont_trace_dep_blocks) s->cont_trace_dep_blocks = persistent_blocks(s, k_cont_trace<1>);
-      launch_cont_trace_pdl<1>(s->cont_trace_dep_blocks, view(s), frame_lights(s), A, C, D, st);
+      launch_cont_trace_pdl<1>(blocks_for(s->cont_trace_dep_blocks, p->n), view(s), frame_lights(s), A, C, D, st);
     }
   } else {
     if (!s->cont_trace_blocks) s->cont_trace_blocks = persistent_blocks(s, k_cont_trace<0>);
-    launch_cont_trace_pdl<0>(s->cont_trace_blocks, view(s), frame_lights(s), A, C, D, st);
+    launch_cont_trace_pdl<0>(blocks_for(s->cont_trace_blocks, p->n), view(s), frame_lights(s), A, C, D, st);
   }
 }
 

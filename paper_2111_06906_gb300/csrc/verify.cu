@@ -100,13 +100,14 @@ __global__ void __launch_bounds__(128, 6) k_continue(SceneView sv, ContArgs A) {
   const int lane = threadIdx.x & 31;
   ContCounters cc;
   Work wk;
+  const uint32_t lanes = lanes_at_work(total, gridDim.x * (blockDim.x / 32u));
   for (uint32_t guard = 0; guard < (1u << 26); ++guard) {
     uint32_t base = 0;
-    if (lane == 0) base = atomicAdd(A.ticket, 32u);
+    if (lane == 0) base = atomicAdd(A.ticket, lanes);
     base = __shfl_sync(0xffffffffu, base, 0);
     if (base >= total) break;
     const uint32_t i = base + lane;
-    if (i < total) continue_path(sv, root, A, A.list[i], cc, wk);
+    if (i < total && (uint32_t)lane < lanes) continue_path(sv, root, A, A.list[i], cc, wk);
     __syncwarp();
   }
   uint32_t* const ctr[4] = {A.stats ? &A.stats->cont_rays : nullptr, A.stats ? &A.stats->n_tail : nullptr,
