@@ -341,14 +341,13 @@ __global__ void __launch_bounds__(128) k_b_continue(const BScene* B, const BFram
   __syncthreads();
   const uint32_t total = s_pre[n_scenes];
   const int lane = threadIdx.x & 31;
-  const uint32_t lanes = lanes_at_work(total, gridDim.x * (blockDim.x / 32u));
   for (uint32_t guard = 0; guard < kGuard; ++guard) {
     uint32_t base = 0;
-    if (lane == 0) base = atomicAdd(&bc->cont, lanes);
+    if (lane == 0) base = atomicAdd(&bc->cont, 32u);
     base = __shfl_sync(0xffffffffu, base, 0);
     if (base >= total) break;
     const uint32_t i = base + lane;
-    if (i < total && (uint32_t)lane < lanes) {
+    if (i < total) {
       const uint32_t sc = scene_of(s_pre, n_scenes, i);
       const ContArgs& A = s_C[sc];
       ContCounters cc;
@@ -429,8 +428,7 @@ __global__ void __launch_bounds__(pvh::kTraceThreads, PV_BATCH_TRACE_MIN_BLOCKS)
   Trav t;
   TStack<S> stk;
   uint32_t sc = 0, c_rays = 0, c_photons = 0;
-  bool has_ray = false;
-  bool exhausted = (uint32_t)lane >= lanes_at_work(total, gridDim.x * (pvh::kTraceThreads / 32));
+  bool has_ray = false, exhausted = false;
   auto flush = [&]() {                         // the finished path's counters to its scene
     if (c_rays) atomicAdd(s_cnt + 4 * sc + 0, c_rays);
     if (c_photons) atomicAdd(s_cnt + 4 * sc + 1, c_photons);
@@ -561,8 +559,9 @@ __global__ void __launch_bounds__(pvh::kTraceThreads, PV_BATCH_CT_MIN_BLOCKS) k_
   Trav t;
   TStack<S> stk;
   uint32_t sc = 0, c_rays = 0, c_photons = 0, cmask = 0, cmeta = 0;
-  bool has_ray = false, cont = false;
-  bool exhausted = (uint32_t)lane >= lanes_at_work(total, gridDim.x * (pvh::kTraceThreads / 32));
+  // All lanes take items also when there are fewer than lanes: spread over the warps, a small batch by itself
+  // is 8 % faster, but batches that overlap on their streams get 10 % less done together.
+  bool has_ray = false, exhausted = false, cont = false;
   auto flush = [&]() {                         // the finished path's counters to its scene
     uint32_t* c = s_cnt + 6 * sc;
     if (c_rays) atomicAdd(c + 0, c_rays);
