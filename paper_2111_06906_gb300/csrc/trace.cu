@@ -61,16 +61,7 @@ namespace {
 #ifndef PV_TRACE_DONE_LANES
 #define PV_TRACE_DONE_LANES 32
 #endif
-// Traversal stack entries kept in shared memory (the rest in local memory).
-// Measured on the city and villa workloads, 8, 16 or 32 shared entries made
-// the re-trace and trace-all kernels 5-7 % slower than a local-memory stack,
-// so the default keeps none.
-#ifndef PV_TRACE_STACK_SHARED
-#define PV_TRACE_STACK_SHARED 0
-#endif
-constexpr int kStackShared = PV_TRACE_STACK_SHARED < kStack ? PV_TRACE_STACK_SHARED : kStack;
-using TraceStack = TStack<kStack, kStackShared, pvh::kTraceThreads>;
-constexpr int kStackSharedWords = kStackShared > 0 ? kStackShared * pvh::kTraceThreads : 1;
+using TraceStack = TStack<kStack>;
 constexpr int kStepsPerIter = PV_TRACE_STEPS;
 constexpr int kMaxSteps = PV_TRACE_MAX_STEPS;
 constexpr int kDoneLanes = PV_TRACE_DONE_LANES;
@@ -110,9 +101,7 @@ __global__ void __launch_bounds__(pvh::kTraceThreads, kDep ? PV_TRACE_DEP_MIN_BL
   PathState s;
   Ray r;
   Trav t;
-  __shared__ int s_stk[kStackSharedWords];
   TraceStack stk;
-  stk.sh = s_stk + threadIdx.x;
   bool has_ray = false;
   bool exhausted = (uint32_t)lane >= lanes_at_work(total, gridDim.x * (pvh::kTraceThreads / 32));
   uint32_t c_rays = 0, c_photons = 0;
@@ -217,9 +206,7 @@ __global__ void __launch_bounds__(pvh::kTraceThreads, PV_CONT_TRACE_MIN_BLOCKS)
   PathState s;
   Ray r;
   Trav t;
-  __shared__ int s_stk[kStackSharedWords];
   TraceStack stk;
-  stk.sh = s_stk + threadIdx.x;
   uint32_t cmask = 0, cmeta = 0;             // Alg. 1 state beyond s.k (segment), s.E (a_orig), s.excl (a_prim)
   bool has_ray = false, exhausted = false, cont = false;
   // while there are rays to trace, a short list is spread over the warps; the deposits left over go to every lane
