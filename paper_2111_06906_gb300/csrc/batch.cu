@@ -466,6 +466,7 @@ __global__ void __launch_bounds__(pvh::kTraceThreads, PV_BATCH_TRACE_MIN_BLOCKS)
     const TraceArgs& A = s_T[sc];
     const bool done = step_warp<kSteps, S>(sv, r, t, stk, st.excl, wk, !has_ray);
     if (!has_ray || !done) continue;
+    trav_end(t, wk);
     ++c_rays;
     if (trace_hit(sv, A, st, r, t, c_photons)) {
       trav_begin(t, s_root[sc]);
@@ -622,6 +623,7 @@ __global__ void __launch_bounds__(pvh::kTraceThreads, PV_BATCH_CT_MIN_BLOCKS) k_
     const SceneView& sv = s_sv[sc];
     const bool done = step_warp<kSteps, S>(sv, r, t, stk, st.excl, wk, !has_ray);
     if (!has_ray || !done) continue;
+    trav_end(t, wk);
     if (cont) {
       const ContArgs& C = s_C[sc];
       ContCounters cc;

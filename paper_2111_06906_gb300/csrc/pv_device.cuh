@@ -305,26 +305,42 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
   return d;
 }
 
+// x = fma(a, m, c), y = fma(b, m, c) in one instruction (sm_100 and later), each
+// rounded as fmaf rounds it.
+__device__ __forceinline__ void fma2(float a, float b, float m, float c, float& x, float& y) {
+  unsigned long long A, M, Cc, R;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(A) : "f"(a), "f"(b));
+  asm("mov.b64 %0, {%1, %1};" : "=l"(M) : "f"(m));
+  asm("mov.b64 %0, {%1, %1};" : "=l"(Cc) : "f"(c));
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(R) : "l"(A), "l"(M), "l"(Cc));
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(R));
+}
+
 // The four child boxes of a wide node against the ray within [tmin, tmax]:
-// entry distances, hit mask (bit c = child c).  For a box with lo <= hi the
-// near plane's distance is exactly the smaller of the two slab distances
-// (fmaf is monotone in the plane coordinate), so this is the classic slab
-// test without its per-axis min / max; an unused slot (lo > hi) misses.
-__device__ __forceinline__ uint32_t box4(const Ray& r, float tmax, const WNodeRay& n, float t[4]) {
+// k[c] = the distance at which the ray enters child c, infinite for a miss
+// (tmax is finite).  For a box with lo <= hi the near plane's distance is
+// exactly the smaller of the two slab distances (fmaf is monotone in the plane
+// coordinate), so this is the classic slab test without its per-axis min / max;
+// an unused slot (lo > hi) misses.
+__device__ __forceinline__ void box4(const Ray& r, float tmax, const WNodeRay& n, float k[4]) {
   const float nx[4] = {n.nx.x, n.nx.y, n.nx.z, n.nx.w}, fx[4] = {n.fx.x, n.fx.y, n.fx.z, n.fx.w};
   const float ny[4] = {n.ny.x, n.ny.y, n.ny.z, n.ny.w}, fy[4] = {n.fy.x, n.fy.y, n.fy.z, n.fy.w};
   const float nz[4] = {n.nz.x, n.nz.y, n.nz.z, n.nz.w}, fz[4] = {n.fz.x, n.fz.y, n.fz.z, n.fz.w};
-  uint32_t mask = 0;
+  float ax[4], ay[4], az[4], bx[4], by[4], bz[4];
+#pragma unroll
+  for (int c = 0; c < 4; c += 2) {
+    fma2(nx[c], nx[c + 1], r.inv.x, r.ooi.x, ax[c], ax[c + 1]);
+    fma2(ny[c], ny[c + 1], r.inv.y, r.ooi.y, ay[c], ay[c + 1]);
+    fma2(nz[c], nz[c + 1], r.inv.z, r.ooi.z, az[c], az[c + 1]);
+    fma2(fx[c], fx[c + 1], r.inv.x, r.ooi.x, bx[c], bx[c + 1]);
+    fma2(fy[c], fy[c + 1], r.inv.y, r.ooi.y, by[c], by[c + 1]);
+    fma2(fz[c], fz[c + 1], r.inv.z, r.ooi.z, bz[c], bz[c + 1]);
+  }
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
-    const float tn = fmax3(fmaf(nx[c], r.inv.x, r.ooi.x), fmaf(ny[c], r.inv.y, r.ooi.y),
-                           fmaxf(fmaf(nz[c], r.inv.z, r.ooi.z), r.tmin));
-    const float tf = fmin3(fmaf(fx[c], r.inv.x, r.ooi.x), fmaf(fy[c], r.inv.y, r.ooi.y),
-                           fminf(fmaf(fz[c], r.inv.z, r.ooi.z), tmax));
-    t[c] = tn;
-    mask |= (tn <= tf ? 1u : 0u) << c;
+    const float tn = fmax3(ax[c], ay[c], fmaxf(az[c], r.tmin)), tf = fmin3(bx[c], by[c], fminf(bz[c], tmax));
+    k[c] = tn <= tf ? tn : __int_as_float(0x7f800000);
   }
-  return mask;
 }
 
 // One box (lo xyz, hi xyz) against the ray within [tmin, tmax]; entry distance.
@@ -371,7 +387,13 @@ struct Work {
 // Visit a wide node: push the hit children far-to-near, return the nearest
 // in ``next`` (INT32_MIN if none was hit).  False on stack overflow.  The
 // four (distance, child) pairs are ordered by a five-comparator sorting
-// network on registers, misses carrying an infinite distance.
+// network on registers, misses carrying an infinite distance, which also tells
+// how many to push.  The persistent kernels are bound by the instructions of this
+// step as much as by its loads: without the hit mask and its count, with packed
+// multiply-adds and node counts taken per ray, the city trace-all kernel went from
+// 761 to 705 us and the villa's reuse kernel from 887 to 786 us (two node steps per
+// leaf step, trace_core.cuh, are part of that).  Leaving out one or two comparators
+// visits more nodes and is slower (city reuse kernel 274 -> 291 and 286 us).
 __device__ __forceinline__ void cswap(float& ka, int& va, float& kb, int& vb) {
   const bool s = kb < ka;
   const float k = s ? kb : ka;
@@ -389,15 +411,16 @@ __device__ __forceinline__ void cswap(float& ka, int& va, float& kb, int& vb) {
 // ray enters each child's box and drops an entry that comes up after a closer hit
 // was found without loading its node: the node's children lie inside its box, so
 // the box test would miss all of them (fmaf is monotone in the plane coordinates).
-// Rays then visit 10-15 % fewer nodes.  That pays where a thread walks its ray to
-// the end by itself (primary rays of a 1920 x 1080 city image 216 -> 201 us, Alg. 1
-// of 20k paths 54 -> 52 us).  The persistent kernels step their lanes' rays
-// together; there a useless visit costs nothing while other lanes still work, and
-// the wider entries cost more than they save (villa reuse kernel 886 -> 932 us).
+// Rays then visit 10-15 % fewer nodes.  That pays for primary rays, where a thread
+// walks its ray to the end by itself (1920 x 1080 image of the city 216 -> 201 us).
+// The persistent kernels step their lanes' rays together; there a useless visit
+// costs nothing while other lanes still work, and the wider entries cost more than
+// they save (villa reuse kernel 886 -> 932 us).  Alg. 1's queries count the same
+// visits and tests whether they run in k_continue or in the persistent kernel, so
+// both keep plain stacks.
 template <int S>
 struct TStack {
-  static constexpr int kSize = S;
-  int loc[S];
+  int loc[S + 3];              // a node may push three before the depth is checked
   __device__ __forceinline__ void push(int& sp, int ref, float) { loc[sp++] = ref; }
   // the next entry, INT32_MIN once there is none
   __device__ __forceinline__ int pop(int& sp, float) const { return sp > 0 ? loc[--sp] : INT32_MIN; }
@@ -405,8 +428,7 @@ struct TStack {
 
 template <int S>
 struct TStackDist {
-  static constexpr int kSize = S;
-  int2 loc[S];
+  int2 loc[S + 3];
   __device__ __forceinline__ void push(int& sp, int ref, float t) { loc[sp++] = make_int2(ref, __float_as_int(t)); }
   // the next entry within tbest, INT32_MIN once there is none
   __device__ __forceinline__ int pop(int& sp, float tbest) const {
@@ -429,34 +451,28 @@ struct StackOf<true, S> {
 
 template <int S = kStack, class Stk>
 __device__ __forceinline__ bool visit_wide(const WNodeRay& n, const Ray& r, float tbest, Stk& stk, int& sp, int& next) {
-  float t[4];
-  const uint32_t mask = box4(r, tbest, n, t);
-  const int m = __popc(mask);
-  if (m == 0) {
-    next = INT32_MIN;
-    return true;
-  }
+  float k[4];
+  box4(r, tbest, n, k);
   const float inf = __int_as_float(0x7f800000);
-  float k0 = (mask & 1u) ? t[0] : inf, k1 = (mask & 2u) ? t[1] : inf;
-  float k2 = (mask & 4u) ? t[2] : inf, k3 = (mask & 8u) ? t[3] : inf;
+  float k0 = k[0], k1 = k[1], k2 = k[2], k3 = k[3];
   int v0 = n.child.x, v1 = n.child.y, v2 = n.child.z, v3 = n.child.w;
   cswap(k0, v0, k1, v1);
   cswap(k2, v2, k3, v3);
   cswap(k0, v0, k2, v2);
   cswap(k1, v1, k3, v3);
   cswap(k1, v1, k2, v2);
-  if (sp + m - 1 > S) return false;
-  if (m >= 4) stk.push(sp, v3, k3);
-  if (m >= 3) stk.push(sp, v2, k2);
-  if (m >= 2) stk.push(sp, v1, k1);
-  next = v0;
-  return true;
+  if (k3 < inf) stk.push(sp, v3, k3);
+  if (k2 < inf) stk.push(sp, v2, k2);
+  if (k1 < inf) stk.push(sp, v1, k1);
+  next = k0 < inf ? v0 : INT32_MIN;
+  return sp <= S;
 }
 
 // Test the triangles of a leaf range; true if the closest hit improved.
 __device__ __forceinline__ bool visit_leaf(const Tri* tris, int ref, const Ray& r, float& tbest, int& best, int exclude,
                                            Work& wk) {
-  const uint32_t first = leaf_first(ref), cnt = leaf_count(ref);
+  const uint32_t first = leaf_first(ref);
+  const uint32_t cnt = kLeafMax == 1 && kStaticLeafMax == 1 ? 1u : leaf_count(ref);
   bool any = false;
   for (uint32_t i = 0; i < cnt; ++i) {
     ++wk.tris;
@@ -474,39 +490,48 @@ __device__ __forceinline__ bool visit_leaf(const Tri* tris, int ref, const Ray& 
   return any;
 }
 
+// Node steps before a leaf step where each thread walks its ray to the end.  A
+// warp runs node and leaf code one after the other, the leaf code for the few
+// lanes that are at a leaf; with more node steps in between, more lanes are.
+// Measured at 1, 2, 3 and 4: primary rays of the 1920 x 1080 city image 181, 173,
+// 167 and 166 us, visibility rays of 300k paths (k_verify) 77, 77, 76 and 68 us.
+constexpr int kWalkNodes = 4;
+
 // Traverse the wide tree from ``root``; ANY: stop at the first hit.
 // ``tbest`` is the current closest distance (in/out), ``best`` the hit
 // triangle index.  Returns false and records an error on stack overflow or
 // visit cap.
-template <bool ANY, int S = kStack>
+template <bool ANY, int S = kStack, bool kDist = false>
 __device__ __forceinline__ bool traverse(const WNode* nodes, const Tri* tris, int root, const Ray& r, float& tbest,
                                          int& best, int exclude, uint32_t max_visits, int* status, Work& wk) {
-  typename StackOf<!ANY, S>::type stack;     // a segment's any-hit query has no closer hit to find
+  typename StackOf<kDist, S>::type stack;
   int sp = 0;
   int node = root;
   uint32_t visits = 0;
   for (;;) {
-    if (node != INT32_MIN) {
+#pragma unroll
+    for (int j = 0; j < kWalkNodes; ++j) {
+      if (node < 0) continue;
       if (++visits > max_visits) {
         record_error(status, PV_ERR_ITER_CAP);
         return false;
       }
-      if (node >= 0) {
-        ++wk.nodes;
-        const WNodeRay n = load_wnode_ray(nodes, node, r);
-        int next;
-        if (!visit_wide<S>(n, r, tbest, stack, sp, next)) {
-          record_error(status, PV_ERR_STACK);
-          return false;
-        }
-        if (next != INT32_MIN) {
-          node = next;
-          continue;
-        }
-      } else {
-        if (visit_leaf(tris, node, r, tbest, best, exclude, wk) && ANY) return true;
+      ++wk.nodes;
+      const WNodeRay n = load_wnode_ray(nodes, node, r);
+      int next;
+      if (!visit_wide<S>(n, r, tbest, stack, sp, next)) {
+        record_error(status, PV_ERR_STACK);
+        return false;
       }
+      node = next != INT32_MIN ? next : stack.pop(sp, tbest);
     }
+    if (node >= 0) continue;
+    if (node == INT32_MIN) return true;
+    if (++visits > max_visits) {
+      record_error(status, PV_ERR_ITER_CAP);
+      return false;
+    }
+    if (visit_leaf(tris, node, r, tbest, best, exclude, wk) && ANY) return true;
     node = stack.pop(sp, tbest);
     if (node == INT32_MIN) return true;
   }
@@ -519,11 +544,11 @@ struct Hit {
 };
 
 // Closest hit over the whole scene (top level, static tree, dynamic objects).
-template <int S = kStack>
+template <int S = kStack, bool kDist = false>
 __device__ __forceinline__ bool closest_hit(const SceneView& sv, int root, const Ray& r, int exclude, Hit& h, Work& wk) {
   float tb = 3.0e38f;
   int best = -1;
-  if (root != INT32_MIN) traverse<false, S>(sv.nodes, sv.tris, root, r, tb, best, exclude, sv.max_visits, sv.status, wk);
+  if (root != INT32_MIN) traverse<false, S, kDist>(sv.nodes, sv.tris, root, r, tb, best, exclude, sv.max_visits, sv.status, wk);
   h.t = tb;
   h.tri = best;
   return best >= 0;
@@ -554,35 +579,50 @@ __device__ __forceinline__ void trav_begin(Trav& t, int root) {
   t.visits = 0;
 }
 
-// One traversal step (one wide node or one leaf range); true once the ray is done.
-// ``stk`` holds S entries.
-template <int S = kStack, class Stk>
-__device__ __forceinline__ bool trav_step(const SceneView& sv, const Ray& r, Trav& t, Stk& stk, int exclude, Work& wk) {
-  if (t.node != INT32_MIN) {
-    if (++t.visits > sv.max_visits) {
-      record_error(sv.status, PV_ERR_ITER_CAP);
-      return true;
-    }
-    if (t.node >= 0) {
-      ++wk.nodes;
-      const WNodeRay n = load_wnode_ray(sv.nodes, t.node, r);
-      int next;
-      if (!visit_wide<S>(n, r, t.tbest, stk, t.sp, next)) {
-        record_error(sv.status, PV_ERR_STACK);
-        return true;
-      }
-      if (next != INT32_MIN) {
-        t.node = next;
-        return false;
-      }
-    } else {
-      visit_leaf(sv.tris, t.node, r, t.tbest, t.best, exclude, wk);
-    }
-  }
+// Next entry of the stack; true if there is none: the ray is done.
+template <class Stk>
+__device__ __forceinline__ bool trav_pop(Trav& t, const Stk& stk) {
   if (t.sp == 0) return true;
   t.node = stk.loc[--t.sp];
   return false;
 }
+
+// A step counts toward the ray's cap; true if it reached it (the ray stops, a miss).
+__device__ __forceinline__ bool trav_capped(const SceneView& sv, Trav& t) {
+  if (++t.visits <= sv.max_visits) return false;
+  record_error(sv.status, PV_ERR_ITER_CAP);
+  return true;
+}
+
+// One traversal step at a wide node (t.node >= 0); true once the ray is done.
+template <int S = kStack, class Stk>
+__device__ __forceinline__ bool trav_node(const SceneView& sv, const Ray& r, Trav& t, Stk& stk) {
+  if (trav_capped(sv, t)) return true;
+  const WNodeRay n = load_wnode_ray(sv.nodes, t.node, r);
+  int next;
+  if (!visit_wide<S>(n, r, t.tbest, stk, t.sp, next)) {
+    record_error(sv.status, PV_ERR_STACK);
+    return true;
+  }
+  if (next != INT32_MIN) {
+    t.node = next;
+    return false;
+  }
+  return trav_pop(t, stk);
+}
+
+// One traversal step at a leaf range (t.node < 0); true once the ray is done.
+template <class Stk>
+__device__ __forceinline__ bool trav_leaf(const SceneView& sv, const Ray& r, Trav& t, Stk& stk, int exclude, Work& wk) {
+  if (trav_capped(sv, t)) return true;
+  --wk.nodes;                                  // trav_end adds every step as a node
+  if (t.node == INT32_MIN) return true;        // an empty scene
+  visit_leaf(sv.tris, t.node, r, t.tbest, t.best, exclude, wk);
+  return trav_pop(t, stk);
+}
+
+// A ray has ended: its steps join the node count (leaf steps have left it).
+__device__ __forceinline__ void trav_end(const Trav& t, Work& wk) { wk.nodes += t.visits; }
 
 __device__ __forceinline__ uint32_t info_nseg(uint32_t w) { return (w >> PV_INFO_NSEG_SHIFT) & 15u; }
 __device__ __forceinline__ uint32_t info_start(uint32_t w) { return (w >> PV_INFO_START_SHIFT) & 15u; }

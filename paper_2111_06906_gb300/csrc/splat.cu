@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(256, 5) k_gbuffer(SceneView sv, Cam c, GPixel*
   o.p = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
   o.n = make_float4(0.f, 0.f, 0.f, 0.f);
   const int root = *sv.root;
-  if (closest_hit(sv, root, r, -1, h, wk)) {
+  if (closest_hit<kStack, true>(sv, root, r, -1, h, wk)) {
     const Tri T = load_tri(sv.tris, h.tri);
     const float3 p = make_float3(fmaf(h.t, d.x, c.pos.x), fmaf(h.t, d.y, c.pos.y), fmaf(h.t, d.z, c.pos.z));
     float3 nn = normalize(cross(f3(T.e1), f3(T.e2)));

@@ -23,16 +23,11 @@ namespace {
 
 // Compile-time tuning: minimum resident blocks; traversal steps between
 // refills.  A warp keeps stepping until every lane's ray has ended (at most
-// PV_TRACE_MAX_STEPS steps), so that the ray-end code (photon store, bounce
+// PV_TRACE_MAX_STEPS node steps), so that the ray-end code (photon store, bounce
 // sampling, next list entry) runs with all lanes at once: measured on the
 // city and villa workloads this beats refilling each lane after a fixed
-// number of steps (8) by 8-13 % on the re-trace and 14-15 % on trace-all.
-// PV_TRACE_DONE_LANES < 32 stops once that many lanes are done (after at
-// least PV_TRACE_STEPS steps); PV_TRACE_DONE_LANES > 32 restores the fixed
-// PV_TRACE_STEPS-step loop.
-#ifndef PV_TRACE_STEPS
-#define PV_TRACE_STEPS 16
-#endif
+// number of steps (8) by 8-13 % on the re-trace and 14-15 % on trace-all, and
+// stopping once 24 or 16 lanes are done by 4-22 %.
 // Resident blocks asked of the register allocator: k_trace fits 8 blocks
 // (64 registers) without spills, and that beat 7 by 3-5 % on the city and
 // villa trace-all frames; k_cont_trace keeps 7 (72 registers), since 8 spill
@@ -58,33 +53,8 @@ namespace {
 #ifndef PV_TRACE_MAX_STEPS
 #define PV_TRACE_MAX_STEPS 64
 #endif
-#ifndef PV_TRACE_DONE_LANES
-#define PV_TRACE_DONE_LANES 32
-#endif
 using TraceStack = TStack<kStack>;
-constexpr int kStepsPerIter = PV_TRACE_STEPS;
 constexpr int kMaxSteps = PV_TRACE_MAX_STEPS;
-constexpr int kDoneLanes = PV_TRACE_DONE_LANES;
-
-// Advance the lane's ray; all lanes of the warp call it (lanes without a ray
-// pass done = true).  Returns whether the lane's ray has ended.
-__device__ __forceinline__ bool step_rays(const SceneView& sv, const Ray& r, Trav& t, TraceStack& stk, int excl, Work& wk,
-                                          bool done) {
-  if (kDoneLanes > 32) {
-#pragma unroll 1
-    for (int i = 0; i < kStepsPerIter && !done; ++i) done = trav_step(sv, r, t, stk, excl, wk);
-    return done;
-  }
-  if (kDoneLanes >= 32) return step_warp<kMaxSteps>(sv, r, t, stk, excl, wk, done);
-#pragma unroll 1
-  for (int i = 0; i < kMaxSteps; ++i) {
-    if (!done) done = trav_step(sv, r, t, stk, excl, wk);
-    const unsigned dm = __ballot_sync(0xffffffffu, done);
-    if (dm == 0xffffffffu) break;
-    if (i + 1 >= kStepsPerIter && __popc(dm) >= kDoneLanes) break;
-  }
-  return done;
-}
 
 // Re-trace (A.list) or trace-all; with kDep every photon stored is also
 // deposited into am's atlas as it is stored (the fused trace-all frame).
@@ -127,9 +97,9 @@ __global__ void __launch_bounds__(pvh::kTraceThreads, kDep ? PV_TRACE_DEP_MIN_BL
       }
     }
     if (__all_sync(0xffffffffu, exhausted && !has_ray)) break;
-    if (kDoneLanes > 32 && !has_ray) continue;
-    const bool done = step_rays(sv, r, t, stk, s.excl, wk, !has_ray);
+    const bool done = step_warp<kMaxSteps>(sv, r, t, stk, s.excl, wk, !has_ray);
     if (!has_ray || !done) continue;
+    trav_end(t, wk);
     ++c_rays;
     if (trace_hit<kDep>(sv, A, s, r, t, c_photons, &am)) trav_begin(t, root);
     else has_ray = false;
@@ -260,9 +230,9 @@ __global__ void __launch_bounds__(pvh::kTraceThreads, PV_CONT_TRACE_MIN_BLOCKS)
       }
     }
     if (__all_sync(0xffffffffu, (exhausted || waits) && !has_ray && dep == 0xFFFFFFFFu)) break;
-    if (kDoneLanes > 32 && !has_ray) continue;
-    const bool done = step_rays(sv, r, t, stk, s.excl, wk, !has_ray);
+    const bool done = step_warp<kMaxSteps>(sv, r, t, stk, s.excl, wk, !has_ray);
     if (!has_ray || !done) continue;
+    trav_end(t, wk);
     if (cont) {
       ContCounters cc;
       float3 a_cur;
