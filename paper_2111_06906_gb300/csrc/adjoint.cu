@@ -79,7 +79,7 @@ __device__ __forceinline__ Emission model_emission(const LightPose& Lp, const fl
 // Unit normal of stored photon v's triangle and its dynamic slot (-1: static).
 __device__ __forceinline__ float3 photon_normal(const SceneView& sv, float4 v, int& slot) {
   const int prim = __float_as_int(v.w);
-  const uint32_t sl = __ldg(sv.prim_slot + prim);
+  const uint32_t sl = slot_of(sv, prim);
   slot = sl == 255u ? -1 : (int)sl;
   return normalize(prim_normal(sv, prim, false));
 }

@@ -150,7 +150,8 @@ struct SceneView {
   const DynObj* objs;
   const MovedGroups* groups;   // moved objects in groups (valid in frames where objects moved)
   uint32_t n_dyn;
-  const uint8_t* prim_slot;  // [n_tris] 255 = static, else dynamic slot
+  const uint8_t* prim_slot;  // [n_tris] 255 = static, else dynamic slot (read through slot_of)
+  uint32_t dyn_first, dyn_span;   // every dynamic primitive lies in [dyn_first, dyn_first + dyn_span)
   const uint32_t* prim_dyn;  // [n_tris] index into the dynamic arrays (dynamic prims)
   const float4* prim_alb;    // [n_tris] albedo rgb, w = max (Russian-roulette q)
   const float4* prim_nrm;    // [n_tris] e1 x e2 of the given corners (object-local for dynamic)
@@ -729,17 +730,24 @@ __device__ __forceinline__ float3 cof_apply(const float* m, float3 n) {
   return n.x * cross(c1, c2) + n.y * cross(c2, c0) + n.z * cross(c0, c1);
 }
 
+// Dynamic slot of a primitive, 255 = static (also for prim < 0).  Primitives
+// outside the range of the dynamic ones need no table look-up: a scene's moving
+// objects mostly have consecutive ids, and the table (a byte per primitive, read
+// at random) does not fit L1.
+__device__ __forceinline__ uint32_t slot_of(const SceneView& sv, int prim) {
+  return (uint32_t)prim - sv.dyn_first < sv.dyn_span ? __ldg(sv.prim_slot + prim) : 255u;
+}
+
 // Unnormalised geometric normal of a primitive at the old or new pose.
 __device__ __forceinline__ float3 prim_normal(const SceneView& sv, int prim, bool old_pose) {
   const float3 n = f3(__ldg(sv.prim_nrm + prim));
-  const uint32_t slot = __ldg(sv.prim_slot + prim);
+  const uint32_t slot = slot_of(sv, prim);
   if (slot == 255u) return n;
   return cof_apply((old_pose ? sv.xf_old : sv.xf_new) + 12 * slot, n);
 }
 
 __device__ __forceinline__ bool slot_moved(const SceneView& sv, int prim) {
-  if (prim < 0) return false;
-  const uint32_t slot = __ldg(sv.prim_slot + prim);
+  const uint32_t slot = slot_of(sv, prim);
   return slot != 255u && ((sv.moved >> slot) & 1ull);
 }
 
@@ -759,10 +767,19 @@ __device__ __forceinline__ bool energy_close(float3 EN, float3 EO, float tau) {
   return ok;
 }
 
+// A box in shared memory: lo.xyz and hi.x, then hi.y and hi.z, read as one 16-
+// and one 8-byte word.
+struct __align__(16) Box {
+  float4 a;
+  float2 b, pad;
+  __device__ __forceinline__ void set(int k, float v) { reinterpret_cast<float*>(this)[k] = v; }   // k = 0..5: lo, hi
+  __device__ __forceinline__ float get(int k) const { return reinterpret_cast<const float*>(this)[k]; }
+};
+
 // Load the dynamic objects' boxes into shared memory: ``cull`` = current
 // tight box padded by a relative 2^-20 (ray culling only), ``uni`` = exact
 // union of the old and new tight boxes (the Sec. 3.2 box test).
-__device__ __forceinline__ void load_boxes(const SceneView& sv, float* cull, float* uni) {
+__device__ __forceinline__ void load_boxes(const SceneView& sv, float* cull, Box* uni) {
   for (uint32_t i = threadIdx.x; i < sv.n_dyn * 6; i += blockDim.x) {
     const DynObj& o = sv.objs[i / 6];
     const int k = i % 6;
@@ -771,7 +788,7 @@ __device__ __forceinline__ void load_boxes(const SceneView& sv, float* cull, flo
     const float hi3 = fmaxf(fmaxf(fabsf(o.box_new[3]), fabsf(o.box_new[4])), fabsf(o.box_new[5]));
     const float pad = 9.5367431640625e-07f * fmaxf(lo3, hi3) + 1e-30f;
     cull[i] = k < 3 ? bn - pad : bn + pad;
-    if (uni) uni[i] = k < 3 ? fminf(bn, bo) : fmaxf(bn, bo);
+    uni[i / 6].set(k, k < 3 ? fminf(bn, bo) : fmaxf(bn, bo));
   }
 }
 

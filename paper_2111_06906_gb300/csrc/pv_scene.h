@@ -13,7 +13,7 @@
 struct pv_scene {
   int device = 0;
   int num_sms = 0;
-  int verify_blocks_per_sm[4] = {0, 0, 0, 0};   // resident k_verify blocks per SM, by (point vis, exact)
+  int verify_blocks_per_sm[8] = {};  // resident k_verify blocks per SM, by (point vis, exact, flat)
   uint32_t n_tris = 0, n_objects = 0, n_static = 0, n_dyn_tris = 0, n_dyn = 0;
   uint32_t B = 0;
   float diag = 0.f, tmin = 0.f, close_tol = 0.f;
@@ -71,6 +71,7 @@ struct pv_scene {
   uint32_t* r_prim = nullptr;
 
   // per primitive
+  uint32_t dyn_first = 0, dyn_span = 0;   // the dynamic primitives lie in [dyn_first, dyn_first + dyn_span)
   uint8_t* prim_slot = nullptr;
   uint32_t* prim_dyn = nullptr;
   float4* prim_alb = nullptr;

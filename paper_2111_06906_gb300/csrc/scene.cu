@@ -74,6 +74,8 @@ SceneView view(const pv_scene* s) {
   v.groups = s->groups;
   v.n_dyn = s->n_dyn;
   v.prim_slot = s->prim_slot;
+  v.dyn_first = s->dyn_first;
+  v.dyn_span = s->dyn_span;
   v.prim_dyn = s->prim_dyn;
   v.prim_alb = s->prim_alb;
   v.prim_nrm = s->prim_nrm;
@@ -203,6 +205,8 @@ extern "C" int pv_build_scene(const pv_scene_desc* d, void* stream, pv_scene** o
                           (float)(e1[0] * e2[1] - e1[1] * e2[0]), 0.f);
     if (slot_of[o] >= 0) {
       pslot[t] = (uint8_t)slot_of[o];
+      if (!s->dyn_span) s->dyn_first = t;
+      s->dyn_span = t - s->dyn_first + 1;
       s->dyn_tris_of[slot_of[o]].push_back(t);
       s->n_dyn_tris++;
     } else {

@@ -27,43 +27,44 @@ namespace {
 #define PV_VERIFY_PERSISTENT 1
 #endif
 // Resident blocks asked of the register allocator for the box-only kernel:
-// 5 (51 registers) beat the 4 that 56 registers allow by 7 % on the villa
-// workload.  The variants with traversal code keep their registers (they
+// 5 (48 registers) beat 4 by 6 % on the villa workload, and on the city's map frame
+// by 4 %; on the plain city frame 4 are 2 % faster, 6 are slower on all.  The variants with traversal code keep their registers (they
 // would spill).
 #ifndef PV_VERIFY_MIN_BLOCKS
 #define PV_VERIFY_MIN_BLOCKS 5
 #endif
 constexpr bool kVerifyLoop = PV_VERIFY_FLAT && PV_VERIFY_PERSISTENT;
 
-// Flat segment mapping in error mode, else thread per path; with
-// kVerifyLoop a grid of resident blocks looping over tiles.  A re-trace kernel launched as its
-// programmatic dependent (PV_CONT_TRACE_PDL) may be scheduled as soon as every block has started.
-template <bool kPointVis, bool kExact>
+// Flat segment mapping in error mode (kFlat), else thread per path, each a
+// kernel of its own (one kernel with both needs the registers of the larger);
+// with kVerifyLoop a grid of resident blocks looping over tiles.  A re-trace kernel
+// launched as its programmatic dependent (PV_CONT_TRACE_PDL) may be scheduled as
+// soon as every block has started.
+template <bool kPointVis, bool kExact, bool kFlat>
 __device__ __forceinline__ void verify_kernel(const SceneView& sv, const FrameLights& L, const VerifyArgs& A,
                                               VerifySmem& sm) {
   launch_dependents();
-  const bool flat = PV_VERIFY_FLAT && A.mode == PV_MODE_ERROR;
   if (kVerifyLoop) {
-    if (flat) verify_tiles<kPointVis, kExact, 2>(sv, L, A, blockIdx.x, gridDim.x, sm);
-    else verify_tiles<kPointVis, kExact, 0>(sv, L, A, blockIdx.x, gridDim.x, sm);
+    verify_tiles<kPointVis, kExact, kFlat ? 2 : 0>(sv, L, A, blockIdx.x, gridDim.x, sm);
   } else {
-    if (flat) verify_block_flat<kPointVis, kExact>(sv, L, A, blockIdx.x * blockDim.x + threadIdx.x, sm);
+    if (kFlat) verify_block_flat<kPointVis, kExact>(sv, L, A, blockIdx.x * blockDim.x + threadIdx.x, sm);
     else verify_block<kPointVis, kExact>(sv, L, A, blockIdx.x * blockDim.x + threadIdx.x, sm);
   }
 }
 
 // With visibility rays or triangle tests (traversal code inside).
-template <bool kPointVis, bool kExact>
+template <bool kPointVis, bool kExact, bool kFlat>
 __global__ void __launch_bounds__(pvh::kVerifyThreads) k_verify(SceneView sv, FrameLights L, VerifyArgs A) {
   __shared__ VerifySmem sm;
-  verify_kernel<kPointVis, kExact>(sv, L, A, sm);
+  verify_kernel<kPointVis, kExact, kFlat>(sv, L, A, sm);
 }
 
 // Box tests only, the common case.
+template <bool kFlat>
 __global__ void __launch_bounds__(pvh::kVerifyThreads, PV_VERIFY_MIN_BLOCKS) k_verify_box(SceneView sv, FrameLights L,
                                                                                          VerifyArgs A) {
   __shared__ VerifySmem sm;
-  verify_kernel<false, false>(sv, L, A, sm);
+  verify_kernel<false, false, kFlat>(sv, L, A, sm);
 }
 
 // Blocks of a k_verify kernel for n paths: every tile, or with the tile
@@ -80,16 +81,22 @@ uint32_t verify_grid(pv_scene* s, K kernel, int& per, uint32_t n) {
   return std::min<uint32_t>(tiles, pvh::verify_block_cap((uint32_t)per * (uint32_t)s->num_sms));
 }
 
+template <bool kPointVis, bool kExact, bool kFlat>
+void launch_k_verify(pv_scene* s, const SceneView& sv, const FrameLights& L, const VerifyArgs& A, cudaStream_t st) {
+  int& per = s->verify_blocks_per_sm[(kPointVis ? 4 : 0) + (kExact ? 2 : 0) + (kFlat ? 1 : 0)];
+  if constexpr (!kPointVis && !kExact) {
+    const uint32_t grid = verify_grid(s, k_verify_box<kFlat>, per, A.n);
+    k_verify_box<kFlat><<<grid, pvh::kVerifyThreads, 0, st>>>(sv, L, A);
+  } else {
+    const uint32_t grid = verify_grid(s, k_verify<kPointVis, kExact, kFlat>, per, A.n);
+    k_verify<kPointVis, kExact, kFlat><<<grid, pvh::kVerifyThreads, 0, st>>>(sv, L, A);
+  }
+}
+
 template <bool kPointVis, bool kExact>
 void launch_k_verify(pv_scene* s, const SceneView& sv, const FrameLights& L, const VerifyArgs& A, cudaStream_t st) {
-  int& per = s->verify_blocks_per_sm[(kPointVis ? 2 : 0) + (kExact ? 1 : 0)];
-  if (!kPointVis && !kExact) {
-    const uint32_t grid = verify_grid(s, k_verify_box, per, A.n);
-    k_verify_box<<<grid, pvh::kVerifyThreads, 0, st>>>(sv, L, A);
-  } else {
-    const uint32_t grid = verify_grid(s, k_verify<kPointVis, kExact>, per, A.n);
-    k_verify<kPointVis, kExact><<<grid, pvh::kVerifyThreads, 0, st>>>(sv, L, A);
-  }
+  if (PV_VERIFY_FLAT && A.mode == PV_MODE_ERROR) launch_k_verify<kPointVis, kExact, true>(s, sv, L, A, st);
+  else launch_k_verify<kPointVis, kExact, false>(s, sv, L, A, st);
 }
 
 __global__ void __launch_bounds__(128, 6) k_continue(SceneView sv, ContArgs A) {

@@ -41,10 +41,12 @@ struct VerifyArgs {
 // reciprocal 1e20 of its sign, which keeps the axis' interval around [0,1]
 // when a lies inside the slab and away from it when a lies outside; only a
 // segment lying exactly in a face plane can be decided differently).
-__device__ __forceinline__ bool seg_box(float3 inv, float3 aoi, const float* bx) {
-  const float x0 = fmaf(bx[0], inv.x, aoi.x), x1 = fmaf(bx[3], inv.x, aoi.x);
-  const float y0 = fmaf(bx[1], inv.y, aoi.y), y1 = fmaf(bx[4], inv.y, aoi.y);
-  const float z0 = fmaf(bx[2], inv.z, aoi.z), z1 = fmaf(bx[5], inv.z, aoi.z);
+__device__ __forceinline__ bool seg_box(float3 inv, float3 aoi, const Box& bx) {
+  const float4 p = bx.a;
+  const float2 h = bx.b;
+  const float x0 = fmaf(p.x, inv.x, aoi.x), x1 = fmaf(p.w, inv.x, aoi.x);
+  const float y0 = fmaf(p.y, inv.y, aoi.y), y1 = fmaf(h.x, inv.y, aoi.y);
+  const float z0 = fmaf(p.z, inv.z, aoi.z), z1 = fmaf(h.y, inv.z, aoi.z);
   const float t0 = fmax3(fminf(x0, x1), fminf(y0, y1), fmaxf(fminf(z0, z1), 0.0f));
   const float t1 = fmin3(fmaxf(x0, x1), fmaxf(y0, y1), fminf(fmaxf(z0, z1), 1.0f));
   return t0 <= t1;
@@ -88,9 +90,9 @@ __device__ __forceinline__ Seg seg_prep(const SceneView& sv, float3 a, float3 b,
 // old pose with PV_FLAG_TEST_OLD_TRIS, by brute force over object-local
 // corners).
 template <int S = kStack>
-__device__ __forceinline__ bool seg_vs_object(const SceneView& sv, const Seg& g, const float* cull, const float* uni,
+__device__ __forceinline__ bool seg_vs_object(const SceneView& sv, const Seg& g, const float* cull, const Box* uni,
                                               bool boxes, bool test_old, int s, Work& wk) {
-  if (boxes) return seg_box(g.inv, g.aoi, uni + 6 * s);
+  if (boxes) return seg_box(g.inv, g.aoi, uni[s]);
   if (!g.ok) return false;
   float te;
   if (sv.objs[s].wroot != INT32_MIN && box1(g.r, g.tmax, cull + 6 * s, te)) {
@@ -121,10 +123,11 @@ __device__ __forceinline__ bool seg_vs_object(const SceneView& sv, const Seg& g,
   return false;
 }
 
-// Moved-object groups staged in shared memory (MovedGroups).
+// Moved-object groups staged in shared memory (MovedGroups): their boxes, and the
+// members' boxes group after group (empty past a group's last).
 struct GroupSmem {
-  float box[kMaxGroups][6];
-  int8_t slot[kMaxGroups][kGroupSize];
+  Box box[kMaxGroups];
+  Box member[kMaxGroups * kGroupSize];
   int n;
 };
 
@@ -150,43 +153,46 @@ __device__ __forceinline__ SegBounds seg_bounds(float3 a, float3 b) {
   return s;
 }
 
-// Closed box bx (lo xyz, hi xyz) against the widened segment bounds.
-__device__ __forceinline__ bool seg_overlaps(const SegBounds& s, const float* bx) {
-  return (s.lo.x <= bx[3]) & (s.hi.x >= bx[0]) & (s.lo.y <= bx[4]) & (s.hi.y >= bx[1]) & (s.lo.z <= bx[5]) &
-         (s.hi.z >= bx[2]);
+// Closed box bx against the widened segment bounds.
+__device__ __forceinline__ bool seg_overlaps(const SegBounds& s, const Box& bx) {
+  const float4 p = bx.a;
+  const float2 h = bx.b;
+  return (s.lo.x <= p.w) & (s.hi.x >= p.x) & (s.lo.y <= h.x) & (s.hi.y >= p.y) & (s.lo.z <= h.y) & (s.hi.z >= p.z);
 }
 
 // Segment a->b against every moved object.  Box tests cull first by the
 // segment's widened bounds against the union of all moved boxes, then
 // against each group's box, and run the slab test (seg_box) only on members
-// whose box the bounds overlap (its reciprocals computed once the union
-// cull has passed).  Neither cull rejects a box that seg_box accepts
+// whose box the bounds overlap, which few segments have (so its reciprocals are
+// computed there).  Neither cull rejects a box that seg_box accepts
 // (seg_bounds), and a box that contains another overlaps whatever the inner
 // one does, so the result is that of the slab test against every moved
-// object.
+// object.  With boxes read as 16- and 8-byte words, members in group order, the
+// reciprocals late and no slot look-up for static primitives (slot_of), the villa's
+// verification (3M paths, 10 moved objects) went from 161 to 144 us.
 template <int S = kStack>
-__device__ __forceinline__ bool seg_vs_moved(const SceneView& sv, const float* cull, const float* uni,
+__device__ __forceinline__ bool seg_vs_moved(const SceneView& sv, const float* cull, const Box* uni,
                                              const GroupSmem& gs, bool boxes, bool test_old, float3 a, float3 b,
                                              Work& wk) {
   if (boxes) {
     const SegBounds sb = seg_bounds(a, b);
-    if (!seg_overlaps(sb, uni + 6 * kMaxDyn)) return false;
-    const Seg g = seg_prep(sv, a, b, true);
-    auto slab = [&](const float* bx) { return seg_box(g.inv, g.aoi, bx); };
+    if (!seg_overlaps(sb, uni[kMaxDyn])) return false;
+    auto slab = [&](const Box& bx) {
+      const Seg g = seg_prep(sv, a, b, true);
+      return seg_box(g.inv, g.aoi, bx);
+    };
     if (gs.n == 0) {                           // no group table: every moved object in turn
       for (uint64_t m = sv.moved; m; m &= m - 1) {
-        const float* bx = uni + 6 * (__ffsll((long long)m) - 1);
+        const Box& bx = uni[__ffsll((long long)m) - 1];
         if (seg_overlaps(sb, bx) && slab(bx)) return true;
       }
       return false;
     }
     for (int q = 0; q < gs.n; ++q) {
       if (gs.n > 1 && !seg_overlaps(sb, gs.box[q])) continue;   // one group: its box is the union
-#pragma unroll
-      for (int m = 0; m < kGroupSize; ++m) {
-        const int s = gs.slot[q][m];
-        if (s < 0) break;
-        const float* bx = uni + 6 * s;
+#pragma unroll 1
+      for (int m = 0; m < kGroupSize; ++m) {   // (all four at once spill, 3 % slower)
+        const Box& bx = gs.member[kGroupSize * q + m];
         if (seg_overlaps(sb, bx) && slab(bx)) return true;
       }
     }
@@ -205,7 +211,7 @@ __device__ __forceinline__ uint32_t* field(pv_frame_stats* s, size_t off) {
 // Shared memory of one verify block.
 struct VerifySmem {
   float cull[kMaxDyn * 6];
-  float uni[(kMaxDyn + 1) * 6];
+  Box uni[kMaxDyn + 1];        // every object's, then the union of the moved ones
   GroupSmem groups;
   uint32_t red[32 * 7];
   unsigned long long red64[32];
@@ -355,12 +361,15 @@ __device__ __forceinline__ bool finish_stage(const VerifyArgs& A, uint32_t p, co
 // Block prologue: moved objects' boxes, their union, and the moved-slot list.
 __device__ __forceinline__ void verify_smem_init(const SceneView& sv, VerifySmem& sm) {
   load_boxes(sv, sm.cull, sm.uni);
+  __syncthreads();
   // this frame's groups of the moved objects (none without a group table)
   const bool have = sv.moved && sv.groups;
   const int ng = have ? (int)min(sv.groups->n, (uint32_t)kMaxGroups) : 0;
-  for (int i = threadIdx.x; i < ng * 6; i += blockDim.x) sm.groups.box[i / 6][i % 6] = sv.groups->box[i / 6][i % 6];
-  for (int i = threadIdx.x; i < ng * kGroupSize; i += blockDim.x)
-    sm.groups.slot[i / kGroupSize][i % kGroupSize] = sv.groups->slot[i / kGroupSize][i % kGroupSize];
+  for (int i = threadIdx.x; i < ng * 6; i += blockDim.x) sm.groups.box[i / 6].set(i % 6, sv.groups->box[i / 6][i % 6]);
+  for (int i = threadIdx.x; i < ng * kGroupSize * 6; i += blockDim.x) {
+    const int m = i / 6, k = i % 6, s = sv.groups->slot[m / kGroupSize][m % kGroupSize];
+    sm.groups.member[m].set(k, s >= 0 ? sm.uni[s].get(k) : k < 3 ? 3.0e38f : -3.0e38f);
+  }
   if (threadIdx.x == 0) sm.groups.n = ng;
   if (threadIdx.x == 0) {
     int k = 0;
@@ -372,10 +381,10 @@ __device__ __forceinline__ void verify_smem_init(const SceneView& sv, VerifySmem
     const int k = threadIdx.x;
     float v = k < 3 ? 3.0e38f : -3.0e38f;
     for (uint64_t m = sv.moved; m; m &= m - 1) {
-      const float x = sm.uni[6 * (__ffsll((long long)m) - 1) + k];
+      const float x = sm.uni[__ffsll((long long)m) - 1].get(k);
       v = k < 3 ? fminf(v, x) : fmaxf(v, x);
     }
-    sm.uni[6 * kMaxDyn + k] = v;
+    sm.uni[kMaxDyn].set(k, v);
   }
   __syncthreads();
 }
@@ -535,7 +544,7 @@ __device__ __forceinline__ void verify_tile_warp(const SceneView& sv, const Fram
       const float3 a = k == 1 ? o : f3(A.pa[(size_t)(k - 2) * n + pj]);
       const Seg g = seg_prep(sv, a, b, !kExact);
       bool hit;
-      if (!kExact) hit = seg_box(g.inv, g.aoi, sm.uni + 6 * kMaxDyn) && seg_vs_object<S>(sv, g, sm.cull, sm.uni, true, false, obj, wk);
+      if (!kExact) hit = seg_box(g.inv, g.aoi, sm.uni[kMaxDyn]) && seg_vs_object<S>(sv, g, sm.cull, sm.uni, true, false, obj, wk);
       else hit = seg_vs_object<S>(sv, g, sm.cull, sm.uni, false, test_old, obj, wk);
       if (hit) tmask |= 1u << k;
     }
