@@ -30,10 +30,11 @@ void launch_compact(pv_scene* s, const uint32_t* info, uint32_t n, uint32_t* lis
     return;
   }
   const uint32_t n_tiles = (n + kTile - 1) / kTile;
-  cudaMemsetAsync(s->ws_tiles, 0, (size_t)n_tiles * sizeof(uint64_t), st);
-  cudaMemsetAsync(s->ws_ctr + CTR_TILE, 0, sizeof(uint32_t), st);
+  // the tile states and, in the word behind them, the tile ticket
+  cudaMemsetAsync(s->ws_tiles, 0, ((size_t)n_tiles + 1) * sizeof(uint64_t), st);
   k_compact<<<n_tiles, kCompactThreads, 0, st>>>(info, n, list, count, reinterpret_cast<unsigned long long*>(s->ws_tiles),
-                                                 s->ws_ctr + CTR_TILE, n_tiles, s->status, stats_listed, nullptr);
+                                                 reinterpret_cast<uint32_t*>(s->ws_tiles + n_tiles), n_tiles, s->status,
+                                                 stats_listed, nullptr);
 }
 
 }  // namespace pvh

@@ -13,7 +13,7 @@ __global__ void __launch_bounds__(256) k_deposit(uint32_t n, uint32_t B, const u
   // whole warps loop, so that the photons of each round's 32 paths are dealt out over the lanes
   for (uint32_t b = blockIdx.x * blockDim.x; b < n; b += gridDim.x * blockDim.x) {
     const uint32_t p = b + threadIdx.x;
-    deposit_warp(am, n, B, info, pa, pb, p < n ? p : 0xFFFFFFFFu);
+    deposit_warp<true>(am, n, B, info, pa, pb, p < n ? p : 0xFFFFFFFFu);
   }
 }
 

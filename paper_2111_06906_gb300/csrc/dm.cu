@@ -92,7 +92,7 @@ int dm_frame(pv_scene* s, const pv_paths* p, const FrameLights& L, const pv_veri
     if (L.dm[l].dims && ((L.moved_mask >> l) & 1u)) moved |= 1u << l;
   if (!moved || p->n == 0) return PV_OK;
   const uint32_t n = p->n, blocks = (n + 255) / 256;
-  PV_CHECK(cudaMemsetAsync(s->dm_ctr, 0, 8 * sizeof(uint32_t), st));
+  // dm_ctr was cleared with the other work counters before verification
   k_dm_prune<<<blocks, 256, 0, st>>>(L, n, p->info, s->dm_flag, prm->seed, prm->frame, stats);
   k_dm_commit<<<blocks, 256, 0, st>>>(L, n, p->info, s->dm_flag, s->dm_ctr);
   launch_compact(s, s->dm_flag, n, s->dm_free, s->dm_ctr + 4, nullptr, st);

@@ -92,7 +92,7 @@ struct pv_scene {
   uint32_t* ws_cont = nullptr;       // [n_paths] continuation list
   uint32_t* ws_list = nullptr;       // [n_paths] re-trace list of pv_verify_retrace
   uint8_t* ws_touched = nullptr;     // [n_paths] paths the frame re-traces or hands to Alg. 1 (fused deposit)
-  uint64_t* ws_tiles = nullptr;      // [n_tiles + 1] decoupled look-back tile states
+  uint64_t* ws_tiles = nullptr;      // [n_tiles + 1] decoupled look-back tile states, then the tile ticket
   uint32_t n_tiles = 0;
   uint32_t* ws_ctr = nullptr;        // [16] work counters
   // distribution maps (Sec. 3.1), per light; workspace shared by the lights
@@ -103,7 +103,7 @@ struct pv_scene {
   uint32_t* dm_free = nullptr;                // [n_paths] free paths, ascending
   uint32_t* dm_scan = nullptr;                // [max cells + 1] deficits, then their exclusive prefix
   uint32_t* dm_sums = nullptr;                // [tiles of the largest map] sums of its tiles (behind dm_scan)
-  uint32_t* dm_ctr = nullptr;                 // [8] free paths per light, free-list length
+  uint32_t* dm_ctr = nullptr;                 // [8] free paths per light, free-list length (ws_ctr + CTR_DM)
   bool has_dm = false;
   uint32_t* b_keys = nullptr;                 // [n_paths] keys of the ray budget's ranking
   uint32_t* b_work = nullptr;                 // [kBudgetWords] its histograms and counts
@@ -145,7 +145,7 @@ inline uint32_t verify_block_cap(uint32_t resident) {
 }
 
 // work counter slots in ws_ctr
-enum { CTR_CONT = 0, CTR_TRACE = 1, CTR_TILE = 2, CTR_ALL = 3, CTR_LIST = 4 };
+enum { CTR_CONT = 0, CTR_TRACE = 1, CTR_ALL = 3, CTR_LIST = 4, CTR_DM = 8 };
 
 pvk::SceneView view(const pv_scene* s);
 pvk::FrameLights frame_lights(const pv_scene* s);
@@ -181,8 +181,10 @@ void launch_compact(pv_scene* s, const uint32_t* info, uint32_t n, uint32_t* lis
 // trace.cu
 // k_trace over ``list`` (nullptr: every path from its light); with an atlas,
 // every photon stored is also deposited into it (the atlas is not cleared here).
+// clear_ticket: false after launch_verify in the same call, which clears all work counters.
 void launch_trace(pv_scene* s, const pv_paths* p, const uint32_t* list, const uint32_t* count, uint64_t seed,
-                  uint32_t frame, pv_frame_stats* stats, cudaStream_t st, const pv_atlas* atlas = nullptr);
+                  uint32_t frame, pv_frame_stats* stats, cudaStream_t st, const pv_atlas* atlas = nullptr,
+                  bool clear_ticket = true);
 // Alg. 1 over the continuation list C fused with the re-trace of ``list``;
 // with an atlas, every path is also deposited (touched: verification's marks;
 // delta: the atlas holds the entry records' deposit, only listed paths change it)

@@ -55,7 +55,7 @@ void free_scene(pv_scene* s) {
                   s->r_hist, s->r_tris, s->r_local, s->r_prim, s->prim_slot, s->prim_dyn, s->prim_alb, s->prim_nrm,
                   s->xf_old, s->xf_new, s->ws_mask, s->ws_cont, s->ws_list, s->ws_touched, s->ws_tiles, s->ws_ctr, s->status, s->b_keys, s->b_work,
                   s->dm_c[0], s->dm_c[1], s->dm_c[2], s->dm_c[3],
-                  s->dm_flag, s->dm_free, s->dm_scan, s->dm_ctr};
+                  s->dm_flag, s->dm_free, s->dm_scan};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   delete s;
@@ -238,6 +238,7 @@ extern "C" int pv_build_scene(const pv_scene_desc* d, void* stream, pv_scene** o
   fail(cudaMalloc(&s->xf_new, kMaxDyn * 12 * sizeof(float)));
   fail(cudaMalloc(&s->status, sizeof(int)));
   fail(cudaMalloc(&s->ws_ctr, 16 * sizeof(uint32_t)));
+  s->dm_ctr = s->ws_ctr + pvh::CTR_DM;
   s->n_tiles = (s->n_paths_total + pvh::kTile - 1) / pvh::kTile;
   fail(cudaMalloc(&s->ws_mask, (size_t)s->n_paths_total * sizeof(uint32_t)));
   fail(cudaMalloc(&s->ws_cont, (size_t)s->n_paths_total * sizeof(uint32_t)));
@@ -254,7 +255,6 @@ extern "C" int pv_build_scene(const pv_scene_desc* d, void* stream, pv_scene** o
     fail(cudaMalloc(&s->dm_free, (size_t)s->n_paths_total * sizeof(uint32_t)));
     fail(cudaMalloc(&s->dm_scan, ((size_t)dm_max + 1 + dm_tiles(dm_max)) * sizeof(uint32_t)));
     s->dm_sums = s->dm_scan + dm_max + 1;
-    fail(cudaMalloc(&s->dm_ctr, 8 * sizeof(uint32_t)));
   }
   fail(cudaMalloc(&s->b_keys, (size_t)s->n_paths_total * sizeof(uint32_t)));
   fail(cudaMalloc(&s->b_work, pvh::kBudgetWords * sizeof(uint32_t)));

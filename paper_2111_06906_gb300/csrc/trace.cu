@@ -319,9 +319,9 @@ TraceArgs trace_args(pv_scene* s, const pv_paths* p, const uint32_t* list, const
 }  // namespace
 
 void launch_trace(pv_scene* s, const pv_paths* p, const uint32_t* list, const uint32_t* count, uint64_t seed,
-                  uint32_t frame, pv_frame_stats* stats, cudaStream_t st, const pv_atlas* atlas) {
+                  uint32_t frame, pv_frame_stats* stats, cudaStream_t st, const pv_atlas* atlas, bool clear_ticket) {
   const TraceArgs A = trace_args(s, p, list, count, seed, frame, stats);
-  cudaMemsetAsync(A.ticket, 0, sizeof(uint32_t), st);
+  if (clear_ticket) cudaMemsetAsync(A.ticket, 0, sizeof(uint32_t), st);
   if (!p->n) return;
   AtlasMap am;
   std::memset(&am, 0, sizeof am);

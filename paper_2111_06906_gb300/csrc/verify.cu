@@ -280,7 +280,7 @@ int verify_retrace(pv_scene* s, const pv_paths* paths, const pv_verify_params* p
     if (s->has_dm && (rc = pvh::dm_frame(s, paths, L, params, d_stats, st)) != PV_OK) return rc;
     pvh::launch_compact(s, paths->info, paths->n, list, count, listed, st);
     mark(3);
-    pvh::launch_trace(s, paths, list, count, params->seed, params->frame, d_stats, st);
+    pvh::launch_trace(s, paths, list, count, params->seed, params->frame, d_stats, st, nullptr, false);
     if (atlas) pvh::launch_deposit(s, paths, atlas, st);
   }
   mark(4);
