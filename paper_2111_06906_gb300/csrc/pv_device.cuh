@@ -111,6 +111,8 @@ struct DmLight {
   uint32_t dims;             // 4 rectangle, 2 point, 0 no map
   uint32_t cells;
   uint32_t n_paths;          // N: DM_T spreads N paths over the cells
+  uint32_t base, rem;        // N / cells, N mod cells
+  uint64_t inv;              // ceil(2^64 / cells): x / cells = the high word of x inv for x cells < 2^64 (0 for one cell)
   uint32_t* dmc;             // DM_C [cells]
 };
 

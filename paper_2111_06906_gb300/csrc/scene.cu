@@ -110,6 +110,9 @@ FrameLights frame_lights(const pv_scene* s) {
     D.cells = s->dm_cells[l];
     D.n_paths = s->lights_new[l].n_paths;
     D.dmc = s->dm_c[l];
+    D.base = D.cells ? D.n_paths / D.cells : 0u;
+    D.rem = D.cells ? D.n_paths % D.cells : 0u;
+    D.inv = D.cells > 1 ? ~0ull / D.cells + 1ull : 0ull;
     for (int k = 0; k < 4; ++k) D.res[k] = s->dm_res[l][k];
   }
   return L;
