@@ -115,6 +115,7 @@ __global__ void k_rs_hist(const uint64_t* keys, uint32_t n, int shift, uint32_t*
 
 // exclusive scan of m counters in place (one block of 1024 threads)
 __global__ void k_rs_scan(uint32_t* hist, uint32_t m) {
+  grid_dependency_wait();
   __shared__ uint32_t sums[1024];
   const uint32_t per = (m + blockDim.x - 1) / blockDim.x;
   const uint32_t b = threadIdx.x * per, e = min(b + per, m);
@@ -533,7 +534,7 @@ void radix_sort(uint64_t*& k0, uint32_t*& v0, uint64_t*& k1, uint32_t*& v1, uint
 
 uint32_t radix_tiles(uint32_t n) { return (n + kRsTile - 1) / kRsTile; }
 
-void exclusive_scan(uint32_t* data, uint32_t m, cudaStream_t st) { k_rs_scan<<<1, 1024, 0, st>>>(data, m); }
+void exclusive_scan(uint32_t* data, uint32_t m, cudaStream_t st) { launch_dependent(k_rs_scan, 1, 1024, 0, st, data, m); }
 
 static inline uint32_t blocks(uint32_t n, uint32_t t) { return (n + t - 1) / t; }
 

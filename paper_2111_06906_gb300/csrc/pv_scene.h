@@ -198,6 +198,24 @@ void launch_deposit(pv_scene* s, const pv_paths* p, const pv_atlas* a, cudaStrea
 // verify.cu: argument checks shared by the entry points
 int check_paths(const pv_scene* s, const pv_paths* p);
 
+// Launch a kernel that begins with pvk::grid_dependency_wait() as a programmatic
+// dependent of the kernel before it on the stream.
+template <typename... Params, typename... Args>
+inline void launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                             Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1] = {};
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
 inline int cuda_status(cudaError_t e) { return e == cudaSuccess ? PV_OK : PV_ERR_CUDA; }
 
 }  // namespace pvh

@@ -130,6 +130,7 @@ constexpr uint32_t kRowsAtOnce = 2;
 __global__ void __launch_bounds__(256) k_photon_count(Cam c, Grid g, float radius, uint32_t n, uint32_t B,
                                                       const uint32_t* info, const float4* pa, uint32_t* counts,
                                                       uint32_t* rank) {
+  grid_dependency_wait();
   const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   const uint32_t L = min(info_nseg(info[p]), B);
@@ -154,6 +155,7 @@ __global__ void __launch_bounds__(256) k_photon_count(Cam c, Grid g, float radiu
 __global__ void __launch_bounds__(256) k_photon_place(Grid g, uint32_t n, uint32_t B, const uint32_t* info,
                                                       const float* origin, const float4* pa, const float4* pb,
                                                       const uint32_t* starts, const uint32_t* rank, Photons out) {
+  grid_dependency_wait();
   const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   const uint32_t L = min(info_nseg(info[p]), B);
@@ -191,6 +193,7 @@ __global__ void __launch_bounds__(256) k_photon_place(Grid g, uint32_t n, uint32
 // Exclusive scan of m = tiles * 4096 counters: tile sums, their scan, then
 // each tile's own scan plus its offset.
 __global__ void __launch_bounds__(1024) k_tile_sums(const uint32_t* v, uint32_t* sums) {
+  grid_dependency_wait();
   __shared__ uint32_t w[32];
   const uint4 x = reinterpret_cast<const uint4*>(v)[(size_t)blockIdx.x * 1024 + threadIdx.x];
   uint32_t t = __reduce_add_sync(0xffffffffu, x.x + x.y + x.z + x.w);
@@ -203,6 +206,7 @@ __global__ void __launch_bounds__(1024) k_tile_sums(const uint32_t* v, uint32_t*
 }
 
 __global__ void __launch_bounds__(1024) k_tile_scan(uint32_t* v, const uint32_t* offs) {
+  grid_dependency_wait();
   __shared__ uint32_t w[32];
   uint4* p = reinterpret_cast<uint4*>(v) + (size_t)blockIdx.x * 1024 + threadIdx.x;
   const uint4 x = *p;
@@ -230,6 +234,35 @@ __global__ void __launch_bounds__(1024) k_tile_scan(uint32_t* v, const uint32_t*
   *p = make_uint4(base, base + x.x, base + x.x + x.y, base + x.x + x.y + x.z);
 }
 
+// Packed single-precision operations of sm_100 and later, each half rounded as
+// the scalar instruction rounds it.
+__device__ __forceinline__ unsigned long long pack2(float2 v) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(v.x), "f"(v.y));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long r) {
+  float2 v;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(v.x), "=f"(v.y) : "l"(r));
+  return v;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)), "l"(pack2(c)));
+  return unpack2(r);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+  return unpack2(r);
+}
+// (a, a) - b
+__device__ __forceinline__ float2 sub2(float a, float2 b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(make_float2(a, a))), "l"(pack2(make_float2(-b.x, -b.y))));
+  return unpack2(r);
+}
+
 // Order-preserving map of floats to integers, for warp-wide minima and maxima.
 __device__ __forceinline__ int ordered(float f) {
   const int i = __float_as_int(f);
@@ -249,23 +282,29 @@ __device__ __forceinline__ float warp_max(float f) { return unordered(__reduce_m
 // over more than kSpread cells beyond the first one (an edge in depth), the
 // warp takes them group by group.  Each warp takes every fourth 32 photons.
 //
+// The kept photons lie word by word, so that four of them are tested with packed
+// arithmetic (fma.rn.f32x2) on 16-byte reads.
+//
 // Bound by issue: on the 1M-path city at 1920 x 1080 and r = 0.3 m (2.0M
-// photons, up to a few thousand in the cells around a point) 3.9e8 warp
-// instructions at 26 of 32 lanes, 67 % of the issue slots.  There it takes
-// 0.47 ms, where a thread per pixel walking 27 hashed cells, which read each
-// photon's previous vertex from the path buffers, took 3.57 ms (1.14 ms with
-// cells sorted by row and the segment in the record: long waits on loads
-// at 12 of 32 lanes).  One warp for 8 x 4 pixels takes 0.99 ms and two 0.62:
-// neighbouring tiles in one block thrash L1 and the densest tiles finish late;
-// two pixels per lane take 0.58 ms and cells of half the radius 0.63 ms.
+// photons, up to a few thousand in the cells around a point) 3.4e8 warp
+// instructions at 25 of 32 lanes, 64 % of the issue slots.  There it takes
+// 0.43 ms (0.46 with one photon tested at a time), where a thread per pixel
+// walking 27 hashed cells, which read each photon's previous vertex from the path
+// buffers, took 3.57 ms (1.14 ms with cells sorted by row and the segment in the
+// record: long waits on loads at 12 of 32 lanes).  One photon at a time, one warp
+// for 8 x 4 pixels took 0.99 ms and two 0.62: neighbouring tiles in one block
+// thrash L1 and the densest tiles finish late; two pixels per lane took 0.58 ms
+// and cells of half the radius 0.63 ms.  Six, seven and eight blocks per SM: 0.49,
+// 0.45 and 0.43 ms.
 constexpr int kParts = 4;          // warps of a block
 constexpr int kSpread = 2;         // measured on the city: 1 0.51 ms, 2 0.47, 3 0.51, 4 0.60
 
-__global__ void __launch_bounds__(32 * kParts) k_gather(SceneView sv, Cam c, Grid g, float radius, const GPixel* gb,
+__global__ void __launch_bounds__(32 * kParts, 8) k_gather(SceneView sv, Cam c, Grid g, float radius, const GPixel* gb,
                                                         const uint32_t* starts, Photons ph, float* image) {
+  grid_dependency_wait();
   constexpr int kBuf = 64;         // photons kept before they are tested: fewer than 32 left over plus 32 new
-  __shared__ float4 s_x[kParts][kBuf], s_d[kParts][kBuf];
-  __shared__ float s_e[kParts][kBuf];
+  enum { kX, kY, kZ, kDx, kDy, kDz, kEx, kEy, kEz, kWords };
+  __shared__ __align__(16) float s_ph[kParts][kWords][kBuf];
   __shared__ float s_acc[kParts][3][32];
   const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
   const uint32_t tiles_x = (c.W + 7u) / 8u;
@@ -273,7 +312,7 @@ __global__ void __launch_bounds__(32 * kParts) k_gather(SceneView sv, Cam c, Gri
   const bool inside = pi < c.W && pj < c.H;
   const float inv_r2 = 1.0f / (radius * radius);
   const float away = 3.0e18f;      // beyond every photon's radius
-  float3 P = make_float3(0.f, 0.f, 0.f), nrm = P, acc = P, Q = P, N = P;   // Q, N: P and nrm within the group
+  float3 P = make_float3(0.f, 0.f, 0.f), nrm = P, Q = P, N = P;   // Q, N: P and nrm within the group
   int prim = -1;
   if (inside) {
     const GPixel* q = gb + ((size_t)pj * c.W + pi);
@@ -287,29 +326,50 @@ __global__ void __launch_bounds__(32 * kParts) k_gather(SceneView sv, Cam c, Gri
   const int3 cell = grid_cell(g, P);
   bool todo = prim >= 0;
   uint32_t kept = 0;               // photons in the buffer
+  float2 sum[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+  float(&ph_s)[kWords][kBuf] = s_ph[part];
+  bool odd = false;                // some photon of the buffer has an energy that is not finite
   auto test_kept = [&]() {
     const uint32_t n4 = (kept + 3u) & ~3u;
-    if (kept + lane < n4) {        // filled up with photons that light no side
-      s_x[part][kept + lane] = make_float4(-away, -away, -away, 0.f);
-      s_d[part][kept + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    if (kept + lane < n4)              // filled up with photons that light no side
+#pragma unroll
+      for (int k = 0; k < kWords; ++k) ph_s[k][kept + lane] = 0.f;
     __syncwarp();
     for (uint32_t i = 0; i < n4; i += 4) {
+      const auto word = [&](int k) { return *reinterpret_cast<const float4*>(&ph_s[k][i]); };
+      const float4 x = word(kX), y = word(kY), z = word(kZ);
+      float2 w[2];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const float4 x = s_x[part][i + u];
-        const float ax = Q.x - x.x, ay = Q.y - x.y, az = Q.z - x.z;
-        const float w = fmaf(-inv_r2, fmaf(az, az, fmaf(ay, ay, ax * ax)), 1.0f);
-        if (!(w > 0.0f)) continue;
-        const float4 d = s_d[part][i + u];
-        if (!(N.x * d.x + N.y * d.y + N.z * d.z < 0.0f)) continue;       // arrives on the visible side
-        acc.x = fmaf(x.w, w, acc.x);
-        acc.y = fmaf(d.w, w, acc.y);
-        acc.z = fmaf(s_e[part][i + u], w, acc.z);
+      for (int h = 0; h < 2; ++h) {
+        const float2 dx = sub2(Q.x, h ? make_float2(x.z, x.w) : make_float2(x.x, x.y));
+        const float2 dy = sub2(Q.y, h ? make_float2(y.z, y.w) : make_float2(y.x, y.y));
+        const float2 dz = sub2(Q.z, h ? make_float2(z.z, z.w) : make_float2(z.x, z.y));
+        w[h] = fma2(make_float2(-inv_r2, -inv_r2), fma2(dz, dz, fma2(dy, dy, mul2(dx, dx))), make_float2(1.f, 1.f));
+      }
+      if (!(fmaxf(fmaxf(w[0].x, w[0].y), fmaxf(w[1].x, w[1].y)) > 0.0f)) continue;
+      const float4 sx = word(kDx), sy = word(kDy), sz = word(kDz), ex = word(kEx), ey = word(kEy), ez = word(kEz);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        // a photon counts within the radius, and where it arrives on the visible side
+        const float2 side = fma2(make_float2(N.x, N.x), h ? make_float2(sx.z, sx.w) : make_float2(sx.x, sx.y),
+                                 fma2(make_float2(N.y, N.y), h ? make_float2(sy.z, sy.w) : make_float2(sy.x, sy.y),
+                                      mul2(make_float2(N.z, N.z), h ? make_float2(sz.z, sz.w) : make_float2(sz.x, sz.y))));
+        const float2 v = make_float2(side.x < 0.0f ? fmaxf(w[h].x, 0.0f) : 0.0f, side.y < 0.0f ? fmaxf(w[h].y, 0.0f) : 0.0f);
+        float2 a = h ? make_float2(ex.z, ex.w) : make_float2(ex.x, ex.y);
+        float2 b = h ? make_float2(ey.z, ey.w) : make_float2(ey.x, ey.y);
+        float2 c = h ? make_float2(ez.z, ez.w) : make_float2(ez.x, ez.y);
+        if (odd) {                     // infinity times a weight of 0 would not be nothing
+          if (!(v.x > 0.0f)) a.x = b.x = c.x = 0.0f;
+          if (!(v.y > 0.0f)) a.y = b.y = c.y = 0.0f;
+        }
+        sum[0] = fma2(a, v, sum[0]);
+        sum[1] = fma2(b, v, sum[1]);
+        sum[2] = fma2(c, v, sum[2]);
       }
     }
     __syncwarp();
     kept = 0;
+    odd = false;
   };
   for (;;) {
     // the group: the first pixel left and those within kSpread cells of it
@@ -372,12 +432,23 @@ __global__ void __launch_bounds__(32 * kParts) k_gather(SceneView sv, Cam c, Gri
           keep = x.x >= bl.x && x.x <= bh.x && x.y >= bl.y && x.y <= bh.y && x.z >= bl.z && x.z <= bh.z;
         }
         const unsigned m = __ballot_sync(0xffffffffu, keep);
+        bool finite = true;
         if (keep) {
           const uint32_t at = kept + __popc(m & ((1u << lane) - 1u));
-          s_x[part][at] = x;
-          s_d[part][at] = __ldg(ph.xd + 2 * (size_t)i + 1);
-          s_e[part][at] = __ldg(ph.e + i);
+          const float4 d = __ldg(ph.xd + 2 * (size_t)i + 1);
+          ph_s[kX][at] = x.x;
+          ph_s[kY][at] = x.y;
+          ph_s[kZ][at] = x.z;
+          ph_s[kDx][at] = d.x;
+          ph_s[kDy][at] = d.y;
+          ph_s[kDz][at] = d.z;
+          ph_s[kEx][at] = x.w;
+          ph_s[kEy][at] = d.w;
+          const float ez = __ldg(ph.e + i);
+          ph_s[kEz][at] = ez;
+          finite = isfinite(x.w) && isfinite(d.w) && isfinite(ez);
         }
+        odd |= !__all_sync(0xffffffffu, finite);
         kept += __popc(m);
         if (kept > 32u) test_kept();
       }
@@ -385,6 +456,7 @@ __global__ void __launch_bounds__(32 * kParts) k_gather(SceneView sv, Cam c, Gri
     if (kept) test_kept();
   }
   // the parts of a pixel's sum meet in shared memory
+  float3 acc = make_float3(sum[0].x + sum[0].y, sum[1].x + sum[1].y, sum[2].x + sum[2].y);
   s_acc[part][0][lane] = acc.x;
   s_acc[part][1][lane] = acc.y;
   s_acc[part][2][lane] = acc.z;
@@ -515,17 +587,21 @@ extern "C" int pv_splat(pv_scene* s, const pv_paths* paths, const pv_camera* cam
   uint32_t* rank = reinterpret_cast<uint32_t*>(w + lay.rank);
   const Photons ph = {reinterpret_cast<float4*>(w + lay.xd), reinterpret_cast<float*>(w + lay.e)};
   const pvk::SceneView sv = pvh::view(s);
+  // after the first, the kernels are dependent launches: six short kernels had a launch's latency between them
   const uint32_t tiles = SplatLayout::tiles(g.cells);
   PV_CHECK(cudaMemsetAsync(counts, 0, (size_t)tiles * 4096 * sizeof(uint32_t), st));
   k_gbuffer<<<((c.W + 15) / 16) * ((c.H + 15) / 16), 256, 0, st>>>(sv, c, gbuf);
   const uint32_t n = paths->n;
   const float4* pa = reinterpret_cast<const float4*>(paths->pa);
   const float4* pb = reinterpret_cast<const float4*>(paths->pb);
-  if (n) k_photon_count<<<(n + 255) / 256, 256, 0, st>>>(c, g, radius, n, s->B, paths->info, pa, counts, rank);
-  k_tile_sums<<<tiles, 1024, 0, st>>>(counts, sums);
+  if (n) pvh::launch_dependent(k_photon_count, (n + 255) / 256, 256, 0, st, c, g, radius, n, s->B, paths->info, pa, counts, rank);
+  pvh::launch_dependent(k_tile_sums, tiles, 1024, 0, st, counts, sums);
   pvh::exclusive_scan(sums, tiles, st);
-  k_tile_scan<<<tiles, 1024, 0, st>>>(counts, sums);
-  if (n) k_photon_place<<<(n + 255) / 256, 256, 0, st>>>(g, n, s->B, paths->info, paths->origin, pa, pb, counts, rank, ph);
-  k_gather<<<((c.W + 7) / 8) * ((c.H + 3) / 4), 32 * kParts, 0, st>>>(sv, c, g, radius, gbuf, counts, ph, d_image);
+  pvh::launch_dependent(k_tile_scan, tiles, 1024, 0, st, counts, sums);
+  if (n)
+    pvh::launch_dependent(k_photon_place, (n + 255) / 256, 256, 0, st, g, n, s->B, paths->info, paths->origin, pa, pb, counts,
+                          rank, ph);
+  pvh::launch_dependent(k_gather, ((c.W + 7) / 8) * ((c.H + 3) / 4), 32 * kParts, 0, st, sv, c, g, radius, gbuf, counts, ph,
+                        d_image);
   return pvh::cuda_status(cudaGetLastError());
 }

@@ -56,3 +56,25 @@ def test_splat_grid_matches_oracle(name, size):
     assert (err <= 1e-4 * want.max() + 1e-4 * np.abs(want)[~amb]).all(), (float(err.max()), float(want.max()))
     assert pv.pv_read_device_status(h) == 0
     pv.pv_destroy_scene(h)
+
+
+def test_photons_out_of_reach_add_nothing_whatever_their_energy():
+    """A photon with infinite energy shows where it is, and only there: the packed
+    sums must not pick up infinity times a weight of zero."""
+    import torch
+    sc = scenes.tiny_box(n_paths=2000)
+    h = gu.lib_scene(sc)
+    P = pv.Paths.allocate(sc.n_paths, sc.max_bounces)
+    pv.pv_trace_all(h, P, 4, 1)
+    cam = pv.PvCamera.make(*BOX, math.radians(25.0), 64, 48)
+    work = torch.empty(pv.pv_splat_workspace_bytes(h, 64, 48), dtype=torch.uint8, device="cuda")
+    plain, odd = (torch.zeros(48, 64, 3, device="cuda") for _ in range(2))
+    pv.pv_splat(h, P, cam, 0.2, plain, work)
+    on_back = torch.nonzero((P.pa[0, :, 2] < -0.99) & (P.pa[0, :, 1] > 0.9)).flatten()
+    P.pb[0, on_back[0], 0] = float("inf")
+    pv.pv_splat(h, P, cam, 0.2, odd, work)
+    assert not bool(torch.isnan(odd).any())
+    bright = torch.isinf(odd[..., 0])
+    assert 0 < int(bright.sum()) < bright.numel() // 2
+    assert torch.allclose(odd[~bright], plain[~bright], rtol=1e-5, atol=1e-5 * float(plain.max()))
+    pv.pv_destroy_scene(h)
