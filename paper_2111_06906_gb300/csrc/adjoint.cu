@@ -270,6 +270,7 @@ __device__ __forceinline__ uint32_t tap_store(TapSmem& T, int lane, const ModelA
 // alignment, 217 us with the photons dealt out a lane each, 141 us with four lanes
 // a photon (16 lanes: 142 us, a quarter more instructions).
 __global__ void __launch_bounds__(128) k_model_deposit(SceneView sv, FrameLights L, ModelArgs A, float* atlas) {
+  grid_dependency_wait();
   __shared__ float s_th[kMaxTheta];
   extern __shared__ __align__(16) unsigned char s_photons[];
   stage_theta(A, s_th);
@@ -359,6 +360,7 @@ __device__ __forceinline__ void shift_down(const float (&w)[16], uint32_t o, flo
 // L1 they spend on summing up and on shared memory.)
 __global__ void __launch_bounds__(128) k_adjoint(SceneView sv, FrameLights L, ModelArgs A, const float* G,
                                                  float* dtheta, float* score) {
+  grid_dependency_wait();
   __shared__ float s_th[kMaxTheta];
   __shared__ float s_acc[kMaxTheta];
   extern __shared__ __align__(16) unsigned char s_photons[];
@@ -545,6 +547,7 @@ template <int kLevel>
 __global__ void __launch_bounds__(kBudgetThreads) k_budget_hist(const uint32_t* list, const uint32_t* count,
                                                                 const float* score, uint32_t n, uint32_t budget,
                                                                 uint32_t* keys, uint32_t* marks, BudgetWork* W) {
+  grid_dependency_wait();
   __shared__ uint32_t s_hist[kBudgetBins];
   __shared__ uint32_t sh[10];
   constexpr uint32_t kShift = kLevel == 0 ? 20u : kLevel == 1 ? 9u : 0u;      // lowest bit of this level
@@ -592,6 +595,7 @@ __global__ void __launch_bounds__(kBudgetThreads) k_budget_hist(const uint32_t* 
 // The last key T, and the paths of key T in every tile of the list (a block per tile).
 __global__ void __launch_bounds__(kBudgetThreads) k_budget_ties(const uint32_t* count, uint32_t n, uint32_t tile,
                                                                 const uint32_t* keys, BudgetWork* W) {
+  grid_dependency_wait();
   __shared__ uint32_t sh[10];
   BudgetState st = W->state[1];
   if (st.want) st.prefix = st.prefix * 512u + budget_pick(W->hist[2], st.want, sh);
@@ -616,6 +620,7 @@ __global__ void __launch_bounds__(kBudgetThreads) k_budget_ties(const uint32_t* 
 __global__ void __launch_bounds__(kBudgetThreads) k_budget_mark(const uint32_t* list, const uint32_t* count, uint32_t n,
                                                                 uint32_t tile, const uint32_t* keys,
                                                                 const BudgetWork* W, uint32_t* marks) {
+  grid_dependency_wait();
   __shared__ uint32_t sh[kBudgetThreads / 32u + 1u];
   const BudgetState st = W->state[2];
   if (!st.want) return;
@@ -700,9 +705,9 @@ extern "C" int pv_model_deposit(pv_scene* s, const pv_paths* paths, const float*
   // 128 threads a block at most 40 KB of shared memory (15 photons a path)
   constexpr uint32_t kThreads = 128;
   if (paths->n)
-    k_model_deposit<<<(paths->n + kThreads - 1) / kThreads, kThreads,
-                      kThreads / 32 * warp_smem_bytes<2>(s->B, sizeof(TapSmem)), st>>>(pvh::view(s), pvh::frame_lights(s), A,
-                                                                                     d_atlas);
+    pvh::launch_dependent(k_model_deposit, (paths->n + kThreads - 1) / kThreads, kThreads,
+                          kThreads / 32 * warp_smem_bytes<2>(s->B, sizeof(TapSmem)), st, pvh::view(s), pvh::frame_lights(s), A,
+                          d_atlas);
   return pvh::cuda_status(cudaGetLastError());
 }
 
@@ -718,8 +723,9 @@ extern "C" int pv_adjoint_deposit(pv_scene* s, const pv_paths* paths, const floa
   s->last_stream = st;
   constexpr uint32_t kThreads = 128;
   if (paths->n)
-    k_adjoint<<<(paths->n + kThreads - 1) / kThreads, kThreads, kThreads / 32 * warp_smem_bytes<3>(s->B, 0), st>>>(
-        pvh::view(s), pvh::frame_lights(s), A, d_grad_atlas, d_dtheta, d_score);
+    pvh::launch_dependent(k_adjoint, (paths->n + kThreads - 1) / kThreads, kThreads,
+                          kThreads / 32 * warp_smem_bytes<3>(s->B, 0), st, pvh::view(s), pvh::frame_lights(s), A, d_grad_atlas,
+                          d_dtheta, d_score);
   return pvh::cuda_status(cudaGetLastError());
 }
 
@@ -732,16 +738,19 @@ extern "C" int pv_budget_list(pv_scene* s, const uint32_t* d_list, const uint32_
   if (n == 0) return pvh::cuda_status(cudaMemsetAsync(d_out_count, 0, sizeof(uint32_t), st));
   BudgetWork* W = reinterpret_cast<BudgetWork*>(s->b_work);
   uint32_t* const keys = s->b_keys;
-  PV_CHECK(cudaMemsetAsync(W, 0, sizeof W->hist, st));
+  pvh::ClearSet C;
+  C.add(W, sizeof W->hist / sizeof(uint32_t));
+  C.add(s->ws_tiles, pvh::compact_words(n));
+  pvh::launch_clear(s, C, st);
   const uint32_t blocks = std::min((n + kBudgetStep - 1) / kBudgetStep, 4u * (uint32_t)s->num_sms);
-  k_budget_hist<0><<<blocks, kBudgetThreads, 0, st>>>(d_list, d_count, d_score, n, budget, keys, s->ws_mask, W);
-  k_budget_hist<1><<<blocks, kBudgetThreads, 0, st>>>(d_list, d_count, d_score, n, budget, keys, s->ws_mask, W);
-  k_budget_hist<2><<<blocks, kBudgetThreads, 0, st>>>(d_list, d_count, d_score, n, budget, keys, s->ws_mask, W);
+  pvh::launch_dependent(k_budget_hist<0>, blocks, kBudgetThreads, 0, st, d_list, d_count, d_score, n, budget, keys, s->ws_mask, W);
+  pvh::launch_dependent(k_budget_hist<1>, blocks, kBudgetThreads, 0, st, d_list, d_count, d_score, n, budget, keys, s->ws_mask, W);
+  pvh::launch_dependent(k_budget_hist<2>, blocks, kBudgetThreads, 0, st, d_list, d_count, d_score, n, budget, keys, s->ws_mask, W);
   // tiles of whole steps, at most kBudgetTiles of them
   const uint32_t tile = std::max<uint32_t>((n / pvh::kBudgetTiles / kBudgetStep + 1u) * kBudgetStep, kBudgetStep);
   const uint32_t tiles = (n + tile - 1) / tile;
-  k_budget_ties<<<tiles, kBudgetThreads, 0, st>>>(d_count, n, tile, keys, W);
-  k_budget_mark<<<tiles, kBudgetThreads, 0, st>>>(d_list, d_count, n, tile, keys, W, s->ws_mask);
-  pvh::launch_compact(s, s->ws_mask, n, d_out, d_out_count, nullptr, st);
+  pvh::launch_dependent(k_budget_ties, tiles, kBudgetThreads, 0, st, d_count, n, tile, keys, W);
+  pvh::launch_dependent(k_budget_mark, tiles, kBudgetThreads, 0, st, d_list, d_count, n, tile, keys, W, s->ws_mask);
+  pvh::launch_compact(s, s->ws_mask, n, d_out, d_out_count, nullptr, st, 0, false);
   return pvh::cuda_status(cudaGetLastError());
 }

@@ -482,6 +482,7 @@ __device__ __forceinline__ void refit_finish(const XformParams& P, const RefitAr
 // slots of the wide nodes above the triangles).
 __global__ void __launch_bounds__(256, PV_REFIT_MIN_BLOCKS) k_refit_wide(XformParams P, RefitArgs R, PairArgs Q,
                                                                           TopArgs T, uint32_t blocks_tri) {
+  grid_dependency_wait();
   if (blockIdx.x < blocks_tri) {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t s = i < R.n ? R.tri_slot[i] : 0u;
@@ -497,6 +498,7 @@ __global__ void __launch_bounds__(256, PV_REFIT_MIN_BLOCKS) k_refit_wide(XformPa
 // The same with the climb of refit_tri, one thread per dynamic triangle (for
 // a scene built with PV_BUILD_REFIT_CLIMB, or without a pair table).
 __global__ void __launch_bounds__(256) k_refit_climb(XformParams P, RefitArgs R, TopArgs T) {
+  grid_dependency_wait();
   const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
   const uint32_t s = i < R.n ? R.tri_slot[i] : 0u;
   const bool mv = i < R.n && ((P.moved >> s) & 1ull);
@@ -508,6 +510,7 @@ __global__ void __launch_bounds__(256) k_refit_climb(XformParams P, RefitArgs R,
 // and the moved objects' groups.  One block of 32 threads.
 __global__ void k_frame_top(XformParams P, DynObj* objs, float* xf_old, float* xf_new, int* obox, WNode* wnodes,
                             const Tri* tris, int top_off, int static_root, int* root_out, MovedGroups* groups) {
+  grid_dependency_wait();
   pose_bookkeeping(P.xf, P.moved, P.n_dyn, objs, xf_old, xf_new, obox);
   if (!P.moved) return;
   build_top_and_groups(wnodes, tris, top_off, static_root, objs, (int)P.n_dyn, root_out, P.moved, groups);
@@ -1082,14 +1085,14 @@ void launch_update_dynamic(pv_scene* s, cudaStream_t st) {
           Q.count = s->pair_count;
           Q.n_pairs = s->n_pairs;
           const uint32_t bt = blocks(n, 256);
-          k_refit_wide<<<bt + blocks(s->n_pairs, 256), 256, 0, st>>>(P, R, Q, T, bt);
+          launch_dependent(k_refit_wide, bt + blocks(s->n_pairs, 256), 256, 0, st, P, R, Q, T, bt);
         } else {
-          k_refit_climb<<<blocks(n, 256), 256, 0, st>>>(P, R, T);
+          launch_dependent(k_refit_climb, blocks(n, 256), 256, 0, st, P, R, T);
         }
         return;
       }
-      k_frame_top<<<1, 32, 0, st>>>(P, s->objs, s->xf_old, s->xf_new, s->obox, s->wnodes, s->tris, (int)s->w_top_off,
-                                    s->s_wroot, s->root, s->groups);
+      launch_dependent(k_frame_top, 1, 32, 0, st, P, s->objs, s->xf_old, s->xf_new, s->obox, s->wnodes, s->tris,
+                       (int)s->w_top_off, s->s_wroot, s->root, s->groups);
       return;
     }
     k_update_objects<<<s->n_dyn, 256, 0, st>>>(P, s->d_local, s->d_tri_prim, dtris, s->objs, s->xf_old, s->xf_new);

@@ -1,4 +1,5 @@
 // Compaction entry points (the kernel body is in compact_core.cuh).
+#include <algorithm>
 #include <mutex>
 
 #include "compact_core.cuh"
@@ -13,28 +14,53 @@ __global__ void __launch_bounds__(pvh::kCompactThreads) k_compact(const uint32_t
                                                                     uint32_t* count, unsigned long long* tiles,
                                                                     uint32_t* ticket, uint32_t n_tiles, int* status,
                                                                     uint32_t* stat_listed, uint32_t* failed) {
+  grid_dependency_wait();
   __shared__ CompactSmem sm;
   if (threadIdx.x == 0) sm.tile = atomicAdd(ticket, 1u);
   __syncthreads();
   compact_tile(info, n, list, count, tiles, sm.tile, n_tiles, status, stat_listed, sm, failed);
 }
 
+// Zero the words of a few arrays of the library's own.  One launch per frame
+// (2 to 3 us), where each memset was a node of its own that the next kernel had to
+// wait out in full; an atlas of the caller's keeps its cudaMemsetAsync, which
+// refuses a pointer that is not the device's.
+__global__ void __launch_bounds__(256) k_clear(pvh::ClearSet C) {
+  grid_dependency_wait();
+  for (uint32_t r = 0; r < C.n; ++r)
+    for (uint32_t i = blockIdx.x * 256u + threadIdx.x; i < C.words[r]; i += gridDim.x * 256u) C.p[r][i] = 0u;
+}
+
 }  // namespace
 
 namespace pvh {
 
+void launch_clear(const pv_scene* s, const ClearSet& C, cudaStream_t st) {
+  uint32_t most = 1;
+  for (uint32_t r = 0; r < C.n; ++r) most = std::max(most, C.words[r]);
+  launch_dependent(k_clear, std::min<uint32_t>((most + 1023u) / 1024u, 4u * (uint32_t)s->num_sms), 256, 0, st, C);
+}
+
+// words of the tile states and ticket for n paths
+uint32_t compact_words(uint32_t n) { return 2u * ((n + kTile - 1) / kTile + 1u); }
+
 void launch_compact(pv_scene* s, const uint32_t* info, uint32_t n, uint32_t* list, uint32_t* count,
-                    uint32_t* stats_listed, cudaStream_t st) {
+                    uint32_t* stats_listed, cudaStream_t st, int states, bool clear) {
   if (n == 0) {
     cudaMemsetAsync(count, 0, sizeof(uint32_t), st);
     return;
   }
   const uint32_t n_tiles = (n + kTile - 1) / kTile;
+  uint64_t* const tiles = s->ws_tiles + (size_t)states * (s->n_tiles + 1);
   // the tile states and, in the word behind them, the tile ticket
-  cudaMemsetAsync(s->ws_tiles, 0, ((size_t)n_tiles + 1) * sizeof(uint64_t), st);
-  k_compact<<<n_tiles, kCompactThreads, 0, st>>>(info, n, list, count, reinterpret_cast<unsigned long long*>(s->ws_tiles),
-                                                 reinterpret_cast<uint32_t*>(s->ws_tiles + n_tiles), n_tiles, s->status,
-                                                 stats_listed, nullptr);
+  if (clear) {
+    ClearSet C;
+    C.add(tiles, compact_words(n));
+    launch_clear(s, C, st);
+  }
+  launch_dependent(k_compact, n_tiles, kCompactThreads, 0, st, info, n, list, count,
+                   reinterpret_cast<unsigned long long*>(tiles), reinterpret_cast<uint32_t*>(tiles + n_tiles), n_tiles,
+                   s->status, stats_listed, nullptr);
 }
 
 }  // namespace pvh

@@ -9,6 +9,7 @@ namespace {
 
 __global__ void __launch_bounds__(256) k_deposit(uint32_t n, uint32_t B, const uint32_t* info, const float4* pa,
                                                  const float4* pb, pv_atlas at) {
+  grid_dependency_wait();
   const AtlasMap am = atlas_map(at);
   // whole warps loop, so that the photons of each round's 32 paths are dealt out over the lanes
   for (uint32_t b = blockIdx.x * blockDim.x; b < n; b += gridDim.x * blockDim.x) {
@@ -31,8 +32,8 @@ void launch_deposit(pv_scene* s, const pv_paths* p, const pv_atlas* a, cudaStrea
   const uint32_t n = p->n;
   if (!n) return;
   const uint32_t blocks = (uint32_t)s->num_sms * 8u;
-  k_deposit<<<blocks, 256, 0, st>>>(n, s->B, p->info, reinterpret_cast<const float4*>(p->pa),
-                                    reinterpret_cast<const float4*>(p->pb), *a);
+  launch_dependent(k_deposit, blocks, 256, 0, st, n, s->B, p->info, reinterpret_cast<const float4*>(p->pa),
+                   reinterpret_cast<const float4*>(p->pb), *a);
 }
 
 }  // namespace pvh

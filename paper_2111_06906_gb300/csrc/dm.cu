@@ -24,6 +24,7 @@ __global__ void k_dm_reset(DmLight D) {
 // Pass 1 (dm_prune_path), flag[p] = 1 for a pruned path.
 __global__ void __launch_bounds__(256) k_dm_prune(FrameLights L, uint32_t n, uint32_t* info, uint32_t* flag,
                                                   uint64_t seed, uint32_t frame, pv_frame_stats* stats) {
+  grid_dependency_wait();
   __shared__ uint32_t s_red[32];
   const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
   uint32_t pruned = 0;
@@ -41,16 +42,19 @@ __global__ void __launch_bounds__(256) k_dm_prune(FrameLights L, uint32_t n, uin
 // compaction) and counted.
 __global__ void __launch_bounds__(256) k_dm_commit(FrameLights L, uint32_t n, const uint32_t* info, uint32_t* flag,
                                                    uint32_t* free_count) {
+  grid_dependency_wait();
   __shared__ uint32_t s_free[PV_MAX_LIGHTS];
   dm_commit_block(L, blockIdx.x * blockDim.x + threadIdx.x, n, info, flag, free_count, s_free);
 }
 
 __global__ void __launch_bounds__(kDmThreads) k_dm_deficit(DmLight D, uint32_t* def, uint32_t* sums) {
+  grid_dependency_wait();
   __shared__ uint32_t sh[kDmThreads / 32];
   dm_deficit_tile(D, blockIdx.x, def, sums, sh);
 }
 
 __global__ void __launch_bounds__(kDmThreads) k_dm_prefix(uint32_t cells, uint32_t* def, const uint32_t* sums) {
+  grid_dependency_wait();
   __shared__ uint32_t sh[64];
   dm_prefix_tile(cells, blockIdx.x, def, sums, sh);
 }
@@ -60,6 +64,7 @@ __global__ void __launch_bounds__(kDmThreads) k_dm_prefix(uint32_t cells, uint32
 __global__ void __launch_bounds__(256) k_dm_fill(FrameLights L, uint32_t l, const uint32_t* free_list,
                                                  const uint32_t* free_count, const uint32_t* pre, uint32_t* info,
                                                  pv_frame_stats* stats) {
+  grid_dependency_wait();
   __shared__ uint32_t s_red[32];
   const DmLight& D = L.dm[l];
   const uint32_t F = free_count[l];
@@ -92,17 +97,17 @@ int dm_frame(pv_scene* s, const pv_paths* p, const FrameLights& L, const pv_veri
     if (L.dm[l].dims && ((L.moved_mask >> l) & 1u)) moved |= 1u << l;
   if (!moved || p->n == 0) return PV_OK;
   const uint32_t n = p->n, blocks = (n + 255) / 256;
-  // dm_ctr was cleared with the other work counters before verification
-  k_dm_prune<<<blocks, 256, 0, st>>>(L, n, p->info, s->dm_flag, prm->seed, prm->frame, stats);
-  k_dm_commit<<<blocks, 256, 0, st>>>(L, n, p->info, s->dm_flag, s->dm_ctr);
-  launch_compact(s, s->dm_flag, n, s->dm_free, s->dm_ctr + 4, nullptr, st);
+  // dm_ctr and the tile states were cleared with the other work counters before verification
+  launch_dependent(k_dm_prune, blocks, 256, 0, st, L, n, p->info, s->dm_flag, prm->seed, prm->frame, stats);
+  launch_dependent(k_dm_commit, blocks, 256, 0, st, L, n, p->info, s->dm_flag, s->dm_ctr);
+  launch_compact(s, s->dm_flag, n, s->dm_free, s->dm_ctr + 4, nullptr, st, 1, false);
   for (uint32_t l = 0; l < s->n_lights; ++l) {
     if (!((moved >> l) & 1u)) continue;
     const DmLight& D = L.dm[l];
-    k_dm_deficit<<<dm_tiles(D.cells), kDmThreads, 0, st>>>(D, s->dm_scan, s->dm_sums);
-    k_dm_prefix<<<dm_tiles(D.cells), kDmThreads, 0, st>>>(D.cells, s->dm_scan, s->dm_sums);
+    launch_dependent(k_dm_deficit, dm_tiles(D.cells), kDmThreads, 0, st, D, s->dm_scan, s->dm_sums);
+    launch_dependent(k_dm_prefix, dm_tiles(D.cells), kDmThreads, 0, st, D.cells, s->dm_scan, s->dm_sums);
     const uint32_t fb = std::min<uint32_t>((s->lights_new[l].n_paths + 255) / 256, 8u * (uint32_t)s->num_sms);
-    k_dm_fill<<<std::max<uint32_t>(fb, 1u), 256, 0, st>>>(L, l, s->dm_free, s->dm_ctr, s->dm_scan, p->info, stats);
+    launch_dependent(k_dm_fill, std::max<uint32_t>(fb, 1u), 256, 0, st, L, l, s->dm_free, s->dm_ctr, s->dm_scan, p->info, stats);
   }
   return cuda_status(cudaGetLastError());
 }

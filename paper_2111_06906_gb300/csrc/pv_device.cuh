@@ -651,10 +651,8 @@ __device__ __forceinline__ uint32_t lanes_at_work(uint32_t items, uint32_t warps
 // Programmatic dependent launch (sm_90 and later).  A kernel launched with
 // programmatic stream serialisation waits in grid_dependency_wait() until the
 // kernel before it has completed and its memory operations are visible; for
-// an ordinary launch the wait returns at once.  launch_dependents() lets the
-// next such kernel be scheduled once every block of this one has issued it.
+// an ordinary launch the wait returns at once.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" :::); }
 
 // Warp-aggregated add of ``v`` to a device counter (the calling lanes only).
 __device__ __forceinline__ void warp_add(uint32_t* ctr, uint32_t v) {

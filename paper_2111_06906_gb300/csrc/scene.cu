@@ -247,7 +247,7 @@ extern "C" int pv_build_scene(const pv_scene_desc* d, void* stream, pv_scene** o
   fail(cudaMalloc(&s->ws_cont, (size_t)s->n_paths_total * sizeof(uint32_t)));
   fail(cudaMalloc(&s->ws_list, (size_t)s->n_paths_total * sizeof(uint32_t)));
   fail(cudaMalloc(&s->ws_touched, (size_t)s->n_paths_total));
-  fail(cudaMalloc(&s->ws_tiles, (size_t)(s->n_tiles + 1) * sizeof(uint64_t)));
+  fail(cudaMalloc(&s->ws_tiles, 2 * (size_t)(s->n_tiles + 1) * sizeof(uint64_t)));
   for (uint32_t l = 0; l < PV_MAX_LIGHTS; ++l)
     if (s->dm_cells[l]) {
       fail(cudaMalloc(&s->dm_c[l], (size_t)s->dm_cells[l] * sizeof(uint32_t)));

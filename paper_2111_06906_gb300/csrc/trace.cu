@@ -61,6 +61,7 @@ constexpr int kMaxSteps = PV_TRACE_MAX_STEPS;
 template <bool kDep>
 __global__ void __launch_bounds__(pvh::kTraceThreads, kDep ? PV_TRACE_DEP_MIN_BLOCKS : PV_TRACE_MIN_BLOCKS)
     k_trace(SceneView sv, FrameLights L, TraceArgs A, AtlasMap am) {
+  grid_dependency_wait();
   __shared__ uint32_t s_red[32 * 2];
   __shared__ unsigned long long s_red64[32];
   const int root = *sv.root;
@@ -147,11 +148,6 @@ __device__ __forceinline__ void cont_flush(ContCounters& cc, uint32_t* s_cnt) {
 }
 
 // kDep: 0 no deposit, 1 deposit into a cleared atlas, 2 carried atlas (delta).
-//
-// Launched as a programmatic dependent of k_verify (PV_CONT_TRACE_PDL), its
-// blocks may be placed on the SMs while k_verify's last blocks run, and wait
-// below until k_verify has finished and its writes are visible; for the
-// default ordinary launch the wait returns at once.
 template <int kDep>
 __global__ void __launch_bounds__(pvh::kTraceThreads, PV_CONT_TRACE_MIN_BLOCKS)
     k_cont_trace(SceneView sv, FrameLights L, TraceArgs A, ContArgs C, DepositArgs D) {
@@ -321,8 +317,12 @@ TraceArgs trace_args(pv_scene* s, const pv_paths* p, const uint32_t* list, const
 void launch_trace(pv_scene* s, const pv_paths* p, const uint32_t* list, const uint32_t* count, uint64_t seed,
                   uint32_t frame, pv_frame_stats* stats, cudaStream_t st, const pv_atlas* atlas, bool clear_ticket) {
   const TraceArgs A = trace_args(s, p, list, count, seed, frame, stats);
-  if (clear_ticket) cudaMemsetAsync(A.ticket, 0, sizeof(uint32_t), st);
   if (!p->n) return;
+  if (clear_ticket) {
+    ClearSet C;
+    C.add(A.ticket, 1);
+    launch_clear(s, C, st);
+  }
   AtlasMap am;
   std::memset(&am, 0, sizeof am);
   if (atlas) {
@@ -331,36 +331,11 @@ void launch_trace(pv_scene* s, const pv_paths* p, const uint32_t* list, const ui
     am.sx = (float)atlas->width / (atlas->x1 - atlas->x0);
     am.sz = (float)atlas->height / (atlas->z1 - atlas->z0);
     if (!s->trace_dep_blocks) s->trace_dep_blocks = persistent_blocks(s, k_trace<true>);
-    k_trace<true><<<blocks_for(s->trace_dep_blocks, p->n), kTraceThreads, 0, st>>>(view(s), frame_lights(s), A, am);
+    launch_dependent(k_trace<true>, blocks_for(s->trace_dep_blocks, p->n), kTraceThreads, 0, st, view(s), frame_lights(s), A, am);
   } else {
     if (!s->trace_blocks) s->trace_blocks = persistent_blocks(s, k_trace<false>);
-    k_trace<false><<<blocks_for(s->trace_blocks, p->n), kTraceThreads, 0, st>>>(view(s), frame_lights(s), A, am);
+    launch_dependent(k_trace<false>, blocks_for(s->trace_blocks, p->n), kTraceThreads, 0, st, view(s), frame_lights(s), A, am);
   }
-}
-
-// k_cont_trace right after k_verify.  With PV_CONT_TRACE_PDL it is a
-// programmatic dependent launch, which may start while k_verify is finishing.
-// That made back-to-back frames 3 % slower (villa 1.182 against 1.147 ms per
-// frame, city 0.440 against 0.427 ms) with the same time from a frame's first
-// launch to its last: the cost fell between frames.  So the launch is an
-// ordinary one by default.
-#ifndef PV_CONT_TRACE_PDL
-#define PV_CONT_TRACE_PDL 0
-#endif
-template <int kDep>
-void launch_cont_trace_pdl(int blocks, const SceneView& sv, const FrameLights& L, const TraceArgs& A,
-                           const ContArgs& C, const DepositArgs& D, cudaStream_t st) {
-  cudaLaunchConfig_t cfg;
-  std::memset(&cfg, 0, sizeof cfg);
-  cfg.gridDim = dim3(blocks);
-  cfg.blockDim = dim3(kTraceThreads);
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = PV_CONT_TRACE_PDL;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, k_cont_trace<kDep>, sv, L, A, C, D);
 }
 
 void launch_cont_trace(pv_scene* s, const pv_paths* p, const ContArgs& C, const uint32_t* list, const uint32_t* count,
@@ -376,14 +351,14 @@ void launch_cont_trace(pv_scene* s, const pv_paths* p, const ContArgs& C, const 
     D.touched = touched;
     if (delta) {
       if (!s->cont_trace_delta_blocks) s->cont_trace_delta_blocks = persistent_blocks(s, k_cont_trace<2>);
-      launch_cont_trace_pdl<2>(blocks_for(s->cont_trace_delta_blocks, p->n), view(s), frame_lights(s), A, C, D, st);
+      launch_dependent(k_cont_trace<2>, blocks_for(s->cont_trace_delta_blocks, p->n), kTraceThreads, 0, st, view(s), frame_lights(s), A, C, D);
     } else {
       if (!s->cont_trace_dep_blocks) s->cont_trace_dep_blocks = persistent_blocks(s, k_cont_trace<1>);
-      launch_cont_trace_pdl<1>(blocks_for(s->cont_trace_dep_blocks, p->n), view(s), frame_lights(s), A, C, D, st);
+      launch_dependent(k_cont_trace<1>, blocks_for(s->cont_trace_dep_blocks, p->n), kTraceThreads, 0, st, view(s), frame_lights(s), A, C, D);
     }
   } else {
     if (!s->cont_trace_blocks) s->cont_trace_blocks = persistent_blocks(s, k_cont_trace<0>);
-    launch_cont_trace_pdl<0>(blocks_for(s->cont_trace_blocks, p->n), view(s), frame_lights(s), A, C, D, st);
+    launch_dependent(k_cont_trace<0>, blocks_for(s->cont_trace_blocks, p->n), kTraceThreads, 0, st, view(s), frame_lights(s), A, C, D);
   }
 }
 

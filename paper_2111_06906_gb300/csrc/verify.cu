@@ -37,13 +37,10 @@ constexpr bool kVerifyLoop = PV_VERIFY_FLAT && PV_VERIFY_PERSISTENT;
 
 // Flat segment mapping in error mode (kFlat), else thread per path, each a
 // kernel of its own (one kernel with both needs the registers of the larger);
-// with kVerifyLoop a grid of resident blocks looping over tiles.  A re-trace kernel
-// launched as its programmatic dependent (PV_CONT_TRACE_PDL) may be scheduled as
-// soon as every block has started.
+// with kVerifyLoop a grid of resident blocks looping over tiles.
 template <bool kPointVis, bool kExact, bool kFlat>
 __device__ __forceinline__ void verify_kernel(const SceneView& sv, const FrameLights& L, const VerifyArgs& A,
                                               VerifySmem& sm) {
-  launch_dependents();
   if (kVerifyLoop) {
     verify_tiles<kPointVis, kExact, kFlat ? 2 : 0>(sv, L, A, blockIdx.x, gridDim.x, sm);
   } else {
@@ -55,6 +52,7 @@ __device__ __forceinline__ void verify_kernel(const SceneView& sv, const FrameLi
 // With visibility rays or triangle tests (traversal code inside).
 template <bool kPointVis, bool kExact, bool kFlat>
 __global__ void __launch_bounds__(pvh::kVerifyThreads) k_verify(SceneView sv, FrameLights L, VerifyArgs A) {
+  grid_dependency_wait();
   __shared__ VerifySmem sm;
   verify_kernel<kPointVis, kExact, kFlat>(sv, L, A, sm);
 }
@@ -63,6 +61,7 @@ __global__ void __launch_bounds__(pvh::kVerifyThreads) k_verify(SceneView sv, Fr
 template <bool kFlat>
 __global__ void __launch_bounds__(pvh::kVerifyThreads, PV_VERIFY_MIN_BLOCKS) k_verify_box(SceneView sv, FrameLights L,
                                                                                          VerifyArgs A) {
+  grid_dependency_wait();
   __shared__ VerifySmem sm;
   verify_kernel<false, false, kFlat>(sv, L, A, sm);
 }
@@ -86,10 +85,10 @@ void launch_k_verify(pv_scene* s, const SceneView& sv, const FrameLights& L, con
   int& per = s->verify_blocks_per_sm[(kPointVis ? 4 : 0) + (kExact ? 2 : 0) + (kFlat ? 1 : 0)];
   if constexpr (!kPointVis && !kExact) {
     const uint32_t grid = verify_grid(s, k_verify_box<kFlat>, per, A.n);
-    k_verify_box<kFlat><<<grid, pvh::kVerifyThreads, 0, st>>>(sv, L, A);
+    pvh::launch_dependent(k_verify_box<kFlat>, grid, pvh::kVerifyThreads, 0, st, sv, L, A);
   } else {
     const uint32_t grid = verify_grid(s, k_verify<kPointVis, kExact, kFlat>, per, A.n);
-    k_verify<kPointVis, kExact, kFlat><<<grid, pvh::kVerifyThreads, 0, st>>>(sv, L, A);
+    pvh::launch_dependent(k_verify<kPointVis, kExact, kFlat>, grid, pvh::kVerifyThreads, 0, st, sv, L, A);
   }
 }
 
@@ -100,6 +99,7 @@ void launch_k_verify(pv_scene* s, const SceneView& sv, const FrameLights& L, con
 }
 
 __global__ void __launch_bounds__(128, 6) k_continue(SceneView sv, ContArgs A) {
+  grid_dependency_wait();
   __shared__ uint32_t s_red[32 * 4];
   __shared__ unsigned long long s_red64[32];
   const int root = *sv.root;
@@ -162,18 +162,22 @@ ContArgs cont_args(pv_scene* s, const pv_paths* paths, const pv_verify_params* p
   return C;
 }
 
-// Work counters reset, DM_C of moved lights with a map cleared, then k_verify
-// (Sec. 3.1 + 3.2).  ``cont``: Alg. 1 has paths to look at this frame.
+// Work counters, the compactions' tile states and DM_C of moved lights with a
+// map cleared, then k_verify (Sec. 3.1 + 3.2).  ``cont``: Alg. 1 has paths to look at this frame.
 template <typename OnCleared = void (*)()>
 int launch_verify(pv_scene* s, const pv_paths* paths, const pv_verify_params* params, pv_frame_stats* d_stats,
                   const SceneView& sv, const FrameLights& L, cudaStream_t st, bool& cont, uint8_t* touched = nullptr,
                   bool direct_list = false, const pv_atlas* sub = nullptr, OnCleared on_cleared = [] {}) {
   const uint32_t n = paths->n;
-  if (cudaMemsetAsync(s->ws_ctr, 0, 16 * sizeof(uint32_t), st) != cudaSuccess) return PV_ERR_CUDA;
+  pvh::ClearSet C;
+  C.add(s->ws_ctr, 16);
+  if (!direct_list) {                              // a compaction follows (two, with maps)
+    C.add(s->ws_tiles, pvh::compact_words(n));
+    if (s->has_dm) C.add(s->ws_tiles + s->n_tiles + 1u, pvh::compact_words(n));
+  }
   for (uint32_t l = 0; l < s->n_lights; ++l)       // DM_C of moved lights with a map is counted afresh
-    if (L.dm[l].dims && ((L.moved_mask >> l) & 1u))
-      if (cudaMemsetAsync(L.dm[l].dmc, 0, (size_t)L.dm[l].cells * sizeof(uint32_t), st) != cudaSuccess)
-        return PV_ERR_CUDA;
+    if (L.dm[l].dims && ((L.moved_mask >> l) & 1u)) C.add(L.dm[l].dmc, L.dm[l].cells);
+  pvh::launch_clear(s, C, st);
   on_cleared();
   VerifyArgs A;
   A.n = n;
@@ -214,7 +218,7 @@ void launch_continue(pv_scene* s, const SceneView& sv, const ContArgs& C, cudaSt
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_continue, 128, 0);
     s->cont_blocks = (per > 0 ? per : 1) * s->num_sms;
   }
-  k_continue<<<s->cont_blocks, 128, 0, st>>>(sv, C);
+  pvh::launch_dependent(k_continue, s->cont_blocks, 128, 0, st, sv, C);
 }
 
 }  // namespace
@@ -232,7 +236,7 @@ extern "C" int pv_verify_paths(pv_scene* s, const pv_paths* paths, const pv_veri
   if ((rc = launch_verify(s, paths, params, d_stats, sv, L, st, cont)) != PV_OK) return rc;
   if (cont) launch_continue(s, sv, cont_args(s, paths, params, d_stats), st);
   if (s->has_dm && (rc = pvh::dm_frame(s, paths, L, params, d_stats, st)) != PV_OK) return rc;
-  pvh::launch_compact(s, paths->info, paths->n, d_list, d_count, d_stats ? &d_stats->n_listed : nullptr, st);
+  pvh::launch_compact(s, paths->info, paths->n, d_list, d_count, d_stats ? &d_stats->n_listed : nullptr, st, 0, false);
   return cudaGetLastError() == cudaSuccess ? PV_OK : PV_ERR_CUDA;
 }
 
@@ -278,7 +282,7 @@ int verify_retrace(pv_scene* s, const pv_paths* paths, const pv_verify_params* p
   } else {
     if (cont) launch_continue(s, sv, C, st);
     if (s->has_dm && (rc = pvh::dm_frame(s, paths, L, params, d_stats, st)) != PV_OK) return rc;
-    pvh::launch_compact(s, paths->info, paths->n, list, count, listed, st);
+    pvh::launch_compact(s, paths->info, paths->n, list, count, listed, st, 0, false);
     mark(3);
     pvh::launch_trace(s, paths, list, count, params->seed, params->frame, d_stats, st, nullptr, false);
     if (atlas) pvh::launch_deposit(s, paths, atlas, st);
