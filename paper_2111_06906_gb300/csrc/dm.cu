@@ -107,7 +107,8 @@ int dm_frame(pv_scene* s, const pv_paths* p, const FrameLights& L, const pv_veri
     launch_dependent(k_dm_deficit, dm_tiles(D.cells), kDmThreads, 0, st, D, s->dm_scan, s->dm_sums);
     launch_dependent(k_dm_prefix, dm_tiles(D.cells), kDmThreads, 0, st, D.cells, s->dm_scan, s->dm_sums);
     const uint32_t fb = std::min<uint32_t>((s->lights_new[l].n_paths + 255) / 256, 8u * (uint32_t)s->num_sms);
-    launch_dependent(k_dm_fill, std::max<uint32_t>(fb, 1u), 256, 0, st, L, l, s->dm_free, s->dm_ctr, s->dm_scan, p->info, stats);
+    launch_dependent(k_dm_fill, std::max<uint32_t>(fb, 1u), 256, 0, st, L, l, s->dm_free, s->dm_ctr, s->dm_scan, p->info,
+                     stats);
   }
   return cuda_status(cudaGetLastError());
 }
