@@ -1,11 +1,11 @@
 // Screen-space photon splat: the renderer's "splat/gather" step of Fig. 2.
 // The paper only cites its splatting method, so this is a plain radius
-// kernel, evaluated as a gather.  k_gbuffer casts one primary ray per pixel
+// kernel, evaluated as a gather.  k_view_count casts one primary ray per pixel
 // through the scene's BVH (visible point, normal facing the camera,
 // primitive).  Photons and visible points are both sorted by the cells of a
 // grid over space (count with ranks, scan, place), skipping photons whose
-// kernel cube reaches the near plane.  k_gather then gives each pixel the
-// photons of the cells around its visible point p: every photon x with
+// kernel cube reaches the near plane.  k_gather and k_gather_dense then give each
+// pixel the photons of the cells around its visible point p: every photon x with
 // energy E arriving on the visible side and s = |p - x| / r < 1 adds
 // rho/pi E 2 (1 - s^2) / (pi r^2).  Each pixel is written once, without
 // atomics, and the work per pixel is bounded by the photons near it, not by
@@ -72,11 +72,11 @@ __device__ __forceinline__ uint32_t grid_index(const Grid& g, int3 c) {
 // the same nodes: city at 1920 x 1080 0.277 ms in rows of 32 pixels, 0.232 ms in
 // tiles, 0.222 ms with five blocks per SM asked of the register allocator; six
 // take 0.237 ms).
-__global__ void __launch_bounds__(256, 5) k_gbuffer(SceneView sv, Cam c, GPixel* g) {
+__device__ __forceinline__ void gbuffer_tile(const SceneView& sv, const Cam& c, GPixel* g, uint32_t tile) {
   const uint32_t tiles_x = (c.W + 15u) / 16u;
   const uint32_t w = threadIdx.x >> 5, l = threadIdx.x & 31u;
-  const uint32_t i = (blockIdx.x % tiles_x) * 16u + (w & 1u) * 8u + (l & 7u);
-  const uint32_t j = (blockIdx.x / tiles_x) * 16u + (w >> 1) * 4u + (l >> 3);
+  const uint32_t i = (tile % tiles_x) * 16u + (w & 1u) * 8u + (l & 7u);
+  const uint32_t j = (tile / tiles_x) * 16u + (w >> 1) * 4u + (l >> 3);
   if (i >= c.W || j >= c.H) return;
   const float x = (2.0f * ((float)i + 0.5f) / (float)c.W - 1.0f) * c.tx;
   const float y = (1.0f - 2.0f * ((float)j + 0.5f) / (float)c.H) * c.ty;
@@ -123,15 +123,14 @@ constexpr uint32_t kSkipped = 0xFFFFFFFFu;
 // Count the photons per cell; rank[k n + p] = the photon's rank within its
 // cell, so that placing needs no second round of atomics.  A thread per path,
 // which has the loads (and then the atomics) of kRowsAtOnce rows in flight.
-// (Measured on the city, 2.0M photons: count 54 us and place 73 us at 2 rows, 57 and 85 us at 4, 49 and 110 us
-// one at a time; a thread per photon, exiting where a path is shorter, 57 and 107 us.)
+// (Measured on the city, 2.0M photons, as kernels of their own: count 54 us and
+// place 73 us at 2 rows, 57 and 85 us at 4, 49 and 110 us one at a time; a thread
+// per photon, exiting where a path is shorter, 57 and 107 us.)
 constexpr uint32_t kRowsAtOnce = 2;
 
-__global__ void __launch_bounds__(256) k_photon_count(Cam c, Grid g, float radius, uint32_t n, uint32_t B,
-                                                      const uint32_t* info, const float4* pa, uint32_t* counts,
-                                                      uint32_t* rank) {
-  grid_dependency_wait();
-  const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void count_photons(const Cam& c, const Grid& g, float radius, uint32_t n, uint32_t B,
+                                              const uint32_t* info, const float4* pa, uint32_t* counts, uint32_t* rank,
+                                              uint32_t p) {
   if (p >= n) return;
   const uint32_t L = min(info_nseg(info[p]), B);
   for (uint32_t k0 = 0; k0 < L; k0 += kRowsAtOnce) {
@@ -190,6 +189,42 @@ __global__ void __launch_bounds__(256) k_photon_place(Grid g, uint32_t n, uint32
   }
 }
 
+// Primary rays and the count of the photons need nothing of each other and are one
+// launch: the count's waits on memory and atomics are hidden behind the rays (a room
+// at 641 x 361 68 -> 62 us; on the city, where both fill the chip, 224 -> 215 us.
+// Placing the photons beside half of the rays in the same way gained nothing more).
+// Two kinds of blocks in one grid, the fewer ones at every stride-th place.
+struct Mix {
+  uint32_t few, stride, total;
+  bool photons_few;
+};
+
+Mix mix_blocks(uint32_t photon_blocks, uint32_t pixel_blocks) {
+  Mix m;
+  m.photons_few = photon_blocks <= pixel_blocks;
+  m.few = std::min(photon_blocks, pixel_blocks);
+  m.total = photon_blocks + pixel_blocks;
+  m.stride = m.few ? m.total / m.few : 1u;
+  return m;
+}
+
+// Whether block b is one of the photons' blocks; index: which one of its kind.
+__device__ __forceinline__ bool mix_photons(const Mix& m, uint32_t b, uint32_t& index) {
+  const uint32_t before = min((b + m.stride - 1u) / m.stride, m.few);    // of the fewer kind
+  const bool few = before < m.few && b == before * m.stride;
+  index = few ? before : b - before;
+  return few == m.photons_few;
+}
+
+__global__ void __launch_bounds__(256, 5) k_view_count(Mix m, SceneView sv, Cam c, Grid g, float radius, uint32_t n,
+                                                       uint32_t B, const uint32_t* info, const float4* pa,
+                                                       uint32_t* counts, uint32_t* rank, GPixel* gb) {
+  grid_dependency_wait();
+  uint32_t i;
+  if (mix_photons(m, blockIdx.x, i)) count_photons(c, g, radius, n, B, info, pa, counts, rank, i * 256u + threadIdx.x);
+  else gbuffer_tile(sv, c, gb, i);
+}
+
 // Exclusive scan of m = tiles * 4096 counters: tile sums, their scan, then
 // each tile's own scan plus its offset.
 __global__ void __launch_bounds__(1024) k_tile_sums(const uint32_t* v, uint32_t* sums) {
@@ -202,6 +237,7 @@ __global__ void __launch_bounds__(1024) k_tile_sums(const uint32_t* v, uint32_t*
   if (threadIdx.x < 32) {
     t = __reduce_add_sync(0xffffffffu, w[threadIdx.x]);
     if (threadIdx.x == 0) sums[blockIdx.x] = t;
+    if (blockIdx.x == 0 && threadIdx.x < 2) sums[gridDim.x + 1 + threadIdx.x] = 0u;    // the dense tiles' counters
   }
 }
 
@@ -272,43 +308,71 @@ __device__ __forceinline__ float unordered(int i) { return __int_as_float(i >= 0
 __device__ __forceinline__ float warp_min(float f) { return unordered(__reduce_min_sync(0xffffffffu, ordered(f))); }
 __device__ __forceinline__ float warp_max(float f) { return unordered(__reduce_max_sync(0xffffffffu, ordered(f))); }
 
-// Every visible pixel gathers the photons around its visible point.  A block
-// takes 8 x 4 pixels, one per lane of each of its four warps, which mostly see
-// points close to each other.  A warp looks up the rows of cells around the box
-// of these points (a lane per row), deals their photons out to its lanes 32 at
-// a time (coalesced loads), keeps those within the radius of the box in shared
-// memory, and walks the kept ones with all lanes together: every photon is a
-// broadcast read and a test against each lane's pixel.  Where the points spread
-// over more than kSpread cells beyond the first one (an edge in depth), the
-// warp takes them group by group.  Each warp takes every fourth 32 photons.
+// Every visible pixel gathers the photons around its visible point, a warp for
+// 8 x 4 pixels, which mostly see points close to each other.  The warp looks up the
+// rows of cells around the box of these points (a lane per row), deals their
+// photons out to its lanes 32 at a time (coalesced loads), keeps those within the
+// radius of the box in shared memory, and walks the kept ones with all lanes
+// together: every photon is a broadcast read and a test against each lane's pixel.
+// Where the points spread over more than kSpread cells beyond the first one (an
+// edge in depth), the warp takes them group by group.  The kept photons lie word by
+// word, so that four of them are tested with packed arithmetic (fma.rn.f32x2) on
+// 16-byte reads.
 //
-// The kept photons lie word by word, so that four of them are tested with packed
-// arithmetic (fma.rn.f32x2) on 16-byte reads.
+// A tile that meets more than kDenseAt photons (under a lamp, or with many groups)
+// is left to k_gather_dense, where a block of kDenseParts warps deals its photons
+// out.  Photons per tile differ by a thousand times within one image: with one
+// warp for every tile the densest finish long after the others, with several the
+// look-up of the rows, which each of them repeats, is most of the light tiles' time.
 //
-// Bound by issue: on the 1M-path city at 1920 x 1080 and r = 0.3 m (2.0M
-// photons, up to a few thousand in the cells around a point) 3.4e8 warp
-// instructions at 25 of 32 lanes, 64 % of the issue slots.  There it takes
-// 0.43 ms (0.46 with one photon tested at a time), where a thread per pixel
-// walking 27 hashed cells, which read each photon's previous vertex from the path
-// buffers, took 3.57 ms (1.14 ms with cells sorted by row and the segment in the
-// record: long waits on loads at 12 of 32 lanes).  One photon at a time, one warp
-// for 8 x 4 pixels took 0.99 ms and two 0.62: neighbouring tiles in one block
-// thrash L1 and the densest tiles finish late; two pixels per lane took 0.58 ms
-// and cells of half the radius 0.63 ms.  Six, seven and eight blocks per SM: 0.49,
-// 0.45 and 0.43 ms.
-constexpr int kParts = 4;          // warps of a block
-constexpr int kSpread = 2;         // measured on the city: 1 0.51 ms, 2 0.47, 3 0.51, 4 0.60
+// Bound by issue: on the 1M-path city at 1920 x 1080 and r = 0.3 m (2.0M photons)
+// the two take 0.34 ms (one warp for every tile 0.61 ms, two 0.45, four 0.43; one
+// photon at a time and four warps 0.46).  With 100k paths 0.105 ms (four warps
+// 0.264), r = 0.15 m 0.215 ms (0.402), at 960 x 360 0.256 ms (0.331), 300k paths of a
+// smaller district at 1076 x 704 0.137 ms (0.151), a room at 641 x 361 31 us (34).
+// A thread per pixel walking 27 hashed cells, which read each photon's
+// previous vertex from the path buffers, took 3.57 ms on the city (1.14 ms with
+// cells sorted by row and the segment in the record: long waits on loads at 12 of
+// 32 lanes); two pixels per lane and cells of half the radius were slower than one
+// and the whole radius (0.58 and 0.63 against 0.47 ms, four warps).
+constexpr int kSpread = 2;         // city, four warps: 1 0.51 ms, 2 0.47, 3 0.51, 4 0.60
+// Photons met (city, room and the district at 1076 x 704, us): 512 348, 31, 141; 1024
+// 341, 31, 137; 1536 349, 31, 138; 2048 358, 31, 147.  Warps, at 1024: 4 358, 31, 140;
+// 16 381, 31, 145.
+constexpr uint32_t kDenseAt = 1024;
+constexpr int kDenseParts = 8;
 
-__global__ void __launch_bounds__(32 * kParts, 8) k_gather(SceneView sv, Cam c, Grid g, float radius, const GPixel* gb,
-                                                        const uint32_t* starts, Photons ph, float* image) {
-  grid_dependency_wait();
+// What the gather reads and writes.  The dense tiles are listed in the unused
+// words of the visible points' normals (a tile has at least one pixel), their
+// number and a ticket follow the photons' total.
+struct Gather {
+  Cam c;
+  Grid g;
+  float radius;
+  GPixel* gb;
+  const uint32_t* starts;
+  Photons ph;
+  uint32_t* dense;                 // number of dense tiles, ticket
+  float* image;
+};
+
+// One tile, by kParts warps of which this is number ``part``.  With kParts = 1 a
+// tile that meets more than kDenseAt photons is listed instead.
+template <int kParts>
+__device__ __forceinline__ void gather_tile(const SceneView& sv, const Gather& G, uint32_t tile, int part) {
+  const Cam& c = G.c;
+  const Grid& g = G.g;
+  const float radius = G.radius;
+  const GPixel* const gb = G.gb;
+  const uint32_t* const starts = G.starts;
+  const Photons& ph = G.ph;
   constexpr int kBuf = 64;         // photons kept before they are tested: fewer than 32 left over plus 32 new
   enum { kX, kY, kZ, kDx, kDy, kDz, kEx, kEy, kEz, kWords };
   __shared__ __align__(16) float s_ph[kParts][kWords][kBuf];
-  __shared__ float s_acc[kParts][3][32];
-  const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
+  __shared__ float s_acc[kParts > 1 ? kParts : 1][3][32];
+  const int lane = threadIdx.x & 31;
   const uint32_t tiles_x = (c.W + 7u) / 8u;
-  const uint32_t pi = (blockIdx.x % tiles_x) * 8u + (lane & 7), pj = (blockIdx.x / tiles_x) * 4u + (lane >> 3);
+  const uint32_t pi = (tile % tiles_x) * 8u + (lane & 7), pj = (tile / tiles_x) * 4u + (lane >> 3);
   const bool inside = pi < c.W && pj < c.H;
   const float inv_r2 = 1.0f / (radius * radius);
   const float away = 3.0e18f;      // beyond every photon's radius
@@ -325,6 +389,7 @@ __global__ void __launch_bounds__(32 * kParts, 8) k_gather(SceneView sv, Cam c, 
   }
   const int3 cell = grid_cell(g, P);
   bool todo = prim >= 0;
+  uint32_t met = 0;                // photons in the rows of cells so far
   uint32_t kept = 0;               // photons in the buffer
   float2 sum[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
   float(&ph_s)[kWords][kBuf] = s_ph[part];
@@ -418,6 +483,11 @@ __global__ void __launch_bounds__(32 * kParts, 8) k_gather(SceneView sv, Cam c, 
       }
       const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
       const uint32_t shift = beg - (incl - cnt);             // the photon of rank t, if in this lane's range: shift + t
+      met += total;
+      if (kParts == 1 && met > kDenseAt) {
+        if (lane == 0) G.gb[atomicAdd(G.dense, 1u)].n.w = __uint_as_float(tile);
+        return;
+      }
       for (uint32_t t0 = 32u * part; t0 < total; t0 += 32u * kParts) {
         const uint32_t t = t0 + lane;
         int row = 0;                                         // the range that holds rank t: the first with incl > t
@@ -457,20 +527,42 @@ __global__ void __launch_bounds__(32 * kParts, 8) k_gather(SceneView sv, Cam c, 
   }
   // the parts of a pixel's sum meet in shared memory
   float3 acc = make_float3(sum[0].x + sum[0].y, sum[1].x + sum[1].y, sum[2].x + sum[2].y);
-  s_acc[part][0][lane] = acc.x;
-  s_acc[part][1][lane] = acc.y;
-  s_acc[part][2][lane] = acc.z;
-  __syncthreads();
-  if (part > 0 || !inside) return;
+  if (kParts > 1) {
+    s_acc[part][0][lane] = acc.x;
+    s_acc[part][1][lane] = acc.y;
+    s_acc[part][2][lane] = acc.z;
+    __syncthreads();
+    if (part > 0) return;
 #pragma unroll
-  for (int q = 1; q < kParts; ++q)
-    acc = acc + make_float3(s_acc[q][0][lane], s_acc[q][1][lane], s_acc[q][2][lane]);
+    for (int q = 1; q < kParts; ++q)
+      acc = acc + make_float3(s_acc[q][0][lane], s_acc[q][1][lane], s_acc[q][2][lane]);
+  }
+  if (!inside) return;
   const float norm = 2.0f / (3.14159265f * radius * radius) / 3.14159265f;   // kernel normalisation and 1/pi
   const float4 alb = prim >= 0 ? __ldg(sv.prim_alb + prim) : make_float4(0.f, 0.f, 0.f, 0.f);
-  float* o = image + 3 * ((size_t)pj * c.W + pi);
+  float* o = G.image + 3 * ((size_t)pj * c.W + pi);
   o[0] = alb.x * acc.x * norm;
   o[1] = alb.y * acc.y * norm;
   o[2] = alb.z * acc.z * norm;
+}
+
+__global__ void __launch_bounds__(32, 32) k_gather(SceneView sv, Gather G) {
+  grid_dependency_wait();
+  gather_tile<1>(sv, G, blockIdx.x, 0);
+}
+
+__global__ void __launch_bounds__(32 * kDenseParts, 32 / kDenseParts) k_gather_dense(SceneView sv, Gather G) {
+  grid_dependency_wait();
+  __shared__ uint32_t s_next;
+  const uint32_t n = G.dense[0];
+  for (;;) {
+    if (threadIdx.x == 0) s_next = atomicAdd(G.dense + 1, 1u);
+    __syncthreads();
+    const uint32_t k = s_next;
+    if (k >= n) break;
+    gather_tile<kDenseParts>(sv, G, __float_as_uint(G.gb[k].n.w), threadIdx.x >> 5);
+    __syncthreads();               // s_next and the parts' sums have been read
+  }
 }
 
 Cam make_cam(const pv_scene* s, const pv_camera* cam) {
@@ -530,7 +622,7 @@ struct SplatLayout {
     gbuf = 0;
     counts = up(gbuf + npx * sizeof(GPixel));
     sums = up(counts + (size_t)tiles(cells) * 4096 * sizeof(uint32_t));
-    rank = up(sums + (size_t)(tiles(cells) + 1) * sizeof(uint32_t));
+    rank = up(sums + (size_t)(tiles(cells) + 3) * sizeof(uint32_t));
     xd = up(rank + (size_t)photons * sizeof(uint32_t));
     e = up(xd + 2 * (size_t)photons * sizeof(float4));
     bytes = up(e + (size_t)photons * sizeof(float));
@@ -590,18 +682,23 @@ extern "C" int pv_splat(pv_scene* s, const pv_paths* paths, const pv_camera* cam
   // after the first, the kernels are dependent launches: six short kernels had a launch's latency between them
   const uint32_t tiles = SplatLayout::tiles(g.cells);
   PV_CHECK(cudaMemsetAsync(counts, 0, (size_t)tiles * 4096 * sizeof(uint32_t), st));
-  k_gbuffer<<<((c.W + 15) / 16) * ((c.H + 15) / 16), 256, 0, st>>>(sv, c, gbuf);
-  const uint32_t n = paths->n;
+  const uint32_t n = paths->n, photon_blocks = (n + 255) / 256;
   const float4* pa = reinterpret_cast<const float4*>(paths->pa);
   const float4* pb = reinterpret_cast<const float4*>(paths->pb);
-  if (n) pvh::launch_dependent(k_photon_count, (n + 255) / 256, 256, 0, st, c, g, radius, n, s->B, paths->info, pa, counts, rank);
+  const uint32_t views = ((c.W + 15) / 16) * ((c.H + 15) / 16);
+  const Mix m = mix_blocks(photon_blocks, views);
+  pvh::launch_dependent(k_view_count, m.total, 256, 0, st, m, sv, c, g, radius, n, s->B, paths->info, pa, counts, rank,
+                        gbuf);
   pvh::launch_dependent(k_tile_sums, tiles, 1024, 0, st, counts, sums);
   pvh::exclusive_scan(sums, tiles, st);
   pvh::launch_dependent(k_tile_scan, tiles, 1024, 0, st, counts, sums);
   if (n)
-    pvh::launch_dependent(k_photon_place, (n + 255) / 256, 256, 0, st, g, n, s->B, paths->info, paths->origin, pa, pb, counts,
-                          rank, ph);
-  pvh::launch_dependent(k_gather, ((c.W + 7) / 8) * ((c.H + 3) / 4), 32 * kParts, 0, st, sv, c, g, radius, gbuf, counts, ph,
-                        d_image);
+    pvh::launch_dependent(k_photon_place, photon_blocks, 256, 0, st, g, n, s->B, paths->info, paths->origin, pa, pb,
+                          counts, rank, ph);
+  const uint32_t gather_tiles = ((c.W + 7) / 8) * ((c.H + 3) / 4);
+  const Gather G = {c, g, radius, gbuf, counts, ph, sums + tiles + 1, d_image};
+  pvh::launch_dependent(k_gather, gather_tiles, 32, 0, st, sv, G);
+  pvh::launch_dependent(k_gather_dense, std::min<uint32_t>(gather_tiles, 32u / kDenseParts * (uint32_t)s->num_sms),
+                        32 * kDenseParts, 0, st, sv, G);
   return pvh::cuda_status(cudaGetLastError());
 }
