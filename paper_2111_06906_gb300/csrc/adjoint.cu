@@ -389,12 +389,17 @@ __global__ void __launch_bounds__(128) k_adjoint(SceneView sv, FrameLights L, Mo
     for (int r = 0; r < 4; ++r) {
       const int tj = b.j0 + r;
       if (tj < 0 || tj >= (int)A.H) continue;
-      float v[12];
+      float gr = 0.f, gdx = 0.f;                  // row sums of ge weighted by wx, dx
+      auto tap = [&](int q, float r0, float r1, float r2) {
+        const float ge = r0 * E0.x + r1 * E0.y + r2 * E0.z;
+        gr = fmaf(ge, b.wx[q], gr);
+        gdx = fmaf(ge, b.dx[q], gdx);
+      };
       const size_t first = 3 * ((size_t)tj * A.W + (size_t)(int64_t)b.i0);
       if (inside && first + 16 <= floats) {
         const uint32_t o = (uint32_t)first & 3u;
         const float4* at = reinterpret_cast<const float4*>(G + (first - o));
-        float w[16];
+        float w[16], v[12];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const float4 x = q < 3 || o ? __ldg(at + q) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -404,19 +409,17 @@ __global__ void __launch_bounds__(128) k_adjoint(SceneView sv, FrameLights L, Mo
           w[4 * q + 3] = x.w;
         }
         shift_down(w, o, v);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) tap(q, v[3 * q], v[3 * q + 1], v[3 * q + 2]);
       } else {
+        // texels outside are left out, not taken as zero: the energy or the weight may be infinite
 #pragma unroll
-        for (int q = 0; q < 12; ++q) {
-          const int ti = b.i0 + q / 3;
-          v[q] = ti >= 0 && ti < (int)A.W ? __ldg(G + 3 * ((size_t)tj * A.W + ti) + q % 3) : 0.f;
+        for (int q = 0; q < 4; ++q) {
+          const int ti = b.i0 + q;
+          if (ti < 0 || ti >= (int)A.W) continue;
+          const float* t = G + 3 * ((size_t)tj * A.W + ti);
+          tap(q, __ldg(t), __ldg(t + 1), __ldg(t + 2));
         }
-      }
-      float gr = 0.f, gdx = 0.f;                  // row sums of ge weighted by wx, dx
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float ge = v[3 * q] * E0.x + v[3 * q + 1] * E0.y + v[3 * q + 2] * E0.z;
-        gr = fmaf(ge, b.wx[q], gr);
-        gdx = fmaf(ge, b.dx[q], gdx);
       }
       g.x = fmaf(gdx, b.wz[r], g.x);
       g.y += gr * b.dz[r];
