@@ -538,9 +538,13 @@ __device__ __forceinline__ void gather_tile(const SceneView& sv, const Gather& G
       acc = acc + make_float3(s_acc[q][0][lane], s_acc[q][1][lane], s_acc[q][2][lane]);
   }
   if (!inside) return;
-  const float norm = 2.0f / (3.14159265f * radius * radius) / 3.14159265f;   // kernel normalisation and 1/pi
-  const float4 alb = prim >= 0 ? __ldg(sv.prim_alb + prim) : make_float4(0.f, 0.f, 0.f, 0.f);
   float* o = G.image + 3 * ((size_t)pj * c.W + pi);
+  if (prim < 0) {                  // nothing seen: zero also where the normalisation overflows
+    o[0] = o[1] = o[2] = 0.0f;
+    return;
+  }
+  const float norm = 2.0f / (3.14159265f * radius * radius) / 3.14159265f;   // kernel normalisation and 1/pi
+  const float4 alb = __ldg(sv.prim_alb + prim);
   o[0] = alb.x * acc.x * norm;
   o[1] = alb.y * acc.y * norm;
   o[2] = alb.z * acc.z * norm;
