@@ -124,7 +124,8 @@ __device__ __forceinline__ bool seg_vs_object(const SceneView& sv, const Seg& g,
 }
 
 // Moved-object groups staged in shared memory (MovedGroups): their boxes, and the
-// members' boxes group after group (empty past a group's last).
+// members' boxes group after group (past a group's last: not a number, which no
+// segment overlaps, not even one that leaves the range of float).
 struct GroupSmem {
   Box box[kMaxGroups];
   Box member[kMaxGroups * kGroupSize];
@@ -368,7 +369,7 @@ __device__ __forceinline__ void verify_smem_init(const SceneView& sv, VerifySmem
   for (int i = threadIdx.x; i < ng * 6; i += blockDim.x) sm.groups.box[i / 6].set(i % 6, sv.groups->box[i / 6][i % 6]);
   for (int i = threadIdx.x; i < ng * kGroupSize * 6; i += blockDim.x) {
     const int m = i / 6, k = i % 6, s = sv.groups->slot[m / kGroupSize][m % kGroupSize];
-    sm.groups.member[m].set(k, s >= 0 ? sm.uni[s].get(k) : k < 3 ? 3.0e38f : -3.0e38f);
+    sm.groups.member[m].set(k, s >= 0 ? sm.uni[s].get(k) : __int_as_float(0x7fffffff));
   }
   if (threadIdx.x == 0) sm.groups.n = ng;
   if (threadIdx.x == 0) {
