@@ -593,9 +593,13 @@ __device__ __forceinline__ bool trav_pop(Trav& t, const Stk& stk) {
   return false;
 }
 
-// A step counts toward the ray's cap; true if it reached it (the ray stops, a miss).
+// A step counts toward the ray's cap; true if the cap refuses it (the ray stops, a
+// miss; the refused step counts as no visit).
 __device__ __forceinline__ bool trav_capped(const SceneView& sv, Trav& t) {
-  if (++t.visits <= sv.max_visits) return false;
+  if (t.visits < sv.max_visits) {
+    ++t.visits;
+    return false;
+  }
   record_error(sv.status, PV_ERR_ITER_CAP);
   return true;
 }
