@@ -343,8 +343,8 @@ constexpr uint32_t kDenseAt = 1024;
 constexpr int kDenseParts = 8;
 
 // What the gather reads and writes.  The dense tiles are listed in the unused
-// words of the visible points' normals (a tile has at least one pixel), their
-// number and a ticket follow the photons' total.
+// words of the visible points' normals (a tile has at least one pixel), which
+// k_gather itself never reads; their number and a ticket follow the photons' total.
 struct Gather {
   Cam c;
   Grid g;
@@ -384,7 +384,8 @@ __device__ __forceinline__ void gather_tile(const SceneView& sv, const Gather& G
     prim = __float_as_int(p.w);
     if (prim >= 0) {
       P = f3(p);
-      nrm = f3(q->n);
+      const float2 nxy = *reinterpret_cast<const float2*>(&q->n);    // not n.w, which other warps write (Gather)
+      nrm = make_float3(nxy.x, nxy.y, q->n.z);
     }
   }
   const int3 cell = grid_cell(g, P);
