@@ -32,21 +32,57 @@ struct GPixel {              // 32 bytes per pixel
 };
 
 // Grid over space for photons and visible points: cells of edge ``edge`` =
-// radius / kCellsPerRadius, wrapped around after nx, ny, nz cells per axis and
-// numbered with x fastest.  A photon within ``radius`` of a point lies at most
-// kReach cells from the point's cell along every axis; each axis has at least
-// 2 kReach + 2 cells, so the cells around a point are distinct and hold every
-// photon once.  Wrapping lets points far apart share a cell: such photons fail
-// the distance test.  Cells next to each other in x are next to each other in
-// the sorted photons, so the cells around points in a box are a few ranges.
+// radius / kCellsPerRadius.  A photon within ``radius`` of a point lies at most
+// kReach cells from the point's cell along every axis.  Cells next to each other
+// in x are next to each other in the sorted photons, so the cells around points in
+// a box are a few ranges (rows).
+//
+// Where the scene's extent has few enough cells, axes wrap around after nx, ny, nz
+// cells, numbered with x fastest; each axis has at least 2 kReach + 2 cells, so the
+// cells around a point are distinct and hold every photon once.  Otherwise (small
+// radii) there is one row of nx = ``cells`` (a power of two) places around which
+// cell (x, y, z) lies at x + sy y + sz z: the rows of a group of points are
+// distinct (rows_distinct), and photons on a plane or in a box spread over all
+// places as a hash spreads them.  (Axes that wrap earlier instead lay the cells of
+// a plane on each other: 2.5M photon places over a floor, 700 x 500 points, r = 2 mm
+// 813 us, 147 in one row; r = 20 mm 330 and 101; the 1M-path city at 1920 x 1080
+// 1149 and 966 us at 2 mm, 541 and 529 at 0.1 m.)  Points far apart may share a
+// place: such photons fail the distance test.
 constexpr int kCellsPerRadius = 1;
 constexpr int kReach = kCellsPerRadius;
+constexpr int kSpread = 2;         // cells between points gathered together (k_gather); city, four warps: 1 0.51 ms, 2 0.47, 3 0.51, 4 0.60
 
 struct Grid {
   float inv_edge;
   int nx, ny, nz;
-  uint32_t cells;              // nx ny nz
+  uint32_t cells;
+  uint32_t sy, sz;             // sy = 0: axes wrap by themselves
 };
+
+// sy and sz of ``cells`` places: the two-dimensional low-discrepancy sequence of the
+// plastic number p = 1.3247 (1/p and 1/p^2 of the places).
+constexpr uint32_t stride_y(uint32_t cells) { return (uint32_t)(0.7548776662466927 * cells) | 1u; }
+constexpr uint32_t stride_z(uint32_t cells) { return (uint32_t)(0.5698402909980532 * cells) | 1u; }
+
+// Whether the rows around a group of points, at most 2 (kSpread + kReach) apart in y
+// and in z and one more cell long, never overlap.
+constexpr bool rows_distinct(uint32_t cells) {
+  constexpr int kSpan = 2 * (kSpread + kReach);
+  for (int dy = -kSpan; dy <= kSpan; ++dy)
+    for (int dz = 0; dz <= kSpan; ++dz) {
+      if (dz == 0 && dy <= 0) continue;
+      const uint32_t d = ((uint32_t)dy * stride_y(cells) + (uint32_t)dz * stride_z(cells)) & (cells - 1u);
+      if (d < kSpan + 1u || cells - d < kSpan + 1u) return false;
+    }
+  return true;
+}
+constexpr uint32_t kMinCells = 4096, kMaxCells = 1u << 30;
+constexpr bool all_rows_distinct() {
+  for (uint32_t c = kMinCells; c <= kMaxCells; c <<= 1)
+    if (!rows_distinct(c)) return false;
+  return true;
+}
+static_assert(all_rows_distinct(), "a photon would be met twice");
 
 __device__ __forceinline__ int3 grid_cell(const Grid& g, float3 x) {
   const float lim = 1.0e9f;
@@ -60,12 +96,18 @@ __device__ __forceinline__ int wrap(int c, int n) {
   return m < 0 ? m + n : m;
 }
 
+// First place of the row of cells (., cy, cz) where axes wrap by themselves.
 __device__ __forceinline__ uint32_t grid_row(const Grid& g, int cy, int cz) {
   return ((uint32_t)wrap(cz, g.nz) * g.ny + (uint32_t)wrap(cy, g.ny)) * g.nx;
 }
 
+// Place of a cell in a grid of one row.
+__device__ __forceinline__ uint32_t row_place(const Grid& g, int cx, int cy, int cz) {
+  return ((uint32_t)cx + g.sy * (uint32_t)cy + g.sz * (uint32_t)cz) & (g.cells - 1u);
+}
+
 __device__ __forceinline__ uint32_t grid_index(const Grid& g, int3 c) {
-  return grid_row(g, c.y, c.z) + (uint32_t)wrap(c.x, g.nx);
+  return g.sy ? row_place(g, c.x, c.y, c.z) : grid_row(g, c.y, c.z) + (uint32_t)wrap(c.x, g.nx);
 }
 
 // One primary ray per pixel, a warp per 8 x 4 pixels (its rays then visit much
@@ -335,7 +377,6 @@ __device__ __forceinline__ float warp_max(float f) { return unordered(__reduce_m
 // cells sorted by row and the segment in the record: long waits on loads at 12 of
 // 32 lanes); two pixels per lane and cells of half the radius were slower than one
 // and the whole radius (0.58 and 0.63 against 0.47 ms, four warps).
-constexpr int kSpread = 2;         // city, four warps: 1 0.51 ms, 2 0.47, 3 0.51, 4 0.60
 // Photons met (city, room and the district at 1076 x 704, us): 512 348, 31, 141; 1024
 // 341, 31, 137; 1536 349, 31, 138; 2048 358, 31, 147.  Warps, at 1024: 4 358, 31, 140;
 // 16 381, 31, 145.
@@ -358,7 +399,7 @@ struct Gather {
 
 // One tile, by kParts warps of which this is number ``part``.  With kParts = 1 a
 // tile that meets more than kDenseAt photons is listed instead.
-template <int kParts>
+template <int kParts, bool kOneRow>
 __device__ __forceinline__ void gather_tile(const SceneView& sv, const Gather& G, uint32_t tile, int part) {
   const Cam& c = G.c;
   const Grid& g = G.g;
@@ -465,11 +506,30 @@ __device__ __forceinline__ void gather_tile(const SceneView& sv, const Gather& G
     // rows of cells around the group (each axis at most once around the grid); a row is two ranges where it wraps
     const int ny = min(hi.y - lo.y + 1 + 2 * kReach, g.ny), nz = min(hi.z - lo.z + 1 + 2 * kReach, g.nz);
     const int len = min(hi.x - lo.x + 1 + 2 * kReach, g.nx);
-    const int x0 = wrap(lo.x - kReach, g.nx), over = x0 + len - g.nx;
-    const int rows = ny * nz, ranges = over > 0 ? 2 * rows : rows;
+    const int rows = ny * nz;
+    int x0 = 0, over = 0;                        // the rows' first cell, and how many lie beyond its end
+    const uint32_t place = kOneRow ? row_place(g, lo.x - kReach, lo.y - kReach, lo.z - kReach) : 0u;   // of row 0
+    const int whole = (rows + 31) & ~31;         // in one row some rows may wrap: their second ranges follow from here
+    if (!kOneRow) {
+      x0 = wrap(lo.x - kReach, g.nx);
+      over = x0 + len - g.nx;
+    }
+    int ranges = over > 0 ? 2 * rows : rows;
     for (int r0 = 0; r0 < ranges; r0 += 32) {
       uint32_t beg = 0, cnt = 0;
-      if (r0 + lane < ranges) {
+      if (kOneRow) {
+        const bool second = r0 >= whole;
+        const int r = r0 + lane - (second ? whole : 0);
+        bool wraps = false;
+        if (r < rows) {
+          const uint32_t x = (place + g.sy * (uint32_t)(r % ny) + g.sz * (uint32_t)(r / ny)) & (g.cells - 1u);
+          const uint32_t end = x + len;
+          wraps = end > g.cells;
+          beg = starts[second ? 0u : x];
+          cnt = starts[!second ? min(end, g.cells) : wraps ? end - g.cells : 0u] - beg;
+        }
+        if (__any_sync(0xffffffffu, wraps)) ranges = whole + rows;
+      } else if (r0 + lane < ranges) {
         const bool second = r0 + lane >= rows;
         const int r = second ? r0 + lane - rows : r0 + lane;
         const uint32_t row = grid_row(g, lo.y - kReach + r % ny, lo.z - kReach + r / ny);
@@ -551,11 +611,13 @@ __device__ __forceinline__ void gather_tile(const SceneView& sv, const Gather& G
   o[2] = alb.z * acc.z * norm;
 }
 
+template <bool kOneRow>
 __global__ void __launch_bounds__(32, 32) k_gather(SceneView sv, Gather G) {
   grid_dependency_wait();
-  gather_tile<1>(sv, G, blockIdx.x, 0);
+  gather_tile<1, kOneRow>(sv, G, blockIdx.x, 0);
 }
 
+template <bool kOneRow>
 __global__ void __launch_bounds__(32 * kDenseParts, 32 / kDenseParts) k_gather_dense(SceneView sv, Gather G) {
   grid_dependency_wait();
   __shared__ uint32_t s_next;
@@ -565,7 +627,7 @@ __global__ void __launch_bounds__(32 * kDenseParts, 32 / kDenseParts) k_gather_d
     __syncthreads();
     const uint32_t k = s_next;
     if (k >= n) break;
-    gather_tile<kDenseParts>(sv, G, __float_as_uint(G.gb[k].n.w), threadIdx.x >> 5);
+    gather_tile<kDenseParts, kOneRow>(sv, G, __float_as_uint(G.gb[k].n.w), threadIdx.x >> 5);
     __syncthreads();               // s_next and the parts' sums have been read
   }
 }
@@ -620,8 +682,8 @@ struct SplatLayout {
   size_t gbuf, counts, sums, rank, xd, e, bytes;
   uint32_t cells;                                   // most cells a grid may have
   SplatLayout(uint64_t photons, uint32_t width, uint32_t height) {
-    cells = 4096;                                   // a power of two >= the photons, at least one scan tile
-    while (cells < photons && cells < (1u << 30)) cells <<= 1;
+    cells = kMinCells;                              // a power of two >= the photons, at least one scan tile
+    while (cells < photons && cells < kMaxCells) cells <<= 1;
     auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t npx = (size_t)width * height;
     gbuf = 0;
@@ -637,8 +699,8 @@ struct SplatLayout {
 };
 
 // Cells of edge radius / kCellsPerRadius over the scene's extent, each axis
-// with at least 2 kReach + 2 cells; where that is more than ``most`` cells, the
-// longest axes wrap around earlier.
+// with at least 2 kReach + 2 cells; one row of ``most`` places (a power of two)
+// where that is more than ``most`` cells.
 Grid make_grid(const pv_scene* s, float radius, uint32_t most) {
   Grid g;
   g.inv_edge = (float)kCellsPerRadius / radius;
@@ -647,14 +709,14 @@ Grid make_grid(const pv_scene* s, float radius, uint32_t most) {
     const double c = ((double)s->box_hi[k] - s->box_lo[k]) * g.inv_edge + 2.0;
     n[k] = c < 1048576.0 ? std::max((int)c, 2 * kReach + 2) : 1048576;      // NaN: the most
   }
-  while ((uint64_t)n[0] * n[1] * n[2] > most) {
-    int* longest = std::max_element(n, n + 3);
-    *longest = std::max((*longest + 1) / 2, 2 * kReach + 2);
-  }
-  g.nx = n[0];
-  g.ny = n[1];
-  g.nz = n[2];
-  g.cells = (uint32_t)n[0] * n[1] * n[2];
+  const uint64_t all = (uint64_t)n[0] * n[1] * n[2];
+  const bool fits = all <= most;
+  g.nx = fits ? n[0] : (int)most;
+  g.ny = fits ? n[1] : 1 << 30;
+  g.nz = fits ? n[2] : 1 << 30;
+  g.cells = fits ? (uint32_t)all : most;
+  g.sy = fits ? 0u : stride_y(most);
+  g.sz = fits ? 0u : stride_z(most);
   return g;
 }
 
@@ -702,8 +764,8 @@ extern "C" int pv_splat(pv_scene* s, const pv_paths* paths, const pv_camera* cam
                           counts, rank, ph);
   const uint32_t gather_tiles = ((c.W + 7) / 8) * ((c.H + 3) / 4);
   const Gather G = {c, g, radius, gbuf, counts, ph, sums + tiles + 1, d_image};
-  pvh::launch_dependent(k_gather, gather_tiles, 32, 0, st, sv, G);
-  pvh::launch_dependent(k_gather_dense, std::min<uint32_t>(gather_tiles, 32u / kDenseParts * (uint32_t)s->num_sms),
-                        32 * kDenseParts, 0, st, sv, G);
+  const uint32_t dense_blocks = std::min<uint32_t>(gather_tiles, 32u / kDenseParts * (uint32_t)s->num_sms);
+  pvh::launch_dependent(g.sy ? k_gather<true> : k_gather<false>, gather_tiles, 32, 0, st, sv, G);
+  pvh::launch_dependent(g.sy ? k_gather_dense<true> : k_gather_dense<false>, dense_blocks, 32 * kDenseParts, 0, st, sv, G);
   return pvh::cuda_status(cudaGetLastError());
 }
