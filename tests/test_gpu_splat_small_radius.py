@@ -49,19 +49,16 @@ def test_either_side_of_the_line(size, radius):
     pv.pv_destroy_scene(h)
 
 
-def test_small_radius_on_a_plane_costs_no_more():
-    """500k photons spread over a floor: at a hundredth of the radius a point has a ten-thousandth of the photons
-    in reach.  (With a grid whose cells of a plane fell on each other the image took four times as long.)"""
+def _best_ms(sc, cam, radii):
+    """Fastest of a dozen images at each radius."""
     import torch
-    sc = kit.rect_light_over_floor(500_000, B=1, R=20.0)
     h = gu.lib_scene(sc)
     P = pv.Paths.allocate(sc.n_paths, sc.max_bounces)
     pv.pv_trace_all(h, P, 3, 1)
-    cam = pv.PvCamera.make((0.0, 4.0, 12.0), (0.0, 0.5, 0.0), (0.0, 1.0, 0.0), math.radians(60.0), 700, 500)
-    img = torch.zeros(500, 700, 3, device="cuda")
-    work = torch.empty(pv.pv_splat_workspace_bytes(h, 700, 500), dtype=torch.uint8, device="cuda")
-
-    def best(radius):
+    img = torch.zeros(cam.height, cam.width, 3, device="cuda")
+    work = torch.empty(pv.pv_splat_workspace_bytes(h, cam.width, cam.height), dtype=torch.uint8, device="cuda")
+    out = []
+    for radius in radii:
         ms = []
         for _ in range(12):
             a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
@@ -70,7 +67,22 @@ def test_small_radius_on_a_plane_costs_no_more():
             b.record()
             torch.cuda.synchronize()
             ms.append(a.elapsed_time(b))
-        return min(ms)
-
-    assert best(0.002) < 2.0 * best(0.2)
+        out.append(min(ms))
     pv.pv_destroy_scene(h)
+    return out
+
+
+def test_small_radius_on_a_plane_costs_no_more():
+    """500k photons spread over a floor: at a hundredth of the radius a point has a ten-thousandth of the photons
+    in reach.  (With a grid whose cells of a plane fell on each other the image took four times as long.)"""
+    cam = pv.PvCamera.make((0.0, 4.0, 12.0), (0.0, 0.5, 0.0), (0.0, 1.0, 0.0), math.radians(60.0), 700, 500)
+    small, large = _best_ms(kit.rect_light_over_floor(500_000, B=1, R=20.0), cam, (0.002, 0.2))
+    assert small < 2.0 * large, (small, large)
+
+
+def test_points_far_apart_cost_little_more():
+    """A large image of a room whose points lie many radii apart.  (With the pixels of a tile taken one after the
+    other it took nearly four times as long as at a thousand times the radius; it takes 1.5 times.)"""
+    cam = pv.PvCamera.make((0.0, 1.5, 0.95), (0.0, 0.2, -0.4), (0.0, 1.0, 0.0), math.radians(60.0), 1920, 1080)
+    small, large = _best_ms(scenes.tiny_box(n_paths=10_000), cam, (0.0001, 0.1))
+    assert small < 2.5 * large, (small, large)
