@@ -76,7 +76,7 @@ constexpr bool rows_distinct(uint32_t cells) {
     }
   return true;
 }
-constexpr uint32_t kMinCells = 4096, kMaxCells = 1u << 30;
+constexpr uint32_t kMinCells = 2048, kMaxCells = 1u << 30;
 constexpr bool all_rows_distinct() {
   for (uint32_t c = kMinCells; c <= kMaxCells; c <<= 1)
     if (!rows_distinct(c)) return false;
@@ -162,18 +162,25 @@ struct Photons {
 
 constexpr uint32_t kSkipped = 0xFFFFFFFFu;
 
-// Count the photons per cell; rank[k n + p] = the photon's rank within its
-// cell, so that placing needs no second round of atomics.  A thread per path,
+// The paths whose photons are sorted and gathered in one pass: all of them, or a
+// part in a workspace that does not hold all (SplatLayout).
+struct PathRange {
+  uint32_t first, count;
+};
+
+// Count the photons per cell; rank[k count + i] = the rank within its cell of
+// photon k of the range's path i, so that placing needs no second round of atomics.  A thread per path,
 // which has the loads (and then the atomics) of kRowsAtOnce rows in flight.
 // (Measured on the city, 2.0M photons, as kernels of their own: count 54 us and
 // place 73 us at 2 rows, 57 and 85 us at 4, 49 and 110 us one at a time; a thread
 // per photon, exiting where a path is shorter, 57 and 107 us.)
 constexpr uint32_t kRowsAtOnce = 2;
 
-__device__ __forceinline__ void count_photons(const Cam& c, const Grid& g, float radius, uint32_t n, uint32_t B,
-                                              const uint32_t* info, const float4* pa, uint32_t* counts, uint32_t* rank,
-                                              uint32_t p) {
-  if (p >= n) return;
+__device__ __forceinline__ void count_photons(const Cam& c, const Grid& g, float radius, PathRange R, uint32_t n,
+                                              uint32_t B, const uint32_t* info, const float4* pa, uint32_t* counts,
+                                              uint32_t* rank, uint32_t i) {
+  if (i >= R.count) return;
+  const uint32_t p = R.first + i;
   const uint32_t L = min(info_nseg(info[p]), B);
   for (uint32_t k0 = 0; k0 < L; k0 += kRowsAtOnce) {
     float4 x[kRowsAtOnce];
@@ -188,17 +195,17 @@ __device__ __forceinline__ void count_photons(const Cam& c, const Grid& g, float
     }
 #pragma unroll
     for (uint32_t q = 0; q < kRowsAtOnce; ++q)
-      if (k0 + q < L) rank[(size_t)(k0 + q) * n + p] = r[q];
+      if (k0 + q < L) rank[(size_t)(k0 + q) * R.count + i] = r[q];
   }
 }
 
 // Place the photons (starts: exclusive prefix of the counts).
-__global__ void __launch_bounds__(256) k_photon_place(Grid g, uint32_t n, uint32_t B, const uint32_t* info,
+__global__ void __launch_bounds__(256) k_photon_place(Grid g, PathRange R, uint32_t n, uint32_t B, const uint32_t* info,
                                                       const float* origin, const float4* pa, const float4* pb,
                                                       const uint32_t* starts, const uint32_t* rank, Photons out) {
   grid_dependency_wait();
-  const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= n) return;
+  const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x, p = R.first + i;
+  if (i >= R.count) return;
   const uint32_t L = min(info_nseg(info[p]), B);
   if (L == 0) return;
   float3 prev = make_float3(origin[p], origin[n + p], origin[2 * (size_t)n + p]);
@@ -211,7 +218,7 @@ __global__ void __launch_bounds__(256) k_photon_place(Grid g, uint32_t n, uint32
       if (k0 + q < L) {
         x[q] = pa[(size_t)(k0 + q) * n + p];
         e[q] = pb[(size_t)(k0 + q) * n + p];
-        r[q] = rank[(size_t)(k0 + q) * n + p];
+        r[q] = rank[(size_t)(k0 + q) * R.count + i];
       }
     }
 #pragma unroll
@@ -258,12 +265,12 @@ __device__ __forceinline__ bool mix_photons(const Mix& m, uint32_t b, uint32_t& 
   return few == m.photons_few;
 }
 
-__global__ void __launch_bounds__(256, 5) k_view_count(Mix m, SceneView sv, Cam c, Grid g, float radius, uint32_t n,
-                                                       uint32_t B, const uint32_t* info, const float4* pa,
+__global__ void __launch_bounds__(256, 5) k_view_count(Mix m, SceneView sv, Cam c, Grid g, float radius, PathRange R,
+                                                       uint32_t n, uint32_t B, const uint32_t* info, const float4* pa,
                                                        uint32_t* counts, uint32_t* rank, GPixel* gb) {
   grid_dependency_wait();
   uint32_t i;
-  if (mix_photons(m, blockIdx.x, i)) count_photons(c, g, radius, n, B, info, pa, counts, rank, i * 256u + threadIdx.x);
+  if (mix_photons(m, blockIdx.x, i)) count_photons(c, g, radius, R, n, B, info, pa, counts, rank, i * 256u + threadIdx.x);
   else gbuffer_tile(sv, c, gb, i);
 }
 
@@ -396,6 +403,7 @@ struct Gather {
   Photons ph;
   uint32_t* dense;                 // number of dense tiles, ticket
   float* image;
+  bool add;                        // onto the image of the passes before
 };
 
 // Each pixel's photons by its own lane, for tiles whose points lie apart: at radii
@@ -664,14 +672,16 @@ __device__ __forceinline__ void gather_tile(const SceneView& sv, const Gather& G
   if (!inside) return;
   float* o = G.image + 3 * ((size_t)pj * c.W + pi);
   if (prim < 0) {                  // nothing seen: zero also where the normalisation overflows
-    o[0] = o[1] = o[2] = 0.0f;
+    if (!G.add) o[0] = o[1] = o[2] = 0.0f;
     return;
   }
   const float norm = 2.0f / (3.14159265f * radius * radius) / 3.14159265f;   // kernel normalisation and 1/pi
   const float4 alb = __ldg(sv.prim_alb + prim);
-  o[0] = alb.x * acc.x * norm;
-  o[1] = alb.y * acc.y * norm;
-  o[2] = alb.z * acc.z * norm;
+  acc = make_float3(alb.x * acc.x * norm, alb.y * acc.y * norm, alb.z * acc.z * norm);
+  if (G.add) acc = acc + make_float3(o[0], o[1], o[2]);
+  o[0] = acc.x;
+  o[1] = acc.y;
+  o[2] = acc.z;
 }
 
 template <bool kOneRow>
@@ -740,25 +750,49 @@ bool camera_ok(const pv_camera* c) {
 }
 
 // Workspace layout: G-buffer, photons per cell (padded to whole scan
-// tiles), tile sums, photon ranks, sorted photons.
+// tiles), tile sums, photon ranks, sorted photons: 40 bytes a photon place, and 4 to
+// 8 for the cells.  A workspace of 32 bytes a place (least_bytes) does as well: half
+// the cells, and the paths in two passes (1M-path city at 1920 x 1080 380 MB, 648 us, and 324 MB, 769 us).
 struct SplatLayout {
   size_t gbuf, counts, sums, rank, xd, e, bytes;
   uint32_t cells;                                   // most cells a grid may have
-  SplatLayout(uint64_t photons, uint32_t width, uint32_t height) {
-    cells = kMinCells;                              // a power of two >= the photons, at least one scan tile
-    while (cells < photons && cells < kMaxCells) cells <<= 1;
-    auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
-    const size_t npx = (size_t)width * height;
+  uint32_t paths;                                   // most paths a pass may have
+  SplatLayout(uint32_t n, uint32_t B, uint32_t width, uint32_t height) {
+    const uint64_t photons = (uint64_t)n * B;
+    cells = full_cells(photons);
+    paths = n;
     gbuf = 0;
-    counts = up(gbuf + npx * sizeof(GPixel));
+    counts = up((size_t)width * height * sizeof(GPixel));
     sums = up(counts + (size_t)tiles(cells) * 4096 * sizeof(uint32_t));
     rank = up(sums + (size_t)(tiles(cells) + 3) * sizeof(uint32_t));
     xd = up(rank + (size_t)photons * sizeof(uint32_t));
     e = up(xd + 2 * (size_t)photons * sizeof(float4));
     bytes = up(e + (size_t)photons * sizeof(float));
   }
+  // Squeeze into ``room`` (at least least_bytes, fewer than ``bytes``).
+  void squeeze(uint32_t n, uint32_t B, size_t room) {
+    cells /= 2;
+    sums = counts + (size_t)tiles(cells) * 4096 * sizeof(uint32_t);
+    xd = (sums + (size_t)(tiles(cells) + 3) * sizeof(uint32_t) + 15) & ~(size_t)15;
+    paths = (uint32_t)std::min<size_t>((room - xd) / (2 * sizeof(float4) + sizeof(float) + sizeof(uint32_t)) / B, n);
+    e = xd + 2 * (size_t)paths * B * sizeof(float4);
+    rank = e + (size_t)paths * B * sizeof(float);
+    bytes = rank + (size_t)paths * B * sizeof(uint32_t);
+  }
+  static size_t least_bytes(uint32_t n, uint32_t B, uint32_t width, uint32_t height) {
+    const uint64_t photons = (uint64_t)n * B;
+    const size_t c = full_cells(photons);
+    return up(up(up((size_t)width * height * sizeof(GPixel)) + c * sizeof(uint32_t)) + (c / 4096 + 1) * sizeof(uint32_t)) +
+           up((size_t)photons * 2 * sizeof(float4));
+  }
+  static uint32_t full_cells(uint64_t photons) {     // a power of two >= the photons, at least one scan tile
+    uint32_t c = 4096;
+    while (c < photons && c < kMaxCells) c <<= 1;
+    return c;
+  }
   // scan tiles over the counters of a grid of c cells and the total behind them
   static uint32_t tiles(uint32_t c) { return (uint32_t)(((uint64_t)c + 1 + 4095) / 4096); }
+  static size_t up(size_t x) { return (x + 255) & ~(size_t)255; }
 };
 
 // Cells of edge radius / kCellsPerRadius over the scene's extent, each axis
@@ -790,7 +824,7 @@ Grid make_grid(const pv_scene* s, float radius, uint32_t most) {
 
 extern "C" size_t pv_splat_workspace_bytes(const pv_scene* s, uint32_t width, uint32_t height) {
   if (!s) return 0;
-  return SplatLayout((uint64_t)s->n_paths_total * s->B, width, height).bytes;
+  return SplatLayout(s->n_paths_total, s->B, width, height).bytes;
 }
 
 extern "C" int pv_splat(pv_scene* s, const pv_paths* paths, const pv_camera* cam, float radius, float* d_image,
@@ -799,8 +833,13 @@ extern "C" int pv_splat(pv_scene* s, const pv_paths* paths, const pv_camera* cam
   if (rc != PV_OK) return rc;
   if (!camera_ok(cam) || !d_image || !d_work || !(radius > 0.0f)) return PV_ERR_ARG;
   if (paths->n > (1u << 27)) return PV_ERR_LIMIT;            // photon ranks are 32-bit
-  const SplatLayout lay((uint64_t)paths->n * paths->max_bounces, cam->width, cam->height);
-  if (work_bytes < lay.bytes || (reinterpret_cast<uintptr_t>(d_work) & 255u)) return PV_ERR_ARG;
+  const uint32_t n = paths->n;
+  SplatLayout lay(n, s->B, cam->width, cam->height);
+  if (reinterpret_cast<uintptr_t>(d_work) & 255u) return PV_ERR_ARG;
+  if (work_bytes < lay.bytes) {
+    if (work_bytes < SplatLayout::least_bytes(n, s->B, cam->width, cam->height)) return PV_ERR_ARG;
+    lay.squeeze(n, s->B, work_bytes);
+  }
   cudaStream_t st = (cudaStream_t)stream;
   s->last_stream = st;
   const Cam c = make_cam(s, cam);
@@ -812,26 +851,32 @@ extern "C" int pv_splat(pv_scene* s, const pv_paths* paths, const pv_camera* cam
   uint32_t* rank = reinterpret_cast<uint32_t*>(w + lay.rank);
   const Photons ph = {reinterpret_cast<float4*>(w + lay.xd), reinterpret_cast<float*>(w + lay.e)};
   const pvk::SceneView sv = pvh::view(s);
-  // after the first, the kernels are dependent launches: six short kernels had a launch's latency between them
+  // after the memset, the kernels are dependent launches: short kernels had a launch's latency between them
   const uint32_t tiles = SplatLayout::tiles(g.cells);
-  PV_CHECK(cudaMemsetAsync(counts, 0, (size_t)tiles * 4096 * sizeof(uint32_t), st));
-  const uint32_t n = paths->n, photon_blocks = (n + 255) / 256;
   const float4* pa = reinterpret_cast<const float4*>(paths->pa);
   const float4* pb = reinterpret_cast<const float4*>(paths->pb);
-  const uint32_t views = ((c.W + 15) / 16) * ((c.H + 15) / 16);
-  const Mix m = mix_blocks(photon_blocks, views);
-  pvh::launch_dependent(k_view_count, m.total, 256, 0, st, m, sv, c, g, radius, n, s->B, paths->info, pa, counts, rank,
-                        gbuf);
-  pvh::launch_dependent(k_tile_sums, tiles, 1024, 0, st, counts, sums);
-  pvh::exclusive_scan(sums, tiles, st);
-  pvh::launch_dependent(k_tile_scan, tiles, 1024, 0, st, counts, sums);
-  if (n)
-    pvh::launch_dependent(k_photon_place, photon_blocks, 256, 0, st, g, n, s->B, paths->info, paths->origin, pa, pb,
-                          counts, rank, ph);
   const uint32_t gather_tiles = ((c.W + 7) / 8) * ((c.H + 3) / 4);
-  const Gather G = {c, g, radius, gbuf, counts, ph, sums + tiles + 1, d_image};
   const uint32_t dense_blocks = std::min<uint32_t>(gather_tiles, 32u / kDenseParts * (uint32_t)s->num_sms);
-  pvh::launch_dependent(g.sy ? k_gather<true> : k_gather<false>, gather_tiles, 32, 0, st, sv, G);
-  pvh::launch_dependent(g.sy ? k_gather_dense<true> : k_gather_dense<false>, dense_blocks, 32 * kDenseParts, 0, st, sv, G);
+  PathRange R = {0, std::min(n, lay.paths)};
+  do {
+    const uint32_t photon_blocks = (R.count + 255) / 256;
+    const uint32_t views = R.first == 0 ? ((c.W + 15) / 16) * ((c.H + 15) / 16) : 0u;
+    const Mix m = mix_blocks(photon_blocks, views);
+    PV_CHECK(cudaMemsetAsync(counts, 0, (size_t)tiles * 4096 * sizeof(uint32_t), st));
+    pvh::launch_dependent(k_view_count, m.total, 256, 0, st, m, sv, c, g, radius, R, n, s->B, paths->info, pa, counts,
+                          rank, gbuf);
+    pvh::launch_dependent(k_tile_sums, tiles, 1024, 0, st, counts, sums);
+    pvh::exclusive_scan(sums, tiles, st);
+    pvh::launch_dependent(k_tile_scan, tiles, 1024, 0, st, counts, sums);
+    if (R.count)
+      pvh::launch_dependent(k_photon_place, photon_blocks, 256, 0, st, g, R, n, s->B, paths->info, paths->origin, pa, pb,
+                            counts, rank, ph);
+    const Gather G = {c, g, radius, gbuf, counts, ph, sums + tiles + 1, d_image, R.first > 0};
+    pvh::launch_dependent(g.sy ? k_gather<true> : k_gather<false>, gather_tiles, 32, 0, st, sv, G);
+    pvh::launch_dependent(g.sy ? k_gather_dense<true> : k_gather_dense<false>, dense_blocks, 32 * kDenseParts, 0, st, sv,
+                          G);
+    R.first += R.count;
+    R.count = std::min(n - R.first, lay.paths);
+  } while (R.first < n);
   return pvh::cuda_status(cudaGetLastError());
 }
