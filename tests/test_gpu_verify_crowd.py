@@ -1,0 +1,92 @@
+"""The naive box test among many moved objects close to each other, where a segment
+overlaps dozens of boxes: parity with the FP64 oracle, and its time, which must not
+go into preparing the segment anew for every box."""
+import numpy as np
+import pytest
+
+import paper_2111_06906_gb300 as pv
+import scenes
+from tests import gpu_util as gu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_2111_06906_gb300 import build
+    build.build()
+    pv.load()
+
+
+def _crowd(n_paths, n_obj=64, spread=2.0):
+    b = scenes._Builder()
+    b.add(scenes._quad_grid((-20, 0, -20), (0, 0, 40), (40, 0, 0), 8, 8), (0.5, 0.5, 0.5))
+    rng = np.random.default_rng(4)
+    at = rng.uniform(-spread, spread, (n_obj, 3))
+    at[:, 1] = rng.uniform(1, 6, n_obj)
+    torus = scenes._torus(8, 8, 0.5, 0.2, vertical=True)
+    ids = [b.add(torus, (0.6, 0.4, 0.5), dynamic=True) for _ in range(n_obj)]
+    verts, obj, dyn, alb = b.arrays()
+
+    def xf(f):
+        x = scenes._identity_xforms(len(dyn))
+        for i in range(n_obj):
+            x[ids[i], [3, 7, 11]] = at[i] + np.array([0.1, 0.0, 0.05]) * (f - 1)
+        return x
+
+    def lf(f):
+        return [scenes.Light(scenes.LIGHT_RECT, (0.02 * (f - 1), 15.0, 0.0), (0.0, -1.0, 0.0), (1.0, 0.0, 0.0),
+                             (4.0, 4.0), (100.0,) * 3, n_paths)]
+
+    return scenes.Scene("crowd", verts, obj, dyn, alb, max_bounces=5, diag=60.0, atlas_rect=(-20.0, -20.0, 20.0, 20.0),
+                        seed=3, frames=2, tau=0.01, _xform_fn=xf, _light_fn=lf)
+
+
+def test_time_of_the_naive_box_test():
+    """2.8 times the error mode's verification; 3.5 times when the segment was prepared for every box."""
+    import torch
+    sc = _crowd(500_000)
+    h = gu.lib_scene(sc)
+    n = sc.n_paths
+    P = pv.Paths.allocate(n, sc.max_bounces)
+    pv.pv_trace_all(h, P, 3, 1)
+    gu.advance(h, sc, 2)
+    base = [t.clone() for t in (P.info, P.origin, P.pa, P.pb)]
+    lst = torch.zeros(n, dtype=torch.int32, device="cuda")
+    cnt = torch.zeros(1, dtype=torch.int32, device="cuda")
+
+    def best(mode):
+        ms = []
+        for _ in range(20):
+            for t, b in zip((P.info, P.origin, P.pa, P.pb), base):
+                t.copy_(b)
+            a, e = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            pv.pv_verify_paths(h, P, mode, 0.01, 0, lst, cnt)
+            e.record()
+            torch.cuda.synchronize()
+            ms.append(a.elapsed_time(e))
+        return min(ms)
+
+    assert best(pv.PV_MODE_NAIVE_AABB) < 3.15 * best(pv.PV_MODE_ERROR)
+    pv.pv_destroy_scene(h)
+
+
+def test_oracle_lists_the_same_paths():
+    import oracle
+    import torch
+    sc = _crowd(600)
+    o = oracle.OracleScene(sc)
+    o.set_frames(1, 1)
+    op = o.trace(np.arange(sc.n_paths, dtype=np.uint32), 5, 1)
+    h = gu.lib_scene(sc)
+    P = pv.Paths.allocate(sc.n_paths, sc.max_bounces)
+    gu.upload(P, op)
+    gu.advance(h, sc, 2)
+    lst = torch.zeros(sc.n_paths, dtype=torch.int32, device="cuda")
+    cnt = torch.zeros(1, dtype=torch.int32, device="cuda")
+    pv.pv_verify_paths(h, P, pv.PV_MODE_NAIVE_AABB, 0.01, 0, lst, cnt)
+    o.set_frames(1, 2)
+    o.verify(op, oracle.MODE_NAIVE_AABB, 0.01)
+    gu.assert_parity(gu.compare(gu.download(P), op, sc.diag))
+    pv.pv_destroy_scene(h)
