@@ -61,9 +61,9 @@ typedef struct {
  *                   2: flat (each warp deals the segments of its 32 paths
  *                   out to its lanes; PV_MODE_ERROR only)
  *  verify_threads   64, 128 or 256 paths per verify block (tile size)
- *  trace_steps      16, 32 or 64: at most this many traversal steps between
- *                   work refills; a warp refills earlier once every lane's
- *                   ray has ended
+ *  trace_steps      16, 32 or 64: at most this many node visits of a ray, and
+ *                   half as many leaf tests, between work refills; a warp
+ *                   refills earlier once every lane's ray has ended
  *  trace_blocks     persistent re-trace blocks per SM, 0 = occupancy limit
  *  stack            32 or 64 traversal stack entries for the continuation
  *                   and the re-trace; 32 only when every scene's wide tree
