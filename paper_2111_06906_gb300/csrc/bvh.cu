@@ -523,10 +523,16 @@ using namespace pvk;
 
 namespace pvh {
 
-void radix_sort(uint64_t*& k0, uint32_t*& v0, uint64_t*& k1, uint32_t*& v1, uint32_t n, uint32_t* hist,
-                       int lo_bit, int hi_bit, cudaStream_t st) {
-  const uint32_t n_tiles = (n + kRsTile - 1) / kRsTile;
-  for (int shift = lo_bit; shift < hi_bit; shift += 8) {
+void exclusive_scan(uint32_t* data, uint32_t m, cudaStream_t st) { launch_dependent(k_rs_scan, 1, 1024, 0, st, data, m); }
+
+static inline uint32_t blocks(uint32_t n, uint32_t t) { return (n + t - 1) / t; }
+
+// Stable LSD radix sort of (key, value) pairs; the buffers swap so that k0/v0 hold
+// the result; hist holds 256 counters per tile of kRsTile pairs.
+static void radix_sort(uint64_t*& k0, uint32_t*& v0, uint64_t*& k1, uint32_t*& v1, uint32_t n, uint32_t* hist,
+                       cudaStream_t st) {
+  const uint32_t n_tiles = blocks(n, kRsTile);
+  for (int shift = 0; shift < 64; shift += 8) {
     k_rs_hist<<<n_tiles, kRsThreads, 0, st>>>(k0, n, shift, hist, n_tiles);
     k_rs_scan<<<1, 1024, 0, st>>>(hist, 256u * n_tiles);
     k_rs_scatter<<<n_tiles, kRsThreads, 0, st>>>(k0, v0, k1, v1, n, shift, hist, n_tiles);
@@ -534,12 +540,6 @@ void radix_sort(uint64_t*& k0, uint32_t*& v0, uint64_t*& k1, uint32_t*& v1, uint
     std::swap(v0, v1);
   }
 }
-
-uint32_t radix_tiles(uint32_t n) { return (n + kRsTile - 1) / kRsTile; }
-
-void exclusive_scan(uint32_t* data, uint32_t m, cudaStream_t st) { launch_dependent(k_rs_scan, 1, 1024, 0, st, data, m); }
-
-static inline uint32_t blocks(uint32_t n, uint32_t t) { return (n + t - 1) / t; }
 
 // ---- oversized-triangle references (host)
 
@@ -845,7 +845,7 @@ int build_bvh(pv_scene* s, const float* h_verts, const std::vector<uint32_t>& st
         fail(cudaStreamSynchronize(st));             // the host vectors go out of scope
       } else {
         k_morton_static<<<blocks(ns, 256), 256, 0, st>>>(d_rbox, ns, f, k0, v0);
-        radix_sort(k0, v0, k1, v1, ns, hist, 0, 64, st);
+        radix_sort(k0, v0, k1, v1, ns, hist, st);
       }
       k_gather_static<<<blocks(ns, 256), 256, 0, st>>>(d_v, d_rtri, d_rbox, v0, d_prim, ns, s->tris, d_lbox);
       if (ns >= 2) {
@@ -951,7 +951,7 @@ int build_bvh(pv_scene* s, const float* h_verts, const std::vector<uint32_t>& st
   uint64_t *k0 = s->r_keys[0], *k1 = s->r_keys[1];
   uint32_t *v0 = s->r_vals[0], *v1 = s->r_vals[1];
   k_morton_dyn<<<blocks(nd, 256), 256, 0, st>>>(tmp_local, nullptr, s->d_tri_slot, nd, d_frames, s->objs, 0, k0, v0);
-  radix_sort(k0, v0, k1, v1, nd, s->r_hist, 0, 64, st);
+  radix_sort(k0, v0, k1, v1, nd, s->r_hist, st);
   k_gather_dyn<<<blocks(nd, 256), 256, 0, st>>>(v0, nd, tmp_local, tmp_prim, nullptr, s->d_local, s->d_tri_prim, nullptr);
   if (nd >= 2)
     k_karras<<<blocks(nd - 1, 256), 256, 0, st>>>(k0, (int)nd, s->nodes, (int)s->d_node_off, (int)s->d_tri_off,
@@ -1101,7 +1101,7 @@ void launch_update_dynamic(pv_scene* s, cudaStream_t st) {
         uint64_t *k0 = s->r_keys[0], *k1 = s->r_keys[1];
         uint32_t *v0 = s->r_vals[0], *v1 = s->r_vals[1];
         k_morton_dyn<<<blocks(n, 256), 256, 0, st>>>(nullptr, dtris, s->d_tri_slot, n, nullptr, s->objs, 1, k0, v0);
-        radix_sort(k0, v0, k1, v1, n, s->r_hist, 0, 64, st);
+        radix_sort(k0, v0, k1, v1, n, s->r_hist, st);
         k_gather_dyn<<<blocks(n, 256), 256, 0, st>>>(v0, n, s->d_local, s->d_tri_prim, dtris, s->r_local, s->r_prim, s->r_tris);
         std::swap(s->d_local, s->r_local);
         std::swap(s->d_tri_prim, s->r_prim);

@@ -165,11 +165,6 @@ int dm_frame(pv_scene* s, const pv_paths* p, const pvk::FrameLights& L, const pv
 // bvh.cu
 // exclusive prefix sum of m counters in place (one block)
 void exclusive_scan(uint32_t* data, uint32_t m, cudaStream_t st);
-// stable LSD radix sort of (key, value) pairs on key bits [lo_bit, hi_bit);
-// the buffers swap so that k0/v0 hold the result; hist holds 256 * radix_tiles(n)
-void radix_sort(uint64_t*& k0, uint32_t*& v0, uint64_t*& k1, uint32_t*& v1, uint32_t n, uint32_t* hist, int lo_bit,
-                int hi_bit, cudaStream_t st);
-uint32_t radix_tiles(uint32_t n);
 int build_bvh(pv_scene* s, const float* h_verts, const std::vector<uint32_t>& static_prims, cudaStream_t st);
 void launch_update_dynamic(pv_scene* s, cudaStream_t st);
 int build_refit_pairs(pv_scene* s, cudaStream_t st);
