@@ -120,6 +120,56 @@ def source_digest() -> str:
     return h.hexdigest()[:16]
 
 
+# Bytes of the printed line.  A reader that keeps the end of the output (3000 bytes of it, say) must find the whole
+# line there; with every row of every kernel and sweep in it the line had grown to 20 KB.
+LINE_BYTES = 2600
+
+CONFIG_KEYS = ("workload", "paths", "max_bounces", "mode", "tau", "frames_timed", "l2", "reuse_ms_per_frame",
+               "trace_all_ms_per_frame", "speedup_vs_trace_all", "batch_frame_ms", "rays_per_frame_reuse",
+               "rays_per_frame_trace_all", "listed_per_frame", "device_status", "parallelism")
+
+
+def _short(v):
+    """Floats to six digits, texts to 120 characters, in plain values, lists and dicts of them."""
+    if isinstance(v, float):
+        return float(f"{v:.6g}")
+    if isinstance(v, str):
+        return v if len(v) <= 120 else v[:117] + "..."
+    if isinstance(v, dict):
+        return {k: _short(x) for k, x in v.items()}
+    if isinstance(v, (list, tuple)):
+        return [_short(x) for x in v]
+    return v
+
+
+def headline(out: dict) -> dict:
+    """The line's values and their explanation in short: the named fields of ``config``, the dominant kernel of
+    ``roofline``, one number per secondary workload."""
+    r = dict(out)
+    cfg = out.get("config", {})
+    r["config"] = {k: cfg[k] for k in CONFIG_KEYS if k in cfg}
+    for name, ms in (("city", "reuse_ms_per_frame"), ("batch16", "batch_frame_ms")):
+        if isinstance(cfg.get(name), dict) and ms in cfg[name]:
+            r["config"][f"{name}_{ms}"] = cfg[name][ms]
+    for key, drop in (("roofline", ("kernels", "fma_probe", "ops_rule", "traffic_note", "hbm_peak")),
+                      ("cpu_baseline", ("frame_s", "ambiguity"))):
+        if isinstance(out.get(key), dict):
+            r[key] = {k: v for k, v in out[key].items() if k not in drop}
+    return {k: v if k in ("value", "ms_per_step", "e2e", "clocks") else _short(v) for k, v in r.items()}
+
+
+def emit(out: dict) -> None:
+    """One JSON line on stdout; every row behind it as another on stderr."""
+    line = headline(out)
+    text = json.dumps(line)
+    for key in ("cpu_baseline", "roofline"):           # explanations give way before the line does
+        if len(text) > LINE_BYTES and key in line:
+            line[key] = {k: v for k, v in line[key].items() if isinstance(v, (int, float)) or k in ("kernel", "unit", "kind")}
+            text = json.dumps(line)
+    print(json.dumps({"details": out}), file=sys.stderr, flush=True)
+    print(text, flush=True)
+
+
 class Clocks:
     """SM clock and clock-event reasons sampled during the timed region: every
     5 ms through NVML (the driver's libnvidia-ml, read-only queries), else
@@ -738,7 +788,7 @@ def run_ours(args, ws, rank, local):
         out["e2e"] = e2e
     if not args.no_cpu_baseline and ws == 1:
         out["cpu_baseline"] = cpu_baseline(args.workload, MODES[args.mode], cfg["tau"], args.cpu_seconds)
-    print(json.dumps(out), flush=True)
+    emit(out)
 
 
 SPLAT_CAMERAS = {"city": ((0.0, 45.0, 35.0), (0.0, 0.0, 0.0), 0.3), "villa": ((10.0, 2.5, 2.0), (14.0, 0.5, 6.0), 0.08)}
@@ -1012,7 +1062,7 @@ def run_batch(args, ws, rank, local, print_line=True):
            # graph kernel nodes per frame: prologue, transform + wide refit with the top levels, verify, Alg. 1 +
            # re-trace
            "gpu_launches": 4 * K, "clocks": clocks.summary()}
-    print(json.dumps(out), flush=True)
+    emit(out)
     return summary
 
 
@@ -1109,7 +1159,7 @@ def run_reference(args, ws, rank):
            "cpu_baseline": {"value": val, "unit": "paths/s", "cores": oracle.num_threads(), "kind": "oracle",
                             "sample": sample},
            "e2e": {"value": val, "unit": "paths/s", "h2d_bytes_per_step": 0, "d2h_bytes_per_step": 0}}
-    print(json.dumps(out), flush=True)
+    emit(out)
 
 
 def main():
