@@ -431,15 +431,14 @@ int pv_read_device_status(pv_scene* s);
  * sum's order within a pixel is not fixed.  d_image: float32
  * [height][width][3] device memory, written.  d_work: 256-byte-aligned device
  * memory (visible points, photon grid), pv_splat_workspace_bytes(s, width,
- * height) bytes: 32 a pixel, 40 a photon place (path x bounce) and 4 to 8 for
- * the cells.  32 a place and as many for the cells, in parts of whole 256 bytes,
- * are accepted too (32 a pixel; 4 a cell, the cells being the power of two, at
- * least 4096, not below the places; 4 for every 4096 cells and one more; 32 a
- * place): the photons are then taken in two passes, which is slower.
- * PV_ERR_ARG for a degenerate
- * camera (zero size, fov outside (0, 3.1), up parallel to the view
- * direction), radius <= 0, or a small or misaligned workspace; PV_ERR_LIMIT
- * for more than 2^27 paths. */
+ * height) bytes: 32 a pixel, 40 a photon place (path x bounce) and 4 to 8 a
+ * place for the cells.  A workspace with 32 bytes a place (its four parts, each
+ * rounded up to 256 bytes: 32 a pixel; 4 a cell, where the cells are the power
+ * of two, at least 4096, not below the places; 4 for every 4096 cells and one
+ * more; 32 a place) is accepted as well: the photons are then taken in two
+ * passes, which is slower.  PV_ERR_ARG for a degenerate camera (zero size, fov
+ * outside (0, 3.1), up parallel to the view direction), radius <= 0, or a small
+ * or misaligned workspace; PV_ERR_LIMIT for more than 2^27 paths. */
 typedef struct {
   float pos[3], target[3], up[3];
   float fov_y;

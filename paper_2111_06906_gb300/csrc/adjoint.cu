@@ -355,7 +355,7 @@ __device__ __forceinline__ void shift_down(const float (&w)[16], uint32_t o, flo
 // reduced per block in shared memory, then added to the global vector.
 // Bound by L1's wavefronts (65 %) and the chains' loads.  City, 2.0M photons:
 // 258 us with a thread per path and 48 scalar reads of the gradient a photon,
-// 172 us with the photons dealt out a lane each and four wide reads a row.  (Four
+// 166 us with the photons dealt out a lane each and four wide reads a row.  (Four
 // lanes a photon, one request a row, 228 us and 16 lanes 316 us: what they save in
 // L1 they spend on summing up and on shared memory.)
 __global__ void __launch_bounds__(128) k_adjoint(SceneView sv, FrameLights L, ModelArgs A, const float* G,

@@ -259,7 +259,7 @@ __global__ void k_b_frame_top(const BScene* S, const BFrame* F) {
 // stages a scene's view, lights, arguments and moved-object boxes in shared
 // memory when its next entry belongs to another scene, and adds that scene's
 // counters when it leaves it.
-// Box-only variants are held to 5 resident blocks of 256 threads (51 registers), as the single-scene kernel.
+// Box-only variants are held to 5 resident blocks of 256 threads (48 registers), as the single-scene kernel.
 template <bool kPointVis, bool kExact, int kMap>
 __global__ void __launch_bounds__(256, (kPointVis || kExact) ? 2 : (kMap == 2 ? PV_BATCH_FLAT_MIN_BLOCKS : 5)) k_b_verify(const BScene* S, const BFrame* F,
                                                                                   const uint32_t* tab, uint32_t n_entries) {
@@ -506,7 +506,8 @@ struct FusedLayout {
   }
 };
 
-// minimum resident blocks per SM of the fused kernel (a compile-time tuning knob)
+// Minimum resident blocks per SM of the fused kernel: 7 spill 38 bytes; batch of six
+// scenes (perf/cases.py) at 6, which spill nothing, 269.5 us, at 7 273.5, at 8 272.7.
 #ifndef PV_BATCH_CT_MIN_BLOCKS
 #define PV_BATCH_CT_MIN_BLOCKS 7
 #endif

@@ -2,10 +2,10 @@
 // The paper only cites its splatting method, so this is a plain radius
 // kernel, evaluated as a gather.  k_view_count casts one primary ray per pixel
 // through the scene's BVH (visible point, normal facing the camera,
-// primitive).  Photons and visible points are both sorted by the cells of a
-// grid over space (count with ranks, scan, place), skipping photons whose
-// kernel cube reaches the near plane.  k_gather and k_gather_dense then give each
-// pixel the photons of the cells around its visible point p: every photon x with
+// primitive).  The photons are sorted by the cells of a grid over space (count with
+// ranks, scan, place), skipping those whose kernel cube reaches the near plane.
+// k_gather and k_gather_dense then take the pixels in tiles of 8 x 4 and give each
+// the photons of the cells around its visible point p: every photon x with
 // energy E arriving on the visible side and s = |p - x| / r < 1 adds
 // rho/pi E 2 (1 - s^2) / (pi r^2).  Each pixel is written once, without
 // atomics, and the work per pixel is bounded by the photons near it, not by
@@ -31,8 +31,7 @@ struct GPixel {              // 32 bytes per pixel
   float4 n;                  // normal facing the camera
 };
 
-// Grid over space for photons and visible points: cells of edge ``edge`` =
-// radius / kCellsPerRadius.  A photon within ``radius`` of a point lies at most
+// Grid over space: cells of edge radius / kCellsPerRadius.  A photon within ``radius`` of a point lies at most
 // kReach cells from the point's cell along every axis.  Cells next to each other
 // in x are next to each other in the sorted photons, so the cells around points in
 // a box are a few ranges (rows).
@@ -240,7 +239,7 @@ __global__ void __launch_bounds__(256) k_photon_place(Grid g, PathRange R, uint3
 
 // Primary rays and the count of the photons need nothing of each other and are one
 // launch: the count's waits on memory and atomics are hidden behind the rays (a room
-// at 641 x 361 68 -> 62 us; on the city, where both fill the chip, 224 -> 215 us.
+// at 641 x 361 68 -> 62 us; on the city, where both fill the chip, 9 us less.
 // Placing the photons beside half of the rays in the same way gained nothing more).
 // Two kinds of blocks in one grid, the fewer ones at every stride-th place.
 struct Mix {
@@ -467,7 +466,7 @@ __device__ __forceinline__ void gather_tile(const SceneView& sv, const Gather& G
   const GPixel* const gb = G.gb;
   const uint32_t* const starts = G.starts;
   const Photons& ph = G.ph;
-  constexpr int kBuf = 64;         // photons kept before they are tested: fewer than 32 left over plus 32 new
+  constexpr int kBuf = 64;         // photons kept before they are tested: at most 32 left over plus 32 new
   enum { kX, kY, kZ, kDx, kDy, kDz, kEx, kEy, kEz, kWords };
   __shared__ __align__(16) float s_ph[kParts][kWords][kBuf];
   __shared__ float s_acc[kParts > 1 ? kParts : 1][3][32];

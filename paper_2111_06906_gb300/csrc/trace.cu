@@ -28,16 +28,18 @@ namespace {
 // city and villa workloads this beats refilling each lane after a fixed
 // number of steps (8) by 8-13 % on the re-trace and 14-15 % on trace-all, and
 // stopping once 24 or 16 lanes are done by 4-22 %.
-// Resident blocks asked of the register allocator: k_trace fits 8 blocks
-// (64 registers) without spills, and that beat 7 by 3-5 % on the city and
-// villa trace-all frames; k_cont_trace keeps 7 (72 registers), since 8 spill
-// (and moving its per-path state to shared memory to avoid that cost more
-// than the eighth block gained).
+// Resident blocks asked of the register allocator: k_trace 8 (64 registers, 36
+// bytes spilled), k_cont_trace 7 (72 registers, 20 bytes), settings found with an
+// earlier traversal step that spilled nothing there.  With this step, at 8 and 7
+// against 7 and 6 (no spills): villa frame 964 and 977 us, city frame 354 and 347,
+// city trace-all 729 and 724, separate calls 196 and 185, maps 496 and 481, ray
+// budget 248 and 234 (cases of perf/cases.py).  k_cont_trace at 8 spills 150 bytes:
+// villa 976, city 369 (and moving its per-path state to shared memory to avoid that
+// cost more than the eighth block gained).
 #ifndef PV_TRACE_MIN_BLOCKS
 #define PV_TRACE_MIN_BLOCKS 8
 #endif
-// k_trace with the deposit (the trace-all frame): 8 blocks spill 24 bytes and
-// still beat 7 blocks without spills by 4-5 % (villa 4.18 against 4.38 ms).
+// k_trace with the deposit (the trace-all frame): as without.
 #ifndef PV_TRACE_DEP_MIN_BLOCKS
 #define PV_TRACE_DEP_MIN_BLOCKS 8
 #endif

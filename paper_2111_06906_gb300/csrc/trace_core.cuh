@@ -156,8 +156,8 @@ constexpr int kNodeSteps = 2;
 
 // Advance every lane's ray until all rays of the warp have ended, or by at most
 // kMax node steps and kMax / kNodeSteps leaf steps (counting both against kMax ends
-// the batch's stretches of 32 too early: 271 -> 278 us); called by all lanes of the warp (a lane without a ray
-// passes done = true).  Returns whether this lane's ray has ended.  Waiting
+// the batch's stretches of 32 too early: 271 -> 278 us); called by all lanes of the
+// warp (a lane without a ray passes done = true).  Returns whether this lane's ray has ended.  Waiting
 // for the whole warp lets the ray-end code that follows run with all lanes.
 template <int kMax, int S = kStack, class Stk>
 __device__ __forceinline__ bool step_warp(const SceneView& sv, const Ray& r, Trav& t, Stk& stk, int excl, Work& wk,

@@ -28,8 +28,9 @@ namespace {
 #endif
 // Resident blocks asked of the register allocator for the box-only kernel:
 // 5 (48 registers) beat 4 by 6 % on the villa workload, and on the city's map frame
-// by 4 %; on the plain city frame 4 are 2 % faster, 6 are slower on all.  The variants with traversal code keep their registers (they
-// would spill).
+// by 4 %; on the plain city frame 4 are 2 % faster, 6 are slower on all.  The variants
+// with traversal code are not held to fewer registers; those with triangle tests
+// spill 36 to 104 bytes as they are.
 #ifndef PV_VERIFY_MIN_BLOCKS
 #define PV_VERIFY_MIN_BLOCKS 5
 #endif
