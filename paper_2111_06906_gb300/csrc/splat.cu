@@ -412,10 +412,11 @@ struct Gather {
 // photons; the tile's groups are then gathered as usual.
 // 1M-path city at 1920 x 1080, r = 1 mm: 975 -> 570 us (hashed cells, a thread a
 // pixel: 768); 100k paths 744 -> 345 (560); a room at 641 x 361, r = 0.1 mm 118 -> 63
-// (88).  Taken where the first group of a tile is one pixel, in grids of one row only:
-// taken at groups of up to 4, 8 or 16 pixels and up to 64 or 256 photons met it is
-// faster still at such radii, but what the tiles that give up have spent costs the
-// city image 2 to 25 % at r = 0.1 to 0.4 m.
+// (88).  Taken where a tile's first pixel and its last are groups of their own, in grids
+// of one row only: taken at groups of up to 4, 8 or 16 pixels and up to 64 or 256
+// photons met it is faster still at such radii, but what the tiles that give up have
+// spent costs the city image 2 to 25 % at r = 0.1 to 0.4 m; on the first pixel alone it
+// cost small images of districts at such radii 2 to 8 %.
 __device__ __forceinline__ bool walk_alone(const Gather& G, bool todo, int3 cell, float3 P, float3 N, float2 (&sum)[3]) {
   const Grid& g = G.g;
   const uint32_t* const starts = G.starts;
@@ -547,7 +548,8 @@ __device__ __forceinline__ void gather_tile(const SceneView& sv, const Gather& G
   if (kParts == 1 && kOneRow) {
     const unsigned left = __ballot_sync(0xffffffffu, todo);
     int3 c0;
-    if (left && __popc(__ballot_sync(0xffffffffu, group(left, c0))) == 1) {
+    const auto single = [&](unsigned from) { return __popc(__ballot_sync(0xffffffffu, group(from, c0))) == 1; };
+    if (left && single(left) && single(0x80000000u >> __clz(left))) {       // the first pixel and the last
       if (walk_alone(G, todo, cell, P, nrm, sum)) todo = false;
       else sum[0] = sum[1] = sum[2] = make_float2(0.f, 0.f);
     }
