@@ -57,13 +57,13 @@ OPS_PER_NODE = 4 * OPS_PER_SLAB
 # only for the kernel sources they were captured on: the digest of csrc/ and include/ at capture time.  Any other
 # source digest reports no traffic.
 NCU_TRAFFIC = {
-    "digest": "eea445baffede396",
-    "villa": {"k_refit_wide": 4974592, "k_verify_box": 367724288, "k_cont_trace<deposit>": 991691136,
-              "k_compact": 12016384, "k_trace (re-trace)": 204486016, "k_deposit": 644327424,
-              "k_trace<deposit> (trace-all)": 892445952},
-    "city": {"k_refit_wide": 825088, "k_verify_box": 88076672, "k_cont_trace<deposit>": 218518272,
-             "k_compact": 4012288, "k_trace (re-trace)": 57209856, "k_deposit": 160499712,
-             "k_trace<deposit> (trace-all)": 164392320},
+    "digest": "44fb8b322c8b28e7",
+    "villa": {"k_refit_wide": 4967424, "k_verify_box": 366611328, "k_cont_trace<deposit>": 1002121600,
+              "k_compact": 12016896, "k_trace (re-trace)": 204643456, "k_deposit": 643118848,
+              "k_trace<deposit> (trace-all)": 891415424},
+    "city": {"k_refit_wide": 822528, "k_verify_box": 88699520, "k_cont_trace<deposit>": 219929216,
+             "k_compact": 4012928, "k_trace (re-trace)": 58534528, "k_deposit": 160472832,
+             "k_trace<deposit> (trace-all)": 164053632},
 }
 TAUS = (0.0, 0.005, 0.01, 0.05)
 
