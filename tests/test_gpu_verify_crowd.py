@@ -43,7 +43,7 @@ def _crowd(n_paths, n_obj=64, spread=2.0):
 
 
 def test_time_of_the_naive_box_test():
-    """2.8 times the error mode's verification; 3.5 times when the segment was prepared for every box."""
+    """2.8 times the error mode's verification; 3.7 times when the segment was prepared for every box."""
     import torch
     sc = _crowd(500_000)
     h = gu.lib_scene(sc)
@@ -68,7 +68,7 @@ def test_time_of_the_naive_box_test():
             ms.append(a.elapsed_time(e))
         return min(ms)
 
-    assert best(pv.PV_MODE_NAIVE_AABB) < 3.15 * best(pv.PV_MODE_ERROR)
+    assert best(pv.PV_MODE_NAIVE_AABB) < 3.3 * best(pv.PV_MODE_ERROR)
     pv.pv_destroy_scene(h)
 
 
